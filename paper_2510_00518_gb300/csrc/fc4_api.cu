@@ -486,6 +486,37 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         t.c3_r12 = d_r12;
         t.c3_ism = d_im;
         t.phi3 = c->phi3;
+        // key = (leg-1 atom, leg-2 atom, R1 - R2), as the 4ph keys below
+        using Key = std::tuple<int, int, int, int>;
+        std::map<Key, std::vector<int>> by_key;
+        for (int i = 0; i < c->nc3; ++i) {
+            const int *a = phi3->atoms + 3 * i, *R = phi3->cells + 6 * i;
+            by_key[Key(a[1] * na + a[2], R[0] - R[3], R[1] - R[4], R[2] - R[5])].push_back(i);
+        }
+        std::vector<int> k_start(1, 0), k_idx, g_start((size_t)na * na + 1, 0);
+        std::vector<int4> kr;
+        for (const auto &kv : by_key) {
+            const int d[3] = {std::get<1>(kv.first), std::get<2>(kv.first), std::get<3>(kv.first)};
+            kr.push_back(phase_vec(d, mesh, L));
+            k_idx.insert(k_idx.end(), kv.second.begin(), kv.second.end());
+            k_start.push_back((int)k_idx.size());
+            g_start[std::get<0>(kv.first) + 1]++;
+        }
+        for (int g = 0; g < na * na; ++g) g_start[g + 1] += g_start[g];
+        t.n_keys3 = (int)kr.size();
+        int *d_ks, *d_ki, *d_gs;
+        int4 *d_kr;
+        double2 *d_P3;
+        FC4_TRY(upload(c, &d_ks, k_start));
+        FC4_TRY(upload(c, &d_ki, k_idx));
+        FC4_TRY(upload(c, &d_gs, g_start));
+        FC4_TRY(upload(c, &d_kr, kr));
+        FC4_TRY(dalloc(c, &d_P3, (size_t)N * kr.size()));
+        t.k3_start = d_ks;
+        t.k3_idx = d_ki;
+        t.grp3_start = d_gs;
+        t.P3 = d_P3;
+        FC4_TRY(fc4::launch_phase_tables(t, t.n_keys3, d_kr, d_P3, nullptr, 0));
     }
 
     // fourth order: key = (leg-2 atom, leg-3 atom, R2 - R3); keys ordered by group, clusters by key
@@ -607,7 +638,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         FC4_TRY(dalloc(c, &d_P4_32, (size_t)N * nk));
         t.P4 = d_P4;
         t.P4_32 = d_P4_32;
-        FC4_TRY(fc4::launch_phase_tables(t, d_kr, d_P4, d_P4_32, 0));
+        FC4_TRY(fc4::launch_phase_tables(t, nk, d_kr, d_P4, d_P4_32, 0));
     }
 
     // modes: device harmonic solve

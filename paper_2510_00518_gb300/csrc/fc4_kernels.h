@@ -46,6 +46,12 @@ struct Tables {
     const int4 *c3_r12;          // [nc3] (R1 - R2)(L/n) mod L
     const double *c3_ism;        // [nc3] 1/sqrt(m_a m_b m_c)
     const double *phi3;          // [nc3][27]
+    // keys of the rate kernel: (leg-1 atom, leg-2 atom, R1 - R2), sorted by (leg-1, leg-2) group
+    int n_keys3;
+    const int *k3_start;         // [n_keys3 + 1] range in k3_idx of each key
+    const int *k3_idx;           // [nc3] clusters grouped by key, ascending within a key
+    const int *grp3_start;       // [n_atoms * n_atoms + 1] key range of group b * n_atoms + c
+    const double2 *P3;           // [N][n_keys3] exp(i q.(R1 - R2)) of each key
     // fourth order: clusters sorted by key; keys sorted by (leg-2 atom, leg-3 atom) group
     int nc4, n_keys;
     const int4 *c4_at;           // [nc4] (a, b, c, d)
@@ -157,7 +163,8 @@ cudaError_t launch_occupations(const Tables &t, double hbar_over_kT, double *occ
 // message returned by fc4_last_error(NULL) (errors of calls without a context)
 void set_host_error(const char *msg);
 
-cudaError_t launch_phase_tables(const Tables &t, const int4 *key_r, double2 *P4, float2 *P4_32,
+// P[q][r] = exp(i q.R_r) of n_keys keys (P32: the FP32 copy, or NULL)
+cudaError_t launch_phase_tables(const Tables &t, int n_keys, const int4 *key_r, double2 *P, float2 *P32,
                                 cudaStream_t s);
 cudaError_t launch_kappa(const Tables &t, double hbar_over_kT, double kB, const double *gamma,
                          int mask, double scale, double *kappa, cudaStream_t s);

@@ -245,21 +245,21 @@ cudaError_t launch_occupations(const Tables &t, double hbar_over_kT, double *occ
     return cudaGetLastError();
 }
 
-__global__ void phase_tables_kernel(const __grid_constant__ Tables t, const int4 *key_r,
-                                    double2 *P4, float2 *P4_32) {
+__global__ void phase_tables_kernel(const __grid_constant__ Tables t, int n_keys, const int4 *key_r,
+                                    double2 *P, float2 *P32) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)t.N * t.n_keys) return;
-    const int q = (int)(i / t.n_keys), r = (int)(i - (long long)q * t.n_keys);
+    if (i >= (long long)t.N * n_keys) return;
+    const int q = (int)(i / n_keys), r = (int)(i - (long long)q * n_keys);
     const double2 p = t.rt[phase_index(t.qc[q], key_r[r], t.L)];
-    P4[i] = p;
-    P4_32[i] = make_float2((float)p.x, (float)p.y);
+    P[i] = p;
+    if (P32) P32[i] = make_float2((float)p.x, (float)p.y);
 }
 
-cudaError_t launch_phase_tables(const Tables &t, const int4 *key_r, double2 *P4, float2 *P4_32,
+cudaError_t launch_phase_tables(const Tables &t, int n_keys, const int4 *key_r, double2 *P, float2 *P32,
                                 cudaStream_t s) {
-    const long long n = (long long)t.N * t.n_keys;
+    const long long n = (long long)t.N * n_keys;
     if (n == 0) return cudaSuccess;
-    phase_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(t, key_r, P4, P4_32);
+    phase_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(t, n_keys, key_r, P, P32);
     return cudaGetLastError();
 }
 
