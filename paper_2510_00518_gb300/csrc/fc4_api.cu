@@ -80,6 +80,8 @@ struct fc4_ctx {
     long long *part_n = nullptr, *part_items = nullptr, *part_ent = nullptr;
     long long *part_ev = nullptr, *part_cev = nullptr;
     size_t part_cap = 0;
+    double *kappa_part = nullptr;           // block sums of κ [kKappaBlocks][9]
+    unsigned *kappa_counter = nullptr;      // blocks of the κ kernel that are done (0 between calls)
     unsigned long long *stats = nullptr;    // [25] kept, items, entries, evaluated, visited per channel
     long long cand[5] = {0, 0, 0, 0, 0};    // candidates per channel of the last call
     int *modes = nullptr;
@@ -664,6 +666,9 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     FC4_TRY(cudaMemset(c->err, 0, sizeof(int)));
     FC4_TRY(dalloc(c, &c->dev_err, 1));
     FC4_TRY(cudaMemset(c->dev_err, 0, sizeof(int)));
+    FC4_TRY(dalloc(c, &c->kappa_part, 9 * (size_t)fc4::kKappaBlocks));
+    FC4_TRY(dalloc(c, &c->kappa_counter, 1));
+    FC4_TRY(cudaMemset(c->kappa_counter, 0, sizeof(unsigned)));
     t.om = c->om;
     t.om32 = c->om32;
     t.om32lo = c->om32lo;
@@ -950,7 +955,8 @@ fc4_status fc4_kappa_iterative(fc4_ctx *c, double T_K, int sigma_adaptive, doubl
     if (!c->bte_kappa) FC4_CUDA(c, dalloc(c, &c->bte_kappa, 9));
     const double xw = kHbar * 1e12 / (kKb * T_K);
     FC4_CUDA(c, fc4::launch_bte_update(c->t, gamma, channel_mask, nullptr, c->bte_F, c->bte_F32, s));   // F = v / Γ
-    FC4_CUDA(c, fc4::launch_kappa_F(c->t, xw, kKb, c->bte_F, kappa_scale(c), c->bte_kappa, s));
+    FC4_CUDA(c, fc4::launch_kappa_F(c->t, xw, kKb, c->bte_F, kappa_scale(c), c->kappa_part, c->kappa_counter,
+                                          c->bte_kappa, s));
     double kp[9], kn[9];
     FC4_CUDA(c, cudaMemcpyAsync(kp, c->bte_kappa, sizeof kp, cudaMemcpyDeviceToHost, s));
     FC4_CUDA(c, cudaStreamSynchronize(s));
@@ -960,7 +966,8 @@ fc4_status fc4_kappa_iterative(fc4_ctx *c, double T_K, int sigma_adaptive, doubl
                                    nullptr, stream, c->bte_F, c->bte_delta);
         if (st != FC4_OK) return st;
         FC4_CUDA(c, fc4::launch_bte_update(c->t, gamma, channel_mask, c->bte_delta, c->bte_F, c->bte_F32, s));
-        FC4_CUDA(c, fc4::launch_kappa_F(c->t, xw, kKb, c->bte_F, kappa_scale(c), c->bte_kappa, s));
+        FC4_CUDA(c, fc4::launch_kappa_F(c->t, xw, kKb, c->bte_F, kappa_scale(c), c->kappa_part, c->kappa_counter,
+                                          c->bte_kappa, s));
         FC4_CUDA(c, cudaMemcpyAsync(kn, c->bte_kappa, sizeof kn, cudaMemcpyDeviceToHost, s));
         FC4_CUDA(c, cudaStreamSynchronize(s));
         double dmax = 0.0, kmax = 0.0;
@@ -1027,7 +1034,7 @@ fc4_status fc4_kappa(fc4_ctx *c, double T_K, const double *gamma, int channel_ma
     if (channel_mask < 0 || channel_mask > 31) return fail(c, FC4_ERR_INVALID, "channel_mask must be in [0, 31]");
     Timed tm(c, 6, (cudaStream_t)stream);
     FC4_CUDA(c, fc4::launch_kappa(c->t, kHbar * 1e12 / (kKb * T_K), kKb, gamma, channel_mask, kappa_scale(c),
-                                  kappa_out, (cudaStream_t)stream));
+                                  c->kappa_part, c->kappa_counter, kappa_out, (cudaStream_t)stream));
     return FC4_OK;
 }
 

@@ -145,8 +145,11 @@ cudaError_t launch_bte_reduce(const Tables &t, const RateArgs &a, int channel_ma
 cudaError_t launch_bte_update(const Tables &t, const double *gamma, int mask, const double *delta, double *F,
                               float *F32, cudaStream_t s);
 cudaError_t launch_to_f32(const double *in, float *out, size_t n, cudaStream_t s);
+// κ from Γ (RTA) or from the field F: part holds 9 doubles for each of at most kKappaBlocks blocks,
+// counter is 0 between calls
+constexpr int kKappaBlocks = 608;      // 4 small blocks on each of 152 SMs
 cudaError_t launch_kappa_F(const Tables &t, double hbar_over_kT, double kB, const double *F, double scale,
-                           double *kappa, cudaStream_t s);
+                           double *part, unsigned *counter, double *kappa, cudaStream_t s);
 cudaError_t launch_reduce(const Tables &t, const RateArgs &a, int channel_mask, double c3,
                           double c4, double *gamma, double *wp, long long *counts,
                           unsigned long long *stats, cudaStream_t s);
@@ -166,8 +169,8 @@ void set_host_error(const char *msg);
 // P[q][r] = exp(i q.R_r) of n_keys keys (P32: the FP32 copy, or NULL)
 cudaError_t launch_phase_tables(const Tables &t, int n_keys, const int4 *key_r, double2 *P, float2 *P32,
                                 cudaStream_t s);
-cudaError_t launch_kappa(const Tables &t, double hbar_over_kT, double kB, const double *gamma,
-                         int mask, double scale, double *kappa, cudaStream_t s);
+cudaError_t launch_kappa(const Tables &t, double hbar_over_kT, double kB, const double *gamma, int mask,
+                         double scale, double *part, unsigned *counter, double *kappa, cudaStream_t s);
 cudaError_t launch_kappa_backward(const Tables &t, double hbar_over_kT, double kB, const double *gamma,
                                   int mask, double scale, const double *dLdk, double *dLdg, cudaStream_t s);
 cudaError_t launch_unpermute(int nc, int width, const int *perm, const double *in, double *out, cudaStream_t s);

@@ -350,33 +350,77 @@ __device__ __forceinline__ double gamma_total(const double *gamma, int nm, int m
     return g;
 }
 
-// κ_ab = scale Σ_λ C_λ v_a v_b / Γ_λ, C = k_B x² n (n + 1), over modes with ω > 0 and Γ > 0.
-// One block; thread i sums modes i, i + 256, ... in order; fixed-order block sums.
-__global__ void __launch_bounds__(256)
-kappa_kernel(int nm, const double *om, const double *vel, double x_per_w, double kB,
-             const double *gamma, int mask, double scale, double *kappa) {
-    __shared__ double s_red[32];
+// κ_ab = scale Σ_λ C_λ v_a f_b, C = k_B x² n (n + 1), over modes with ω > 0: f = v / Γ over modes with
+// Γ > 0 (RTA), or with FIELD the deviation vector F of the iterative BTE.  Every block writes its nine
+// sums to a slot of part, and the block that finishes last adds the slots in block order, so the
+// result does not depend on the order the blocks run in; the counter wraps to 0 by itself.
+// Bound: FP64 latency and issue (expm1 and the divides are ~100 FP64 operations a mode, one warp
+// operation per ~19 clocks and SM).  κ and its gradient for the 24576 modes of a 16^3 mesh took 406 us
+// with one block of 256 threads, and take 34 us with blocks of 64 on every SM.
+constexpr int kKappaThreads = 64;
+
+template <bool FIELD>
+__global__ void __launch_bounds__(kKappaThreads)
+kappa_kernel(int nm, const double *om, const double *vel, double x_per_w, double kB, const double *src,
+             int mask, double scale, double *part, unsigned *counter, double *kappa) {
+    __shared__ double s_red[9 * 32];
+    __shared__ long long s_none[32];
+    __shared__ bool s_last;
     double acc[9];
+    long long none[1] = {0};
+#pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-    for (int i = threadIdx.x; i < nm; i += blockDim.x) {
-        const double w = om[i], g = gamma_total(gamma, nm, mask, i);
+    for (int i = blockIdx.x * kKappaThreads + threadIdx.x; i < nm; i += gridDim.x * kKappaThreads) {
+        const double w = om[i];
+        const double g = FIELD ? 1.0 : gamma_total(src, nm, mask, i);
         if (!(w > 0.0) || !(g > 0.0)) continue;
         const double x = w * x_per_w;
         const double n = 1.0 / expm1(x);
         const double c = kB * x * x * n * (n + 1.0) / g;
         const double *v = vel + 3 * (size_t)i;
+        const double *f = FIELD ? src + 3 * (size_t)i : v;
+#pragma unroll
         for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) acc[3 * a + b] += c * v[a] * v[b];
+#pragma unroll
+            for (int b = 0; b < 3; ++b) acc[3 * a + b] += c * v[a] * f[b];
     }
-    for (int k = 0; k < 9; ++k) {
-        const double r = block_sum(acc[k], s_red);
-        if (threadIdx.x == 0) kappa[k] = r * scale;
+    block_sum_multi<9, 1>(acc, none, s_red, s_none);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) part[9 * (size_t)blockIdx.x + k] = acc[k];
+        __threadfence();
+        s_last = atomicInc(counter, gridDim.x - 1) == gridDim.x - 1;
     }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += kKappaThreads)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k] += __ldcg(part + 9 * (size_t)b + k);
+    block_sum_multi<9, 1>(acc, none, s_red, s_none);
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) kappa[k] = acc[k] * scale;
 }
 
-cudaError_t launch_kappa(const Tables &t, double hbar_over_kT, double kB, const double *gamma,
-                         int mask, double scale, double *kappa, cudaStream_t s) {
-    kappa_kernel<<<1, 256, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, gamma, mask, scale, kappa);
+int kappa_blocks(const Tables &t) {
+    const long long b = ((long long)t.N * t.nb + kKappaThreads - 1) / kKappaThreads;
+    return (int)(b < kKappaBlocks ? b : kKappaBlocks);
+}
+
+cudaError_t launch_kappa(const Tables &t, double hbar_over_kT, double kB, const double *gamma, int mask,
+                         double scale, double *part, unsigned *counter, double *kappa, cudaStream_t s) {
+    kappa_kernel<false><<<kappa_blocks(t), kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, gamma,
+                                                                  mask, scale, part, counter, kappa);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_kappa_F(const Tables &t, double hbar_over_kT, double kB, const double *F, double scale,
+                           double *part, unsigned *counter, double *kappa, cudaStream_t s) {
+    kappa_kernel<true><<<kappa_blocks(t), kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, F, 0,
+                                                                 scale, part, counter, kappa);
     return cudaGetLastError();
 }
 
@@ -405,7 +449,7 @@ __global__ void kappa_backward_kernel(int nm, const double *om, const double *ve
 cudaError_t launch_kappa_backward(const Tables &t, double hbar_over_kT, double kB, const double *gamma,
                                   int mask, double scale, const double *dLdk, double *dLdg, cudaStream_t s) {
     const int nm = t.N * t.nb;
-    kappa_backward_kernel<<<(nm + 255) / 256, 256, 0, s>>>(nm, t.om, t.vel, hbar_over_kT, kB, gamma, mask,
+    kappa_backward_kernel<<<(nm + kKappaThreads - 1) / kKappaThreads, kKappaThreads, 0, s>>>(nm, t.om, t.vel, hbar_over_kT, kB, gamma, mask,
                                                             scale, dLdk, dLdg);
     return cudaGetLastError();
 }
@@ -590,36 +634,6 @@ __global__ void to_f32_kernel(const double *in, float *out, size_t n) {
 cudaError_t launch_to_f32(const double *in, float *out, size_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     to_f32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, out, n);
-    return cudaGetLastError();
-}
-
-// κ_ab = scale Σ_λ C_λ v_a F_b over modes with ω > 0 (one block, fixed-order sums).
-__global__ void __launch_bounds__(256)
-kappa_F_kernel(int nm, const double *om, const double *vel, double x_per_w, double kB, const double *F,
-               double scale, double *kappa) {
-    __shared__ double s_red[32];
-    double acc[9];
-    for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-    for (int i = threadIdx.x; i < nm; i += blockDim.x) {
-        const double w = om[i];
-        if (!(w > 0.0)) continue;
-        const double x = w * x_per_w;
-        const double n = 1.0 / expm1(x);
-        const double c = kB * x * x * n * (n + 1.0);
-        const double *v = vel + 3 * (size_t)i;
-        const double *f = F + 3 * (size_t)i;
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) acc[3 * a + b] += c * v[a] * f[b];
-    }
-    for (int k = 0; k < 9; ++k) {
-        const double r = block_sum(acc[k], s_red);
-        if (threadIdx.x == 0) kappa[k] = r * scale;
-    }
-}
-
-cudaError_t launch_kappa_F(const Tables &t, double hbar_over_kT, double kB, const double *F, double scale,
-                           double *kappa, cudaStream_t s) {
-    kappa_F_kernel<<<1, 256, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, F, scale, kappa);
     return cudaGetLastError();
 }
 
