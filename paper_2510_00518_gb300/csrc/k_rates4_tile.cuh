@@ -6,8 +6,10 @@
 // kQPT q'' (over the unit's triangle where the partner-swap symmetry holds), tests the window
 // against every j' at once (branch-free FP32 prefilter, rare ambiguous candidates decided by the
 // exact FP64 Δ), compacts the (q'', j', masks) entries with a block scan, and evaluates them:
-//   FP32: X[c,d][γδ] = Σ_{r in (c,d)} P_r^s2 W_r[γδ] once per entry, Y = X e*''' per j''' (36 MACs);
-//   FP64: Y[cγ] = Σ_r P_r^s2 Σ_δ W_r[γδ] e*'''(dδ) per j''' (register-light).
+//   X[c,d][γδ] = Σ_{r in (c,d)} P_r^s2 W_r[γδ] once per entry, Y = X e*''' per j''' (36 MACs).
+// FP64 holds X too (2 blocks of 255 registers per SM): its pipe issues a warp operation every ~19
+// clocks and SM, so what counts is the 306 + 36 items complex multiply-adds of an entry, against 408
+// an item key by key; 4 q points of 8^3 went from 239 to 71.5 ms.
 // The same window decision, weights and accumulation as the general kernel (k_rates4.cuh).
 #pragma once
 #include "k_rates4.cuh"
@@ -118,12 +120,11 @@ w4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, 
 //   Δ_λ = Σ_p γ_p Σ_k s_k (ω_k / ω_λ) F_k  (partner signs: ++ (-, -, +), +- (-, +, +), -- (+, +, +)),
 // into a.part_d; the partner combination is symmetric under the swap the triangular domain uses.
 template <typename R, int NA, bool ADA, int kQPT, bool BTE = false, bool NOCOMP = false>
-__global__ void __launch_bounds__(kTileQ, ADA ? 3 : 4)
+__global__ void __launch_bounds__(kTileQ, sizeof(R) == 8 ? 2 : ADA ? 3 : 4)
 rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int ch,
                    int mode0, const Cplx<R> *__restrict__ wall) {
     using C = Cplx<R>;
     constexpr int NB = 3 * NA;
-    constexpr bool XROUTE = (sizeof(R) == 4);
     const int s1 = (ch == 4) ? -1 : 1;
     const int s2 = (ch == 2) ? 1 : -1;
     const int N = t.N, nk = t.n_keys;
@@ -372,23 +373,21 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                 }
                 const C *Prow = P4 + (size_t)iq2 * nk;
                 const C *Wj = sW + j1 * nk * 9;
-                C X[XROUTE ? NA : 1][XROUTE ? NA : 1][9];
-                if constexpr (XROUTE) {
+                C X[NA][NA][9];
 #pragma unroll
-                    for (int c = 0; c < NA; ++c)
+                for (int c = 0; c < NA; ++c)
 #pragma unroll
-                        for (int d = 0; d < NA; ++d) {
+                    for (int d = 0; d < NA; ++d) {
 #pragma unroll
-                            for (int k = 0; k < 9; ++k) X[c][d][k] = czero<C>();
-                            const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
-                            for (int r = r0; r < r1; ++r) {
-                                const C ph = cconj_if(Prow[r], s2 < 0);
-                                const C *Wr = Wj + 9 * r;
+                        for (int k = 0; k < 9; ++k) X[c][d][k] = czero<C>();
+                        const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
+                        for (int r = r0; r < r1; ++r) {
+                            const C ph = cconj_if(Prow[r], s2 < 0);
+                            const C *Wr = Wj + 9 * r;
 #pragma unroll
-                                for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
-                            }
+                            for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
                         }
-                }
+                    }
 #pragma unroll 1
                 for (int j3 = 0; j3 < NB; ++j3) {
                     unsigned m = (unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u);
@@ -404,30 +403,12 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                         C e3[3];
 #pragma unroll
                         for (int dl = 0; dl < 3; ++dl) e3[dl] = cconj(ev[(iq3 * NB + 3 * d + dl) * NB + j3]);
-                        if constexpr (XROUTE) {
 #pragma unroll
-                            for (int c = 0; c < NA; ++c)
+                        for (int c = 0; c < NA; ++c)
 #pragma unroll
-                                for (int g = 0; g < 3; ++g)
+                            for (int g = 0; g < 3; ++g)
 #pragma unroll
-                                    for (int dl = 0; dl < 3; ++dl) Y[c][g] = cfma(X[c][d][3 * g + dl], e3[dl], Y[c][g]);
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < NA; ++c) {
-                                const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
-                                for (int r = r0; r < r1; ++r) {
-                                    const C ph = cconj_if(Prow[r], s2 < 0);
-                                    const C *Wr = Wj + 9 * r;
-#pragma unroll
-                                    for (int g = 0; g < 3; ++g) {
-                                        C u = cmul(Wr[3 * g], e3[0]);
-                                        u = cfma(Wr[3 * g + 1], e3[1], u);
-                                        u = cfma(Wr[3 * g + 2], e3[2], u);
-                                        Y[c][g] = cfma(ph, u, Y[c][g]);
-                                    }
-                                }
-                            }
-                        }
+                                for (int dl = 0; dl < 3; ++dl) Y[c][g] = cfma(X[c][d][3 * g + dl], e3[dl], Y[c][g]);
                     }
                     const int m3 = iq3 * NB + j3;
                     const R n3 = occ[m3], iw3 = invw[m3];
