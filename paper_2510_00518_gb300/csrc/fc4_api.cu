@@ -101,6 +101,7 @@ struct fc4_ctx {
     float *bte_F32 = nullptr;
     size_t part_d_cap = 0;
     std::vector<int> w_modes;
+    int *swap12_dev = nullptr, *swap23_dev = nullptr;   // swap partners in device slots (gradients)
     int *perm4_dev = nullptr;              // device cluster slot -> input index (gradients)
     double *adj_part = nullptr;            // per-mode gradient slices of fc4_rates_backward
     size_t adj_cap = 0;
@@ -623,6 +624,17 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         FC4_TRY(upload(c, &d_kbi, kb_idx));
         FC4_TRY(upload(c, &d_kr, kr));
         FC4_TRY(upload(c, &c->perm4_dev, c->perm4));
+        {   // swap partners between device slots (-1 where a cluster has none)
+            std::vector<int> slot(c->nc4), s12(c->nc4), s23(c->nc4);
+            for (int s = 0; s < c->nc4; ++s) slot[c->perm4[s]] = s;
+            for (int s = 0; s < c->nc4; ++s) {
+                const int i12 = c->swap12[c->perm4[s]], i23 = c->swap23[c->perm4[s]];
+                s12[s] = i12 < 0 ? -1 : slot[i12];
+                s23[s] = i23 < 0 ? -1 : slot[i23];
+            }
+            FC4_TRY(upload(c, &c->swap12_dev, s12));
+            FC4_TRY(upload(c, &c->swap23_dev, s23));
+        }
         FC4_TRY(dalloc(c, &c->adj_tmp, 81 * (size_t)std::max(1, c->nc4)));
         t.c4_at = d_at;
         t.c4_r3 = d_r3;
@@ -746,6 +758,30 @@ namespace {
 // κ's prefactor 1/(N V_cell) with v in Å/ps (x 100 m/s) and 1/Γ in ps (x 1e-12 s): W/(m K)
 double kappa_scale(const fc4_ctx *c) { return 1e4 * 1e-12 / ((double)c->t.N * c->volume * 1e-30); }
 
+// Cap of the W scratch in bytes: fc4_set_mode_chunk's, or max(4 GiB, a quarter of the device memory).
+size_t w_cap(const fc4_ctx *c) {
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) total_b = 0;
+    return c->w_limit ? c->w_limit : std::max<size_t>(4ull << 30, total_b / 4);
+}
+
+// Grow the W scratch to at least bytes.
+fc4_status ensure_wbuf(fc4_ctx *c, size_t bytes) {
+    if (c->wbuf_bytes >= bytes) return FC4_OK;
+    if (c->wbuf) {
+        cudaFree(c->wbuf);
+        c->owned.erase(std::find(c->owned.begin(), c->owned.end(), c->wbuf));
+        c->wbuf = nullptr;
+        c->wbuf_bytes = 0;
+    }
+    unsigned char *w = nullptr;
+    FC4_CUDA(c, dalloc(c, &w, bytes));
+    c->wbuf = w;
+    c->wbuf_bytes = bytes;
+    c->w_s1 = 0;
+    return FC4_OK;
+}
+
 // The rates call behind fc4_rates and the iterative BTE: with bte_F set (device [N nb][3]), the
 // kernels also accumulate the BTE's off-diagonal term, reduced into delta_out [n_q nb][3]; Γ, WP
 // and counts are written when gamma_out is set.
@@ -797,10 +833,7 @@ fc4_status rates_call(fc4_ctx *c, double T_K, int sigma_adaptive, double sigma_v
     size_t chunk = (size_t)nm;
     if (c->mode_chunk > 0) chunk = std::min(chunk, (size_t)c->mode_chunk);
     if (per_mode) {
-        size_t free_b = 0, total_b = 0;
-        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) total_b = 0;
-        const size_t cap_bytes = c->w_limit ? c->w_limit : std::max<size_t>(4ull << 30, total_b / 4);
-        chunk = std::max<size_t>(1, std::min(chunk, cap_bytes / per_mode));
+        chunk = std::max<size_t>(1, std::min(chunk, w_cap(c) / per_mode));
     }
     const size_t need = (size_t)5 * chunk * N;
     if (need > c->part_cap) {
@@ -830,18 +863,9 @@ fc4_status rates_call(fc4_ctx *c, double T_K, int sigma_adaptive, double sigma_v
         if (!c->bte_F32) FC4_CUDA(c, dalloc(c, &c->bte_F32, (size_t)3 * N * nb));
         FC4_CUDA(c, fc4::launch_to_f32(bte_F, c->bte_F32, (size_t)3 * N * nb, s));
     }
-    if (per_mode && c->wbuf_bytes < chunk * per_mode) {     // W scratch of the tiled 4ph path
-        if (c->wbuf) {
-            cudaFree(c->wbuf);
-            c->owned.erase(std::find(c->owned.begin(), c->owned.end(), c->wbuf));
-            c->wbuf = nullptr;
-            c->wbuf_bytes = 0;
-        }
-        unsigned char *w = nullptr;
-        FC4_CUDA(c, dalloc(c, &w, chunk * per_mode));
-        c->wbuf = w;
-        c->wbuf_bytes = chunk * per_mode;
-        c->w_s1 = 0;
+    if (per_mode) {                         // W scratch of the tiled 4ph path
+        const fc4_status sw = ensure_wbuf(c, chunk * per_mode);
+        if (sw != FC4_OK) return sw;
     }
     if (modes != c->modes_on_device) {      // unchanged subsets need no copy (stream capture)
         FC4_CUDA(c, cudaMemcpyAsync(c->modes, modes.data(), nm * sizeof(int), cudaMemcpyHostToDevice, s));
@@ -1087,6 +1111,19 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
     a.n_modes = nm;
     a.modes = c->modes;
     set_window(c, a, c->last_adaptive, c->last_sigma);
+    // FP64 cells of up to two atoms: the tiled adjoint, in chunks of modes whose W fits in the W scratch
+    if (c->precision == FC4_FP64 && dphi4 && c->nc4 && (c->last_mask & 0b11100) && fc4::adj4_tiled(c->t)) {
+        const size_t per_mode = fc4::rates4_wbuf_per_mode(c->t, 1);
+        if (per_mode) {
+            if (c->wbuf_bytes < per_mode) {
+                st = ensure_wbuf(c, std::max<size_t>(1, std::min((size_t)nm, w_cap(c) / per_mode)) * per_mode);
+                if (st != FC4_OK) return st;
+            }
+            a.wbuf = c->wbuf;
+            a.wbuf_bytes = c->wbuf_bytes;
+            c->w_s1 = 0;                    // the W of the last rates call is overwritten
+        }
+    }
     const double N = (double)c->t.N;
     bool first3 = true, first4 = true;
     for (int ch = 0; ch < 5; ++ch) {
@@ -1099,10 +1136,12 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
         FC4_CUDA(c, fc4::launch_adjoint(c->t, a, ch, dL_dgamma, cst, c->adj_part, fp64, s));
         c->n_launches += 1;
         if (ch < 2) {
-            FC4_CUDA(c, fc4::launch_sum_slices(nm, 27 * c->nc3, c->adj_part, dphi3, first3 ? 0 : 1, 0, s));
+            FC4_CUDA(c, fc4::launch_sum_slices(nm, 27 * c->nc3, c->adj_part, dphi3, first3 ? 0 : 1, 0, nullptr, 0, s));
             first3 = false;
         } else {
-            FC4_CUDA(c, fc4::launch_sum_slices(nm, 81 * c->nc4, c->adj_part, c->adj_tmp, first4 ? 0 : 1, !fp64, s));
+            const bool swapped = a.wbuf && (a.tri & (ch == 3 ? 1 : 2));
+            FC4_CUDA(c, fc4::launch_sum_slices(nm, 81 * c->nc4, c->adj_part, c->adj_tmp, first4 ? 0 : 1, !fp64,
+                                               !swapped ? nullptr : ch == 3 ? c->swap23_dev : c->swap12_dev, ch != 3, s));
             first4 = false;
         }
         c->n_launches += 1;

@@ -513,11 +513,25 @@ size_t tile_w_bytes_per_mode(const Tables &t) {
     return sizeof(Cplx<R>) * (size_t)t.N * 3 * NA * t.n_keys * 9;
 }
 
+// W of the units of modes [m, m + nm) into a.wbuf.
+template <typename R, int NA>
+cudaError_t launch_w4(const Tables &t, const RateArgs &a, int ch, int m, int nm, cudaStream_t s) {
+    using C = Cplx<R>;
+    constexpr int NB = 3 * NA;
+    const size_t wsmem = sizeof(C) * ((size_t)t.nc4 * 28 + NB * NB + NB + (size_t)t.n_keys * NA * 27);
+    cudaError_t e = cudaFuncSetAttribute(w4_kernel<R, NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
+    if (e != cudaSuccess) return e;
+    const long long ngrp = (t.N + kW4Group - 1) / kW4Group;
+    w4_kernel<R, NA><<<(unsigned)(nm * ngrp), kW4Threads, wsmem, s>>>(t, a, ch, m, reinterpret_cast<C *>(a.wbuf));
+    e = cudaGetLastError();
+    if (e == cudaSuccess && a.n_kernels) ++*a.n_kernels;
+    return e;
+}
+
 // Launch W (global) then the tiled kernel, over mode chunks that fit in the W buffer.
 template <typename R, int NA, bool ADA, bool BTE = false>
 cudaError_t launch4_tile(const Tables &t, const RateArgs &a, int ch, cudaStream_t s) {
     using C = Cplx<R>;
-    constexpr int NB = 3 * NA;
     const bool dense = ch == 3;
     const size_t smem = tile_smem_bytes<R, NA>(t, qpt_of<ADA>(dense), ADA);
     auto kern = dense ? rates4_tile_kernel<R, NA, ADA, qpt_of<ADA>(true), BTE>
@@ -528,21 +542,14 @@ cudaError_t launch4_tile(const Tables &t, const RateArgs &a, int ch, cudaStream_
                          : rates4_tile_kernel<R, NA, ADA, qpt_of<ADA>(false), false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const size_t wsmem = sizeof(C) * ((size_t)t.nc4 * 28 + NB * NB + NB + (size_t)t.n_keys * NA * 27);
-    e = cudaFuncSetAttribute(w4_kernel<R, NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
-    if (e != cudaSuccess) return e;
     const size_t per_mode = tile_w_bytes_per_mode<R, NA>(t);
     const int chunk = (int)(a.wbuf_bytes / per_mode);
     if (chunk < 1) return cudaErrorInvalidValue;
     for (int m = 0; m < a.n_modes; m += chunk) {
         const int nm = min(chunk, a.n_modes - m);
-        const long long ngrp = (t.N + kW4Group - 1) / kW4Group;
         if (!(a.w_reuse && nm == a.n_modes)) {           // W of the previous channel with the same s1
-            w4_kernel<R, NA><<<(unsigned)((long long)nm * ngrp), kW4Threads, wsmem, s>>>(t, a, ch, m,
-                                                                                  reinterpret_cast<C *>(a.wbuf));
-            e = cudaGetLastError();
+            e = launch_w4<R, NA>(t, a, ch, m, nm, s);
             if (e != cudaSuccess) return e;
-            if (a.n_kernels) ++*a.n_kernels;
         }
         if constexpr (sizeof(R) == 4 && !BTE) {
             if (ch == 3 && a.use_tc) {                  // +-: cluster contraction on the tensor cores

@@ -165,3 +165,47 @@ def test_rates_backward_mixed_precision(sysm, mesh, sub):
     assert_close(d3.cpu().numpy().reshape(-1), g3.reshape(-1), 1e-8, floor_frac=1e-9, what="dphi3 (mixed context)")
     err = np.abs(d4.cpu().numpy() - g4).max() / np.abs(g4).max()
     assert err <= 1e-4, err
+
+
+@pytest.mark.parametrize("mesh,shells,w_modes,sigma,adaptive", [
+    ((5, 5, 5), 2, 0, 0.1, False), ((4, 4, 8), 2, 0, 0.05, False), ((5, 5, 6), 2, 0, 0.1, False),
+    ((2, 3, 4), 3, 4, 0.3, False), ((3, 3, 2), 2, 1, 1.0, True)])
+def test_tiled_backward_edges(mesh, shells, w_modes, sigma, adaptive):
+    """The tiled FP64 adjoint at its rounds of 128 q'', with more clusters than one block of its fold
+    holds (227; three shells give 394), and over several chunks of the W buffer.  Γ is quadratic in Φ,
+    so L(Φ + Φ') - L(Φ - Φ') = 2 <dL/dΦ, Φ'> up to the rounding of the two L (1e-10 of each, the FP64
+    bar; dL/dΓ > 0, so L has no cancellation between modes), for Φ' on one cluster at a time."""
+    from synth import diamond_crystal, morse_ifcs
+    c = diamond_crystal()
+    sysm = (c,) + morse_ifcs(c, seed=6, anharmonic_shells=shells)
+    e = make_engine(sysm, mesh, precision=0, inject=False)
+    sub = [int(np.prod(mesh)) // 2] if np.prod(mesh) > 100 else [0, 5]
+    dL = np.random.default_rng(3).uniform(0.5, 1.5, (5, 6 * len(sub)))
+    dL[:, 1] = 0.0
+    dL = torch.tensor(dL, device="cuda")
+
+    def rates(engine):
+        return engine.rates(300.0, sigma, 31, q_subset=sub, adaptive=adaptive)[0]
+
+    rates(e)
+    d3, d4 = e.backward(dL)
+    if w_modes:
+        f = make_engine(sysm, mesh, precision=0, inject=False)
+        f.set_mode_chunk(0, w_modes * f.memory()["w_per_mode"])
+        rates(f)
+        x3, x4 = f.backward(dL)
+        assert torch.equal(d3, x3) and torch.equal(d4, x4)
+    rng = np.random.default_rng(5)
+    n3, n4 = sysm[2].n_clusters, sysm[3].n_clusters
+    for order, k in [(3, 0), (3, n3 - 1), (3, n3 // 2)] + [(4, k) for k in [0, n4 - 1, *rng.integers(1, n4 - 1, 8)]]:
+        phi = sysm[order - 1].phi
+        step = np.zeros_like(phi)
+        step[k] = rng.normal(size=phi.shape[1]) * np.abs(phi).max()
+        L = []
+        for sgn in (1, -1):
+            mod = phi + sgn * step
+            e.update_anharmonic(mod if order == 3 else None, mod if order == 4 else None)
+            L.append(float((dL * rates(e)).sum()))
+        e.update_anharmonic(sysm[2].phi, sysm[3].phi)
+        got = float(((d3 if order == 3 else d4).cpu().numpy() * step).sum())
+        assert abs((L[0] - L[1]) / 2 - got) <= 1e-10 * (abs(L[0]) + abs(L[1])), (order, k, L, got)
