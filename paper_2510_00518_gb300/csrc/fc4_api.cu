@@ -608,10 +608,15 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
                 kb_idx[fill[(size_t)r * na + at[s].y]++] = s;
             }
         }
+        std::vector<int> key_order(nk);
+        std::iota(key_order.begin(), key_order.end(), 0);
+        std::stable_sort(key_order.begin(), key_order.end(), [&](int x, int y) {
+            return key_start[x + 1] - key_start[x] > key_start[y + 1] - key_start[y];
+        });
         int4 *d_at, *d_r3, *d_r13, *d_kr;
         double *d_im;
         float *d_im32;
-        int *d_ks, *d_kbs, *d_kbi;
+        int *d_ks, *d_ko, *d_kbs, *d_kbi;
         FC4_TRY(upload(c, &d_at, at));
         FC4_TRY(upload(c, &d_r3, r3));
         FC4_TRY(upload(c, &d_r13, r13));
@@ -620,6 +625,8 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         FC4_TRY(upload(c, &c->phi4, ph));
         FC4_TRY(upload(c, &c->phi4_32, ph32));
         FC4_TRY(upload(c, &d_ks, key_start));
+        FC4_TRY(upload(c, &d_ko, key_order));
+        t.key_order = d_ko;
         FC4_TRY(upload(c, &d_kbs, kb_start));
         FC4_TRY(upload(c, &d_kbi, kb_idx));
         FC4_TRY(upload(c, &d_kr, kr));

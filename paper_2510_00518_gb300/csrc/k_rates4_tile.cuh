@@ -116,6 +116,134 @@ w4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, 
     }
 }
 
+// The same in FP32, for a group of q' per block: a thread owns a column (r, γδ) for kW4Pair q' at a time.
+// It folds the cluster phases into its six
+//   Ψ_rb[β][γδ] = Σ_{c in r, b(c) = b} exp(i(s1 q'.(R1 - R3) - q.R3)) Φ~_c[β][γδ]   (fixed order)
+// in registers and writes W_r[γδ] = Σ_b Σ_β e^s1_λ'(bβ) Ψ_rb[β][γδ] for every j' (the same sums in the
+// same order).
+//
+// Bound: FP32 issue and shared-memory loads; 17000 complex multiply-adds a unit (the 14.7 KB a unit
+// written take an eighth of the time).  Ψ in registers needs no barrier between the two sums, and a
+// column reads its six Ψ once for all j' and its Φ~ once for two q'; keys are taken from the
+// longest cluster list down, so that the two keys with R2 = R3 (49 of 226 clusters each, the others 4)
+// share a warp, which moves over the warps from block to block.  Both signs of all modes of 8^3:
+// 29.3 ms, against 57 ms with Ψ in shared memory.
+constexpr int kW4Pair = 2;
+
+template <int NA>
+struct W4Smem {
+    using C = float2;
+    static constexpr int NB = 3 * NA;
+    C *Pt, *Ph, *E1, *e0;
+    int *i3, *kb, *idx;
+    __host__ __device__ static size_t bytes(const Tables &t) {
+        return sizeof(C) * ((size_t)t.nc4 * 27 + (size_t)t.nc4 * kW4Pair + NB * NB * kW4Pair + NB) +
+               sizeof(int) * ((size_t)2 * t.nc4 + (size_t)t.n_keys * NA + 1);
+    }
+    __device__ __forceinline__ W4Smem(unsigned char *smem, const Tables &t) {
+        Ph = reinterpret_cast<C *>(smem);                       // [nc4][kW4Pair] phases
+        E1 = Ph + t.nc4 * kW4Pair;                              // [kW4Pair][NB][NB] e^s1_λ'(comp) per j'
+        Pt = E1 + NB * NB * kW4Pair;                            // [nc4][3][9]
+        e0 = Pt + t.nc4 * 27;                                   // [NB]
+        i3 = reinterpret_cast<int *>(e0 + NB);                  // [nc4] phase index of q.R3
+        idx = i3 + t.nc4;                                       // [nc4] clusters by (key, leg-1 atom)
+        kb = idx + t.nc4;                                       // [n_keys NA + 1] their ranges
+    }
+};
+
+template <int NA>
+__global__ void __launch_bounds__(384, 2)
+w4_column_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int ch, int mode0, int group,
+                 float2 *wout) {
+    using C = float2;
+    using R = float;
+    constexpr int NB = 3 * NA;
+    const int s1 = (ch == 4) ? -1 : 1;
+    const int N = t.N, nk = t.n_keys, nc4 = t.nc4;
+    const int ngrp = (N + group - 1) / group;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const W4Smem<NA> sm(smem, t);
+    const int ml = blockIdx.x / ngrp, qg = blockIdx.x - ml * ngrp;
+    const int m0 = a.modes[mode0 + ml];
+    const int q0 = m0 / NB, j0 = m0 - q0 * NB;
+    const C *ev = Sel<R>::ev(t);
+    const C *rt = Sel<R>::rt(t);
+    const R *phi4 = Sel<R>::phi4(t);
+    const R *ism4 = Sel<R>::ism4(t);
+    const int4 c0 = t.qc[q0];
+    for (int k = threadIdx.x; k < NB; k += blockDim.x) sm.e0[k] = ev[(q0 * NB + k) * NB + j0];
+    for (int c = threadIdx.x; c < nc4; c += blockDim.x) {
+        sm.i3[c] = phase_index(c0, t.c4_r3[c], t.L);
+        sm.idx[c] = t.kb_idx[c];
+    }
+    for (int k = threadIdx.x; k <= nk * NA; k += blockDim.x) sm.kb[k] = t.kb_start[k];
+    __syncthreads();
+    for (int k = threadIdx.x; k < nc4 * 27; k += blockDim.x) {
+        const int c = k / 27, rem = k - c * 27;
+        const int a0 = t.c4_at[c].x;
+        const R *ph4 = phi4 + 81 * c + rem;
+        C v = czero<C>();
+#pragma unroll
+        for (int al = 0; al < 3; ++al) v = crfma(ph4[27 * al], sm.e0[3 * a0 + al], v);
+        sm.Pt[k] = cmake(v.x * ism4[c], v.y * ism4[c]);
+    }
+    // the warp with the long keys sits on another scheduler in every block
+    const int nw = blockDim.x >> 5;
+    const int col0 = ((int)threadIdx.x + 32 * (int)(blockIdx.x % nw)) % (int)blockDim.x;
+    const int q1_end = min(N, (qg + 1) * group);
+    for (int q1 = qg * group; q1 < q1_end; q1 += kW4Pair) {
+        const int nq = min(kW4Pair, q1_end - q1);
+        __syncthreads();                                         // Pt ready / previous q' done
+        for (int k = threadIdx.x; k < nc4 * kW4Pair; k += blockDim.x) {
+            const int c = k / kW4Pair, qq = min(k - c * kW4Pair, nq - 1);
+            const int4 c1 = t.qc[q1 + qq], r = t.c4_r13[c];
+            sm.Ph[k] = rt[mod_pos(s1 * (c1.x * r.x + c1.y * r.y + c1.z * r.z) - sm.i3[c], t.L)];
+        }
+        for (int k = threadIdx.x; k < NB * NB * nq; k += blockDim.x) {
+            const int qq = k / (NB * NB), rem = k - qq * NB * NB;
+            const int j1 = rem / NB, comp = rem - j1 * NB;
+            sm.E1[k] = cconj_if(ev[((q1 + qq) * NB + comp) * NB + j1], s1 < 0);
+        }
+        __syncthreads();
+        for (int k = col0; k < nk * 9; k += blockDim.x) {
+            const int r = t.key_order[k / 9], gd = k % 9;
+            C psi[kW4Pair][NB];
+#pragma unroll
+            for (int qq = 0; qq < kW4Pair; ++qq)
+#pragma unroll
+                for (int bb = 0; bb < NB; ++bb) psi[qq][bb] = czero<C>();
+#pragma unroll
+            for (int b = 0; b < NA; ++b)
+                for (int i = sm.kb[r * NA + b]; i < sm.kb[r * NA + b + 1]; ++i) {
+                    const int c = sm.idx[i];
+                    const C *pt = sm.Pt + c * 27 + gd;
+                    C ph[kW4Pair];
+#pragma unroll
+                    for (int qq = 0; qq < kW4Pair; ++qq) ph[qq] = sm.Ph[c * kW4Pair + qq];
+#pragma unroll
+                    for (int be = 0; be < 3; ++be) {
+                        const C x = pt[be * 9];
+#pragma unroll
+                        for (int qq = 0; qq < kW4Pair; ++qq) psi[qq][3 * b + be] = cfma(ph[qq], x, psi[qq][3 * b + be]);
+                    }
+                }
+#pragma unroll
+            for (int qq = 0; qq < kW4Pair; ++qq) {
+                if (qq >= nq) break;
+                C *wo = wout + (((size_t)ml * N + q1 + qq) * NB * nk + r) * 9 + gd;
+                const C *e1 = sm.E1 + qq * NB * NB;
+#pragma unroll
+                for (int j1 = 0; j1 < NB; ++j1) {
+                    C acc = czero<C>();
+#pragma unroll
+                    for (int bb = 0; bb < NB; ++bb) acc = cfma(e1[j1 * NB + bb], psi[qq][bb], acc);
+                    wo[(size_t)j1 * nk * 9] = acc;
+                }
+            }
+        }
+    }
+}
+
 // BTE = true also accumulates the off-diagonal term of the iterative Boltzmann equation,
 //   Δ_λ = Σ_p γ_p Σ_k s_k (ω_k / ω_λ) F_k  (partner signs: ++ (-, -, +), +- (-, +, +), -- (+, +, +)),
 // into a.part_d; the partner combination is symmetric under the swap the triangular domain uses.
@@ -518,11 +646,26 @@ template <typename R, int NA>
 cudaError_t launch_w4(const Tables &t, const RateArgs &a, int ch, int m, int nm, cudaStream_t s) {
     using C = Cplx<R>;
     constexpr int NB = 3 * NA;
-    const size_t wsmem = sizeof(C) * ((size_t)t.nc4 * 28 + NB * NB + NB + (size_t)t.n_keys * NA * 27);
-    cudaError_t e = cudaFuncSetAttribute(w4_kernel<R, NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
-    if (e != cudaSuccess) return e;
-    const long long ngrp = (t.N + kW4Group - 1) / kW4Group;
-    w4_kernel<R, NA><<<(unsigned)(nm * ngrp), kW4Threads, wsmem, s>>>(t, a, ch, m, reinterpret_cast<C *>(a.wbuf));
+    C *w = reinterpret_cast<C *>(a.wbuf);
+    cudaError_t e;
+    if constexpr (sizeof(R) == 8) {
+        const size_t smem = sizeof(C) * ((size_t)t.nc4 * 28 + NB * NB + NB + (size_t)t.n_keys * NA * 27);
+        e = cudaFuncSetAttribute(w4_kernel<R, NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const long long ngrp = (t.N + kW4Group - 1) / kW4Group;
+        w4_kernel<R, NA><<<(unsigned)(nm * ngrp), kW4Threads, smem, s>>>(t, a, ch, m, w);
+    } else {
+        const size_t smem = W4Smem<NA>::bytes(t);
+        e = cudaFuncSetAttribute(w4_column_kernel<NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        // q' per block: up to 32 share a Φ~ as long as the grid still fills the device
+        int group = 32;
+        while (group > 4 && (long long)nm * ((t.N + group - 1) / group) < 1216) group /= 2;
+        const long long ngrp = (t.N + group - 1) / group;
+        const int cols = t.n_keys * 9, rounds = std::max(1, (cols + 383) / 384);
+        const int threads = std::max(32, ((cols + rounds - 1) / rounds + 31) / 32 * 32);
+        w4_column_kernel<NA><<<(unsigned)(nm * ngrp), threads, smem, s>>>(t, a, ch, m, group, w);
+    }
     e = cudaGetLastError();
     if (e == cudaSuccess && a.n_kernels) ++*a.n_kernels;
     return e;
