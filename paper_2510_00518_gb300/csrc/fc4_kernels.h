@@ -33,10 +33,13 @@ struct Tables {
     const float *omT32;          // ω hi
     const float4 *vpT32;         // P hi
     const float4 *vpTlo;         // P lo
+    const float4 *wrange;        // [N] over participating branches: min ω, max ω (FP32 hi parts; +inf, -inf if
+                                 // none), max |P| (1 + 2^-14)
     double recip[9];             // reciprocal vectors b_k (rows, 1/Å), a_i . b_k = 2π δ_ik
     // occupations at the current T
     const double *occ;           // [N*nb]
     const float *occ32;          // [N*nb]
+    const float4 *mode4;         // [N*nb] (ω hi, ω lo, occupation, 1/ω) in FP32: one load of a mode's scalars
     const double *invw;          // [N*nb] 1/ω (0 for excluded)
     const float *invw32;         // [N*nb]
     // third order
@@ -161,9 +164,9 @@ cudaError_t launch_harmonic(const Tables &t, int nc2, const int4 *c2_at, const i
 cudaError_t launch_mode_tables(const Tables &t, double *om, float *om32, float *om32lo,
                                float2 *ev32, const double2 *ev, unsigned *vmask, double *invw,
                                float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
-                               float4 *vpTlo, cudaStream_t s);
+                               float4 *vpTlo, float4 *wrange, cudaStream_t s);
 cudaError_t launch_occupations(const Tables &t, double hbar_over_kT, double *occ, float *occ32,
-                               cudaStream_t s);
+                               float4 *mode4, cudaStream_t s);
 // message returned by fc4_last_error(NULL) (errors of calls without a context)
 void set_host_error(const char *msg);
 

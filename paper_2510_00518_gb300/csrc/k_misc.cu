@@ -179,7 +179,7 @@ cudaError_t launch_harmonic(const Tables &t, int nc2, const int4 *c2_at, const i
 __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om, float *om32, float *om32lo,
                                    float2 *ev32, const double2 *ev, unsigned *vmask, double *invw,
                                    float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
-                                   float4 *vpTlo) {
+                                   float4 *vpTlo, float4 *wrange) {
     const int N = t.N, nb = t.nb;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nm = (long long)N * nb;
@@ -212,36 +212,52 @@ __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om,
     }
     if (i < N) {
         unsigned m = 0;
+        float lo = __int_as_float(0x7f800000), hi = -lo, pm = 0.0f;
         for (int j = 0; j < nb; ++j)
-            if (!(i == 0 && j < 3) && om[i * nb + j] > 0.0) m |= 1u << j;
+            if (!(i == 0 && j < 3) && om[i * nb + j] > 0.0) {
+                m |= 1u << j;
+                const float w = (float)om[i * nb + j];
+                lo = fminf(lo, w);
+                hi = fmaxf(hi, w);
+                const double *v = t.vel + 3 * (i * nb + j);
+                double p2 = 0.0;
+                for (int k = 0; k < 3; ++k) {
+                    const double p = (v[0] * t.recip[3 * k] + v[1] * t.recip[3 * k + 1] + v[2] * t.recip[3 * k + 2]) / t.mesh[k];
+                    p2 += p * p;
+                }
+                pm = fmaxf(pm, (float)(sqrt(p2) * (1.0 + 0x1p-14)));
+            }
         vmask[i] = m;
+        wrange[i] = make_float4(lo, hi, pm, 0.0f);
     }
 }
 
 cudaError_t launch_mode_tables(const Tables &t, double *om, float *om32, float *om32lo,
                                float2 *ev32, const double2 *ev, unsigned *vmask, double *invw,
                                float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
-                               float4 *vpTlo, cudaStream_t s) {
+                               float4 *vpTlo, float4 *wrange, cudaStream_t s) {
     const long long n = (long long)t.N * t.nb * t.nb;
     mode_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(t, om, om32, om32lo, ev32, ev, vmask, invw,
-                                                                    invw32, vp32, vp32lo, omT32, vpT32, vpTlo);
+                                                                    invw32, vp32, vp32lo, omT32, vpT32, vpTlo, wrange);
     return cudaGetLastError();
 }
 
-__global__ void occupations_kernel(int nm, const double *om, double x_per_w, double *occ,
-                                   float *occ32) {
+__global__ void occupations_kernel(int nm, const double *om, const float *om32, const float *om32lo,
+                                   const float *invw32, double x_per_w, double *occ, float *occ32, float4 *mode4) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nm) return;
     const double w = om[i];
     const double n = w > 0.0 ? 1.0 / expm1(w * x_per_w) : 0.0;
     occ[i] = n;
     occ32[i] = (float)n;
+    mode4[i] = make_float4(om32[i], om32lo[i], (float)n, invw32[i]);
 }
 
 cudaError_t launch_occupations(const Tables &t, double hbar_over_kT, double *occ, float *occ32,
-                               cudaStream_t s) {
+                               float4 *mode4, cudaStream_t s) {
     const int nm = t.N * t.nb;
-    occupations_kernel<<<(nm + 255) / 256, 256, 0, s>>>(nm, t.om, hbar_over_kT, occ, occ32);
+    occupations_kernel<<<(nm + 255) / 256, 256, 0, s>>>(nm, t.om, t.om32, t.om32lo, t.invw32, hbar_over_kT, occ,
+                                                        occ32, mode4);
     return cudaGetLastError();
 }
 

@@ -174,6 +174,37 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
     return n;
 }
 
+// One row of the window of (λ, λ'; q''): bit j'' set iff the process with λ''' = (q3, j3) is kept,
+// restricted to the triangular domain.  A row none of whose |Δ32| can reach the window (FP32 sums are
+// monotonic in ω''; lo2, hi2: range of s2 ω'' over the participating branches; thr bounds the window of
+// every pair) is decided without looking at its pairs.
+template <int NB, bool ADA>
+__device__ __forceinline__ unsigned window_row(const Tables &t, const RateArgs &a, int ch, int s2, float base32,
+                                               int m0, int m1, int j1, double w0, int q2, int q3, unsigned v2,
+                                               int j3, int tri, float lo2, float hi2, float thr) {
+    const float w3 = t.om32[q3 * NB + j3];
+    if ((base32 + lo2) - w3 > thr || (base32 + hi2) - w3 < -thr) return 0u;
+    const unsigned dom = tri == 2 ? (2u << j3) - 1u : tri == 3 ? ~((1u << j1) - 1u) : ~0u;
+    if constexpr (ADA) {
+        return window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3 * NB + j3, v2) & dom;
+    } else {
+        unsigned near = 0;
+#pragma unroll
+        for (int j2 = 0; j2 < NB; ++j2)
+            near |= (unsigned)(fabsf((base32 + (float)s2 * t.om32[q2 * NB + j2]) - w3) <= a.hi32) << j2;
+        near &= v2 & dom;
+        unsigned m = 0;
+        while (near) {
+            const int j2 = __ffs(near) - 1;
+            near &= near - 1;
+            const float ad = fabsf((base32 + (float)s2 * t.om32[q2 * NB + j2]) - w3);
+            if (ad <= a.lo32 || window_exact4(ch, w0, t.om[m1], t.om[q2 * NB + j2], t.om[q3 * NB + j3], a.two_sigma))
+                m |= 1u << j2;
+        }
+        return m;
+    }
+}
+
 // Kahan-compensated FP32 accumulator (mixed path) / plain FP64 accumulator (FP64 path).
 template <typename R> struct Acc {
     double s = 0.0;
@@ -191,28 +222,77 @@ template <> struct Acc<float> {
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
+// Shared memory of the general kernel (dynamic).  W of one j' is built in pieces of as many clusters as
+// the evaluation's buffers hold; both phases share that space.
+constexpr int kSubBatch = 64;      // entries expanded into items at a time
+template <typename R, int NA>
+struct GeneralSmem {
+    using C = Cplx<R>;
+    static constexpr int NB = 3 * NA;
+    static constexpr bool XROUTE = NA <= 2;
+    C *W, *Ph, *E, *e0, *Con;
+    unsigned long long *Q;         // X route: entries (q'', masks) [kQChunk]
+    unsigned short *ent;           // else: entries (q'') [kQChunk]
+    unsigned *mask;                // [NB][kSubBatch] kept j'' per (j''', entry of the sub-batch)
+    unsigned long long *item;      // [kSubBatch * NB]
+    R *proc;                       // [128 * NB][2] weight and |V|^2 of a pass' processes
+    int n_con;                     // clusters per piece
+    __host__ __device__ static size_t buffer_bytes() {
+        const size_t ev = XROUTE ? sizeof(unsigned long long) * kQChunk
+                                 : sizeof(unsigned) * NB * kSubBatch + sizeof(unsigned long long) * kSubBatch * NB +
+                                       2 * sizeof(R) * 128 * NB;
+        return ev > 16384 ? ev : 16384;
+    }
+    __host__ __device__ static size_t bytes(const Tables &t) {
+        size_t b = sizeof(C) * ((size_t)t.n_keys * 9 + t.nc4 + NA * NA * 9 + NB + (NB & 1)) + buffer_bytes() +
+                   (XROUTE ? 0 : sizeof(unsigned short) * kQChunk);
+        return (b + 15) & ~size_t(15);
+    }
+    __device__ __forceinline__ GeneralSmem(unsigned char *smem, const Tables &t) {
+        e0 = reinterpret_cast<C *>(smem);                           // [NB]       e_λ
+        E = e0 + NB + (NB & 1);                                     // [NA*NA*9]  e_λ(aα) e^s1_λ'(bβ)
+        W = E + NA * NA * 9;                                        // [n_keys * 9]
+        Ph = W + t.n_keys * 9;                                      // [nc4]      phase of a cluster at (q, q')
+        unsigned char *buf = reinterpret_cast<unsigned char *>(
+            (reinterpret_cast<size_t>(Ph + t.nc4) + 15) & ~size_t(15));
+        Con = reinterpret_cast<C *>(buf);                           // [n_con * 9] per-cluster terms
+        n_con = (int)(buffer_bytes() / (9 * sizeof(C)));
+        Q = reinterpret_cast<unsigned long long *>(buf);
+        item = reinterpret_cast<unsigned long long *>(buf);
+        proc = reinterpret_cast<R *>(item + kSubBatch * NB);
+        mask = reinterpret_cast<unsigned *>(proc + 2 * 128 * NB);
+        ent = reinterpret_cast<unsigned short *>(buf + buffer_bytes());
+    }
+};
+
 // One (λ, q') unit of the general kernel, run by the whole block (the body of rates4_kernel and of
 // the batched persistent kernel, which takes its units from a work list over many contexts).
+//
+// Up to two atoms, X[c,d][γδ] = Σ_r P_r W_r[γδ] is formed once per entry (q'') by the entry's thread, then
+// 36 complex multiply-adds per (q'', j''') item.  Larger cells list their entries, expand them into
+// items a sub-batch at a time and take one item per thread: an item's Y (12 n_keys complex multiply-
+// adds) is the bulk of the work, and entries carry 1 to nb of them.  The weights of a pass go
+// through shared memory to the entry's owner thread, which adds them in order, so Γ's bits are those
+// of a thread that walks its entries alone.
+// Bound: latency of the item work at 3-4 blocks per SM.  One thread per entry walked its items alone (20
+// entries on 128 threads at 4^3) and formed the window three times: one q point of 4^3 with eight
+// atoms 314 -> 26 ms (three channels), three q points of 5x5x4 with four atoms and adaptive σ 68 -> 24 ms.
 template <typename R, int NA, bool ADA>
 __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, int ch, int unit) {
     using C = Cplx<R>;
+    using Smem = GeneralSmem<R, NA>;
     constexpr int NB = 3 * NA;
-    // X-route (FP32, <= 2 atoms): X[c,d][γδ] = Σ_r P_r W_r[γδ] once per q'', then 36 complex
-    // MACs per (q'', j''') item.  Otherwise Y[cγ] is contracted key by key per item.
-    constexpr bool XROUTE = (sizeof(R) == 4) && (NA <= 2);
+    constexpr bool XROUTE = Smem::XROUTE;
     const int s1 = (ch == 4) ? -1 : 1;
     const int s2 = (ch == 2) ? 1 : -1;
     const int N = t.N;
 
     extern __shared__ __align__(16) unsigned char smem[];
-    C *sW = reinterpret_cast<C *>(smem);                        // [n_keys * 9]
-    C *sCon = sW + t.n_keys * 9;                                // [nc4 * 9]  per-cluster terms
-    C *sE = sCon + t.nc4 * 9;                                   // [NA*NA*9]  e_λ(aα) e^s1_λ'(bβ)
-    C *se0 = sE + NA * NA * 9;                                  // [NB]       e_λ
-    unsigned long long *sQ = reinterpret_cast<unsigned long long *>(se0 + NB + (NB & 1));  // [kQChunk]
+    const Smem sm(smem, t);
     __shared__ int s_scan[32];
-    __shared__ double s_red[32];
-    __shared__ long long s_redn[32];
+    __shared__ int s_off[XROUTE ? 1 : 129];                     // process offset of each item of a pass
+    __shared__ double s_red[2 * 32];
+    __shared__ long long s_redn[5 * 32];
 
     const int ms = unit / N, q1 = unit - ms * N;
     const int m0 = a.modes[ms];
@@ -235,7 +315,33 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
         const double w0 = t.om[m0];
         const float w0f = t.om32[m0];
         const unsigned vm1 = t.vmask[q1];
-        for (int k = threadIdx.x; k < NB; k += blockDim.x) se0[k] = ev[(q0 * NB + k) * NB + j0];
+        __syncthreads();                           // batched form: the previous unit is done with Ph
+        for (int k = threadIdx.x; k < NB; k += blockDim.x) sm.e0[k] = ev[(q0 * NB + k) * NB + j0];
+        for (int c = threadIdx.x; c < t.nc4; c += blockDim.x)
+            sm.Ph[c] = rt[mod_pos(s1 * phase_index(c1, t.c4_r13[c], t.L) - phase_index(c0, t.c4_r3[c], t.L), t.L)];
+
+        // weight of one process, times the number of processes it stands for
+        auto weight = [&](int m1, double w1, int m2, int m3, int wt) -> R {
+            R w;
+            if constexpr (sizeof(R) == 8) {
+                const double d = delta_exact(ch, w0, w1, t.om[m2], t.om[m3]);
+                double g;
+                if constexpr (ADA) g = gauss_adaptive(t, a, d, m2, m3);
+                else g = exp(-(d * d) * a.inv_sigma2) * a.gnorm;
+                w = sym4<double>(ch) * occupation_factor<double>(ch, occ[m1], occ[m2], occ[m3]) *
+                    g * invw[m0] * invw[m1] * invw[m2] * invw[m3];
+            } else {
+                const float4 k0 = t.mode4[m0], k1 = t.mode4[m1], k2 = t.mode4[m2], k3 = t.mode4[m3];
+                const float df = delta_comp(k0.x, k0.y, k1.x, k1.y, k2.x, k2.y, k3.x, k3.y, s1, s2);
+                float g;
+                if constexpr (ADA) g = gauss_adaptive32(t, a, df, m2, m3);
+                else g = __expf(-(df * df) * a.inv_sigma2_32) * a.gnorm32;
+                w = sym4<float>(ch) * occupation_factor<float>(ch, k1.z, k2.z, k3.z) * g *
+                    (k0.w * k1.w) * (k2.w * k3.w);
+            }
+            w *= (R)wt;
+            return w;
+        };
 
         for (int j1 = 0; j1 < NB; ++j1) {
             if (!((vm1 >> j1) & 1u)) continue;
@@ -246,30 +352,32 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                 const int at = ab / NA, bt = ab - at * NA;
                 const int al = ij / 3, be = ij - al * 3;
                 C y = cconj_if(ev[(q1 * NB + 3 * bt + be) * NB + j1], s1 < 0);
-                sE[k] = cmul(se0[3 * at + al], y);
+                sm.E[k] = cmul(sm.e0[3 * at + al], y);
             }
-            __syncthreads();
-            // per-cluster terms exp(-i q.R3 + i s1 q'.(R1 - R3)) / sqrt(m) Σ_αβ Φ[αβγδ] E[αβ]
-            for (int k = threadIdx.x; k < t.nc4 * 9; k += blockDim.x) {
-                const int c = k / 9, gd = k - c * 9;
-                const int4 at = t.c4_at[c];
-                const int idx = mod_pos(s1 * phase_index(c1, t.c4_r13[c], t.L) -
-                                            phase_index(c0, t.c4_r3[c], t.L), t.L);
-                const R *ph4 = phi4 + 81 * c + gd;
-                const C *E = sE + (at.x * NA + at.y) * 9;
-                C v = czero<C>();
+            // W_r[γδ]: per-cluster terms exp(-i q.R3 + i s1 q'.(R1 - R3)) / sqrt(m) Σ_αβ Φ[αβγδ] E[αβ] of a
+            // piece, added to their keys in cluster order (deterministic)
+            for (int cb = 0; cb < t.nc4; cb += sm.n_con) {
+                const int ce = min(t.nc4, cb + sm.n_con);
+                __syncthreads();
+                for (int k = threadIdx.x; k < (ce - cb) * 9; k += blockDim.x) {
+                    const int c = cb + k / 9, gd = k % 9;
+                    const int4 at = t.c4_at[c];
+                    const R *ph4 = phi4 + 81 * c + gd;
+                    const C *E = sm.E + (at.x * NA + at.y) * 9;
+                    C v = czero<C>();
 #pragma unroll
-                for (int ab = 0; ab < 9; ++ab) v = crfma(ph4[9 * ab], E[ab], v);
-                const C p = cmul(rt[idx], v);
-                sCon[k] = cmake(p.x * ism4[c], p.y * ism4[c]);
-            }
-            __syncthreads();
-            // W_r[γδ]: clusters of a key summed in order (deterministic)
-            for (int k = threadIdx.x; k < t.n_keys * 9; k += blockDim.x) {
-                const int r = k / 9, gd = k - r * 9;
-                C acc = czero<C>();
-                for (int c = t.key_start[r]; c < t.key_start[r + 1]; ++c) acc = cadd(acc, sCon[c * 9 + gd]);
-                sW[k] = acc;
+                    for (int ab = 0; ab < 9; ++ab) v = crfma(ph4[9 * ab], E[ab], v);
+                    const C p = cmul(sm.Ph[c], v);
+                    sm.Con[k] = cmake(p.x * ism4[c], p.y * ism4[c]);
+                }
+                __syncthreads();
+                for (int k = threadIdx.x; k < t.n_keys * 9; k += blockDim.x) {
+                    const int r = k / 9, gd = k - r * 9;
+                    C acc = cb ? sm.W[k] : czero<C>();
+                    for (int c = max(cb, t.key_start[r]); c < min(ce, t.key_start[r + 1]); ++c)
+                        acc = cadd(acc, sm.Con[(c - cb) * 9 + gd]);
+                    sm.W[k] = acc;
+                }
             }
             __syncthreads();
 
@@ -278,61 +386,40 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
             // ++ and -- on their triangle (q'' >= q') start at q'' = q'
             for (int qb = (ch != 3 && (a.tri & 2)) ? q1 : 0; qb < N; qb += kQChunk) {
                 const int qe = min(N, qb + kQChunk);
-                // pass 1: window masks of this thread's q''; the X-route keeps those with a kept
-                // process in a small local list (q'' packed with the 36 mask bits) and counts them
-                constexpr int kPer = kQChunk / 64;              // blockDim >= 64
-                unsigned long long ent[XROUTE ? kPer : 1];
-                int n_act = 0;
-                for (int q2 = qb + threadIdx.x; q2 < qe; q2 += blockDim.x) {
-                    const int4 c2 = t.qc[q2];
-                    const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
-                                           t.mesh[0], t.mesh[1], t.mesh[2]);
-                    unsigned mask[NB];
-                    if (tri_code_sampled(a, ch, m0, q1, q2, q3, N) >= 0) acc_cev += NB * NB;   // visited
-                    if (window_masks<NB, ADA>(t, a, ch, s2, base32, m0, m1, w0, w1, q2, q3, mask) > 0) {
-                        if constexpr (XROUTE) {
-                            unsigned long long e = (unsigned long long)q2 << 40;
-#pragma unroll
-                            for (int j3 = 0; j3 < NB; ++j3) e |= (unsigned long long)mask[j3] << (NB * j3);
-                            ent[n_act] = e;
-                        }
-                        ++n_act;
-                    }
-                }
                 int total;
-                int off = block_exclusive_scan(n_act, s_scan, &total);
-                // pass 2: write them in order
                 if constexpr (XROUTE) {
-                    for (int k = 0; k < n_act; ++k) sQ[off + k] = ent[k];
-                } else if (n_act) {
+                    // window masks of this thread's q''; those with a kept process go to the entry list (q''
+                    // packed with the 36 mask bits)
+                    constexpr int kPer = kQChunk / 64;              // blockDim >= 64
+                    unsigned long long ent[kPer];
+                    int n_act = 0;
                     for (int q2 = qb + threadIdx.x; q2 < qe; q2 += blockDim.x) {
                         const int4 c2 = t.qc[q2];
                         const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
                                                t.mesh[0], t.mesh[1], t.mesh[2]);
                         unsigned mask[NB];
-                        if (window_masks<NB, ADA>(t, a, ch, s2, base32, m0, m1, w0, w1, q2, q3, mask) > 0) sQ[off++] = q2;
-                    }
-                }
-                __syncthreads();
-
-                for (int it = threadIdx.x; it < total; it += blockDim.x) {
-                    ++acc_ent;
-                    const unsigned long long e = sQ[it];
-                    const int iq2 = XROUTE ? (int)(e >> 40) : (int)e;
-                    const int4 c2 = t.qc[iq2];
-                    const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
-                                           t.mesh[0], t.mesh[1], t.mesh[2]);
-                    unsigned mask[NB];
-                    const int tri = tri_code_sampled(a, ch, m0, q1, iq2, q3, N);
-                    if constexpr (XROUTE) {
+                        if (tri_code_sampled(a, ch, m0, q1, q2, q3, N) >= 0) acc_cev += NB * NB;   // visited
+                        if (window_masks<NB, ADA>(t, a, ch, s2, base32, m0, m1, w0, w1, q2, q3, mask) > 0) {
+                            unsigned long long e = (unsigned long long)q2 << 40;
 #pragma unroll
-                        for (int j3 = 0; j3 < NB; ++j3) mask[j3] = (unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u);
-                    } else {
-                        window_masks<NB, ADA>(t, a, ch, s2, base32, m0, m1, w0, w1, iq2, q3, mask);
+                            for (int j3 = 0; j3 < NB; ++j3) e |= (unsigned long long)mask[j3] << (NB * j3);
+                            ent[n_act++] = e;
+                        }
                     }
-                    const C *P = P4 + (size_t)iq2 * t.n_keys;
-                    C X[XROUTE ? NA : 1][XROUTE ? NA : 1][9];
-                    if constexpr (XROUTE) {
+                    const int off = block_exclusive_scan(n_act, s_scan, &total);
+                    for (int k = 0; k < n_act; ++k) sm.Q[off + k] = ent[k];
+                    __syncthreads();
+
+                    for (int it = threadIdx.x; it < total; it += blockDim.x) {
+                        ++acc_ent;
+                        const unsigned long long e = sm.Q[it];
+                        const int iq2 = (int)(e >> 40);
+                        const int4 c2 = t.qc[iq2];
+                        const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
+                                               t.mesh[0], t.mesh[1], t.mesh[2]);
+                        const int tri = tri_code_sampled(a, ch, m0, q1, iq2, q3, N);
+                        const C *P = P4 + (size_t)iq2 * t.n_keys;
+                        C X[NA][NA][9];
 #pragma unroll
                         for (int c = 0; c < NA; ++c)
 #pragma unroll
@@ -342,23 +429,21 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                                 const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
                                 for (int r = r0; r < r1; ++r) {
                                     const C ph = cconj_if(P[r], s2 < 0);
-                                    const C *Wr = sW + 9 * r;
+                                    const C *Wr = sm.W + 9 * r;
 #pragma unroll
                                     for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
                                 }
                             }
-                    }
 #pragma unroll 1
-                    for (int j3 = 0; j3 < NB; ++j3) {
-                        unsigned m = mask[j3];
-                        if (!m) continue;
-                        ++acc_items;
-                        C Y[NA][3];
+                        for (int j3 = 0; j3 < NB; ++j3) {
+                            unsigned m = (unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u);
+                            if (!m) continue;
+                            ++acc_items;
+                            C Y[NA][3];
 #pragma unroll
-                        for (int c = 0; c < NA; ++c)
+                            for (int c = 0; c < NA; ++c)
 #pragma unroll
-                            for (int g = 0; g < 3; ++g) Y[c][g] = czero<C>();
-                        if constexpr (XROUTE) {
+                                for (int g = 0; g < 3; ++g) Y[c][g] = czero<C>();
                             // Y[cγ] = Σ_dδ X[c,d][γδ] e*_λ'''(dδ)
 #pragma unroll
                             for (int d = 0; d < NA; ++d) {
@@ -372,105 +457,198 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
 #pragma unroll
                                         for (int dl = 0; dl < 3; ++dl) Y[c][g] = cfma(X[c][d][3 * g + dl], e3[dl], Y[c][g]);
                             }
-                        } else {
-                            // Y[cγ] = Σ_d Σ_{r in (c,d)} P_r^s2 Σ_δ W_r[γδ] e*_λ'''(dδ)
+                            const int m3 = q3 * NB + j3;
+                            while (m) {
+                                const int j2 = __ffs(m) - 1;
+                                m &= m - 1;
+                                C V = czero<C>();
 #pragma unroll
-                            for (int c = 0; c < NA; ++c) {
+                                for (int c = 0; c < NA; ++c)
 #pragma unroll
-                                for (int d = 0; d < NA; ++d) {
-                                    const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
-                                    if (r0 == r1) continue;
-                                    C e3[3];
+                                    for (int g = 0; g < 3; ++g)
+                                        V = cfma(cconj_if(ev[(iq2 * NB + 3 * c + g) * NB + j2], s2 < 0), Y[c][g], V);
+                                const int wt = tri_weight(tri, j1, j2, j3);
+                                const R w = weight(m1, w1, iq2 * NB + j2, m3, wt);
+                                acc_wp.add(w);
+                                acc_g.add(w * (V.x * V.x + V.y * V.y));
+                                acc_n += wt;
+                                acc_ev += 1;
+                            }
+                        }
+                    }
+                } else {
+                    // closure, domain and window range of a q''
+                    struct Point { int q3, tri; unsigned v2, v3; float lo2, hi2, thr; };
+                    auto point = [&](int q2) -> Point {
+                        Point z;
+                        const int4 c2 = t.qc[q2];
+                        z.q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z, t.mesh[0], t.mesh[1], t.mesh[2]);
+                        z.tri = tri_code_sampled(a, ch, m0, q1, q2, z.q3, N);
+                        z.v2 = t.vmask[q2];
+                        z.v3 = t.vmask[z.q3];
+                        const float4 r2 = t.wrange[q2], r3 = t.wrange[z.q3];
+                        z.lo2 = s2 > 0 ? r2.x : -r2.y;
+                        z.hi2 = s2 > 0 ? r2.y : -r2.x;
+                        z.thr = ADA ? fmaf(a.ad_rhi, a.ad_c32 * (r2.z + r3.z), a.ad_e0) : a.hi32;
+                        return z;
+                    };
+                    auto row = [&](const Point &z, int q2, int j3) -> unsigned {
+                        return ((z.v3 >> j3) & 1u) ? window_row<NB, ADA>(t, a, ch, s2, base32, m0, m1, j1, w0, q2, z.q3,
+                                                                         z.v2, j3, z.tri, z.lo2, z.hi2, z.thr)
+                                                   : 0u;
+                    };
+                    unsigned found = 0;                             // bit i: this thread's i-th q'' is an entry
+                    int i = 0;
+                    for (int q2 = qb + threadIdx.x; q2 < qe; q2 += blockDim.x, ++i) {
+                        const Point z = point(q2);
+                        if (z.tri < 0) continue;
+                        acc_cev += NB * NB;                         // visited
+#pragma unroll 1
+                        for (int j3 = 0; j3 < NB; ++j3)
+                            if (row(z, q2, j3)) {
+                                found |= 1u << i;
+                                break;
+                            }
+                    }
+                    int off = block_exclusive_scan(__popc(found), s_scan, &total);
+                    for (; found; found &= found - 1)
+                        sm.ent[off++] = (unsigned short)((__ffs(found) - 1) * blockDim.x + threadIdx.x);
+                    __syncthreads();
+
+                    const int sub = blockDim.x % kSubBatch ? 32 : kSubBatch;
+                    for (int eb = 0; eb < total; eb += sub) {
+                        // expand: the entry's owner (the thread it % blockDim of the whole list) lists its items
+                        const int mine = (int)threadIdx.x - eb % (int)blockDim.x;     // slot in the sub-batch
+                        const bool own = mine >= 0 && mine < sub && eb + mine < total;
+                        int n_it = 0, q2 = 0, tri = 0;
+                        if (own) {
+                            ++acc_ent;
+                            q2 = qb + sm.ent[eb + mine];
+                            const Point z = point(q2);
+                            tri = z.tri;
+#pragma unroll 1
+                            for (int j3 = 0; j3 < NB; ++j3) {
+                                const unsigned m = row(z, q2, j3);
+                                sm.mask[j3 * kSubBatch + mine] = m;
+                                n_it += m != 0;
+                            }
+                        }
+                        int n_items;
+                        const int it0 = block_exclusive_scan(n_it, s_scan, &n_items), it1 = it0 + n_it;
+                        if (own) {
+                            int o = it0;
+#pragma unroll 1
+                            for (int j3 = 0; j3 < NB; ++j3) {
+                                const unsigned m = sm.mask[j3 * kSubBatch + mine];
+                                if (m) sm.item[o++] = ((unsigned long long)(unsigned)q2 << 36) | ((unsigned long long)tri << 32) |
+                                                      ((unsigned long long)j3 << 24) | m;
+                            }
+                        }
+                        __syncthreads();
+                        for (int pb = 0; pb < n_items; pb += blockDim.x) {
+                            const int n_pass = min((int)blockDim.x, n_items - pb);
+                            unsigned long long e = 0;
+                            if ((int)threadIdx.x < n_pass) e = sm.item[pb + threadIdx.x];
+                            unsigned m = (unsigned)e & 0xffffffu;
+                            int n_proc;
+                            int po = block_exclusive_scan(__popc(m), s_scan, &n_proc);
+                            if ((int)threadIdx.x < n_pass) s_off[threadIdx.x] = po;
+                            if (threadIdx.x == 0) s_off[n_pass] = n_proc;
+                            if (m) {
+                                ++acc_items;
+                                const int iq2 = (int)(e >> 36), itri = (int)((e >> 32) & 3u), j3 = (int)((e >> 24) & 0xffu);
+                                const int4 c2 = t.qc[iq2];
+                                const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
+                                                       t.mesh[0], t.mesh[1], t.mesh[2]);
+                                const C *P = P4 + (size_t)iq2 * t.n_keys;
+                                // Y[cγ] = Σ_d Σ_{r in (c,d)} P_r^s2 Σ_δ W_r[γδ] e*_λ'''(dδ)
+                                C Y[NA][3];
 #pragma unroll
-                                    for (int dl = 0; dl < 3; ++dl) e3[dl] = cconj(ev[(q3 * NB + 3 * d + dl) * NB + j3]);
-                                    for (int r = r0; r < r1; ++r) {
-                                        const C ph = cconj_if(P[r], s2 < 0);
-                                        const C *Wr = sW + 9 * r;
+                                for (int c = 0; c < NA; ++c) {
 #pragma unroll
-                                        for (int g = 0; g < 3; ++g) {
-                                            C u = cmul(Wr[3 * g], e3[0]);
-                                            u = cfma(Wr[3 * g + 1], e3[1], u);
-                                            u = cfma(Wr[3 * g + 2], e3[2], u);
-                                            Y[c][g] = cfma(ph, u, Y[c][g]);
+                                    for (int g = 0; g < 3; ++g) Y[c][g] = czero<C>();
+#pragma unroll 1
+                                    for (int d = 0; d < NA; ++d) {
+                                        const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
+                                        if (r0 == r1) continue;
+                                        C e3[3];
+#pragma unroll
+                                        for (int dl = 0; dl < 3; ++dl) e3[dl] = cconj(ev[(q3 * NB + 3 * d + dl) * NB + j3]);
+                                        for (int r = r0; r < r1; ++r) {
+                                            const C ph = cconj_if(P[r], s2 < 0);
+                                            const C *Wr = sm.W + 9 * r;
+#pragma unroll
+                                            for (int g = 0; g < 3; ++g) {
+                                                C u = cmul(Wr[3 * g], e3[0]);
+                                                u = cfma(Wr[3 * g + 1], e3[1], u);
+                                                u = cfma(Wr[3 * g + 2], e3[2], u);
+                                                Y[c][g] = cfma(ph, u, Y[c][g]);
+                                            }
                                         }
                                     }
                                 }
-                            }
-                        }
-                        const int m3 = q3 * NB + j3;
-                        const R n3 = occ[m3], iw3 = invw[m3];
-                        while (m) {
-                            const int j2 = __ffs(m) - 1;
-                            m &= m - 1;
-                            const int m2 = iq2 * NB + j2;
-                            C V = czero<C>();
+                                const int m3 = q3 * NB + j3;
+                                    while (m) {
+                                    const int j2 = __ffs(m) - 1;
+                                    m &= m - 1;
+                                    C V = czero<C>();
 #pragma unroll
-                            for (int c = 0; c < NA; ++c)
+                                    for (int c = 0; c < NA; ++c)
 #pragma unroll
-                                for (int g = 0; g < 3; ++g)
-                                    V = cfma(cconj_if(ev[(iq2 * NB + 3 * c + g) * NB + j2], s2 < 0), Y[c][g], V);
-                            R w;
-                            if constexpr (sizeof(R) == 8) {
-                                const double d = delta_exact(ch, w0, w1, t.om[m2], t.om[m3]);
-                                double g;
-                                if constexpr (ADA) g = gauss_adaptive(t, a, d, m2, m3);
-                                else g = exp(-(d * d) * a.inv_sigma2) * a.gnorm;
-                                w = sym4<double>(ch) * occupation_factor<double>(ch, occ[m1], occ[m2], n3) *
-                                    g * invw[m0] * invw[m1] * invw[m2] * iw3;
-                            } else {
-                                const float df = delta_comp(t.om32[m0], t.om32lo[m0], t.om32[m1], t.om32lo[m1],
-                                                            t.om32[m2], t.om32lo[m2], t.om32[m3], t.om32lo[m3], s1, s2);
-                                float g;
-                                if constexpr (ADA) g = gauss_adaptive32(t, a, df, m2, m3);
-                                else g = __expf(-(df * df) * a.inv_sigma2_32) * a.gnorm32;
-                                w = sym4<float>(ch) * occupation_factor<float>(ch, occ[m1], occ[m2], n3) * g *
-                                    (invw[m0] * invw[m1]) * (invw[m2] * iw3);
+                                        for (int g = 0; g < 3; ++g)
+                                            V = cfma(cconj_if(ev[(iq2 * NB + 3 * c + g) * NB + j2], s2 < 0), Y[c][g], V);
+                                    const int wt = tri_weight(itri, j1, j2, j3);
+                                    const R w = weight(m1, w1, iq2 * NB + j2, m3, wt);
+                                    sm.proc[2 * po] = w;
+                                    sm.proc[2 * po + 1] = V.x * V.x + V.y * V.y;
+                                    ++po;
+                                    acc_n += wt;
+                                    acc_ev += 1;
+                                }
                             }
-                            const int wt = tri_weight(tri, j1, j2, j3);
-                            w *= (R)wt;
-                            acc_wp.add(w);
-                            acc_g.add(w * (V.x * V.x + V.y * V.y));
-                            acc_n += wt;
-                            acc_ev += 1;
+                            __syncthreads();
+                            // the owner adds its entry's processes of this pass, in order
+                            const int lo = max(it0, pb) - pb, hi = min(it1, pb + n_pass) - pb;
+                            if (lo < hi)
+                                for (int k = s_off[lo]; k < s_off[hi]; ++k) {
+                                    acc_wp.add(sm.proc[2 * k]);
+                                    acc_g.add(sm.proc[2 * k] * sm.proc[2 * k + 1]);
+                                }
+                            __syncthreads();       // proc, s_off and item reused
                         }
                     }
                 }
-                __syncthreads();                   // sQ reused by the next chunk
+                __syncthreads();                   // the entry list is reused by the next chunk
             }
         }
     }
-    const double g = block_sum(acc_g.value(), s_red);
-    const double wp = block_sum(acc_wp.value(), s_red);
-    const long long n = block_sum(acc_n, s_redn);
-    const long long ni = block_sum(acc_items, s_redn);
-    const long long ne = block_sum(acc_ent, s_redn);
-    const long long nev = block_sum(acc_ev, s_redn);
-    const long long ncv = block_sum(acc_cev, s_redn);
+    double sums[2] = {acc_g.value(), acc_wp.value()};
+    long long cnts[5] = {acc_n, acc_items, acc_ent, acc_ev, acc_cev};
+    block_sum_multi<2, 5>(sums, cnts, s_red, s_redn);
     if (threadIdx.x == 0) {
         const size_t o = ((size_t)ch * a.n_modes + ms) * N + q1;
-        a.part_g[o] = g;
-        a.part_wp[o] = wp;
-        a.part_n[o] = n;
-        a.part_items[o] = ni;
-        a.part_ent[o] = ne;
-        if (a.part_ev) a.part_ev[o] = nev;
-        if (a.part_cev) a.part_cev[o] = ncv;
+        a.part_g[o] = sums[0];
+        a.part_wp[o] = sums[1];
+        a.part_n[o] = cnts[0];
+        a.part_items[o] = cnts[1];
+        a.part_ent[o] = cnts[2];
+        if (a.part_ev) a.part_ev[o] = cnts[3];
+        if (a.part_cev) a.part_cev[o] = cnts[4];
     }
 }
 
+// Blocks per SM: 4 (128 registers); FP64 cells of up to two atoms hold X (2 blocks, 255 registers).
+template <typename R, int NA> constexpr int general_blocks() { return sizeof(R) == 8 && NA <= 2 ? 2 : 4; }
+
 template <typename R, int NA, bool ADA>
-__global__ void __launch_bounds__(128, 4)
+__global__ void __launch_bounds__(128, general_blocks<R, NA>())
 rates4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int ch) {
     rates4_unit<R, NA, ADA>(t, a, ch, blockIdx.x);
 }
 
 template <typename R, int NA, bool ADA>
 cudaError_t launch4(const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s) {
-    using C = Cplx<R>;
-    constexpr int NB = 3 * NA;
-    size_t smem = sizeof(C) * ((size_t)t.n_keys * 9 + (size_t)t.nc4 * 9 + NA * NA * 9 + NB) +
-                  sizeof(C) + sizeof(unsigned long long) * (size_t)kQChunk;
-    smem = (smem + 15) & ~size_t(15);
+    const size_t smem = GeneralSmem<R, NA>::bytes(t);
     cudaError_t e = cudaFuncSetAttribute(rates4_kernel<R, NA, ADA>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -485,13 +663,7 @@ cudaError_t launch4(const Tables &t, const RateArgs &a, int ch, int threads, cud
 
 // Dynamic shared memory of the general kernel for one context's tables.
 template <typename R, int NA>
-size_t general_smem_bytes(const Tables &t) {
-    using C = Cplx<R>;
-    constexpr int NB = 3 * NA;
-    size_t smem = sizeof(C) * ((size_t)t.n_keys * 9 + (size_t)t.nc4 * 9 + NA * NA * 9 + NB) +
-                  sizeof(C) + sizeof(unsigned long long) * (size_t)kQChunk;
-    return (smem + 15) & ~size_t(15);
-}
+size_t general_smem_bytes(const Tables &t) { return GeneralSmem<R, NA>::bytes(t); }
 
 template <typename R, int NA, int HI>
 size_t general_smem_atoms(int na, const Tables &t) {
