@@ -141,7 +141,37 @@ __device__ __forceinline__ float vel_diff_norm32(float4 ha, float4 la, float4 hb
     return __fsqrt_rn(x * x + y * y + z * z);
 }
 
+// The same for a prefilter only: sqrt.approx (relative error at most 2^-23 = 2u) in place of the rounded
+// square root, which takes more instructions than the rest of the width.
+__device__ __forceinline__ float vel_diff_norm32_approx(float4 ha, float4 la, float4 hb, float4 lb) {
+    const float x = (ha.x - hb.x) + (la.x - lb.x);
+    const float y = (ha.y - hb.y) + (la.y - lb.y);
+    const float z = (ha.z - hb.z) + (la.z - lb.z);
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x * x + y * y + z * z));
+    return r;
+}
+
 // ------------------------------------------------------------------------------ block helpers
+
+// Exclusive scan of one int per lane (all lanes of the warp take part).
+__device__ __forceinline__ int warp_exclusive_scan(int v) {
+    const int lane = threadIdx.x & 31;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += y;
+    }
+    return x - v;
+}
+
+// A complex value of another lane (all lanes of the warp take part).
+template <typename C> __device__ __forceinline__ C cshfl(C z, int src) {
+    z.x = __shfl_sync(kFull, z.x, src);
+    z.y = __shfl_sync(kFull, z.y, src);
+    return z;
+}
 
 // Exclusive scan of one int per thread across the block (blockDim.x a multiple of 32, <= 1024).
 // Deterministic.  s_warp must hold 32 ints.  Returns the prefix; *total gets the block sum.

@@ -6,7 +6,7 @@
 // σ > σ_min = 1e-9 rad/ps and |Δ| <= 2σ, both in FP64 in the order of the definition (velocities
 // equal by symmetry differ by rounding noise only; the 1/σ weight of such a width is meaningless).  The FP32 prefilter works on
 // P_k = (v . b_k) / n_k stored per mode as hi/lo pairs and on the FP32 mismatch; with
-//   |Δ32 - Δ| <= 13 u ω_max  and  |2σ32 - 2σ| <= 10 u 2σ32 + 2^-41 (2s/√6) Q   (u = 2^-24,
+//   |Δ32 - Δ| <= 13 u ω_max  and  |2σ32 - 2σ| <= 12 u 2σ32 + 2^-41 (2s/√6) Q   (u = 2^-24,
 //   Q >= max_k |P_k| and the FP64 rounding of the oracle's own σ, see the host's margin),
 // a candidate is kept for sure when |Δ32| <= (1 - 32u) 2σ32 - e0 and 2σ32 > g_min (which
 // implies σ > σ_min), rejected for sure when

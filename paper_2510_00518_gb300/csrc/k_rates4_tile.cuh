@@ -39,7 +39,8 @@ constexpr int kTriChunk = 1024;
 // cluster phases are folded first, per key r and leg-1 atom b,
 //   Ψ_rb[β][γδ] = Σ_{c in r, b(c) = b} exp(i(s1 q'.(R1 - R3) - q.R3)) Φ~_c[β][γδ]   (fixed order),
 // and then W_r[γδ] = Σ_b Σ_β e^s1_λ'(bβ) Ψ_rb[β][γδ] for every j' (coalesced writes): the phase
-// work is shared by all partner branches.
+// work is shared by all partner branches.  FP64: the work is spread evenly over the threads, which the FP64
+// pipe needs (4.7 ms for both signs of 4 q points of 8^3, against 5.7 ms for the column kernel below).
 constexpr int kW4Group = 8;
 
 constexpr int kW4Threads = 256;
@@ -253,6 +254,8 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                    int mode0, const Cplx<R> *__restrict__ wall) {
     using C = Cplx<R>;
     constexpr int NB = 3 * NA;
+    constexpr bool WARP = sizeof(R) == 8 && !NOCOMP;
+    constexpr bool SPARSE = !ADA && kQPT == qpt_of<ADA>(false) && !NOCOMP;
     const int s1 = (ch == 4) ? -1 : 1;
     const int s2 = (ch == 2) ? 1 : -1;
     const int N = t.N, nk = t.n_keys;
@@ -260,11 +263,19 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     extern __shared__ __align__(16) unsigned char smem[];
     C *sW = reinterpret_cast<C *>(smem);                        // [NB][nk][9]
     unsigned long long *sQ = reinterpret_cast<unsigned long long *>(sW + NB * nk * 9);   // [kTileQ * NB * kQPT]
+    // SPARSE: candidates [kTileQ * NB * kQPT] in the upper half of sQ (entry o is written after candidate
+    // o + 127 has been read at the latest, so the two lists never meet)
+    unsigned *sC = reinterpret_cast<unsigned *>(sQ) + kTileQ * NB * kQPT;
     float *s_g = reinterpret_cast<float *>(sQ + kTileQ * NB * kQPT);   // adaptive σ: [NB * NB][kTileQ] widths
     __shared__ int s_scan[32];
     __shared__ double s_red[(BTE ? 5 : 2) * 32];
     __shared__ long long s_redn[5 * 32];
     __shared__ unsigned short s_tri[kTriChunk];                 // +- triangle: q'' - chunk start
+    // per warp, of one pass: its items (entry lane, j'''), their processes (item lane, j'') and the
+    // processes' weight, weight |V|^2 (and BTE terms)
+    constexpr int NV = BTE ? 5 : 2;
+    __shared__ unsigned char s_item[WARP ? kTileQ * NB : 1], s_proc[WARP ? kTileQ * NB : 1];
+    __shared__ R s_val[WARP ? kTileQ * NB * NV : 1];
 
     const int unit = blockIdx.x;                                // (mode - mode0) * N + q'
     const int ml = unit / N, q1 = unit - ml * N;
@@ -322,8 +333,122 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
             __syncthreads();
           }
           for (int qb = 0; qb < cnt; qb += kTileQ * kQPT) {
+            int total, n_ent = 0, off = 0;
+            if constexpr (SPARSE) {
+                // ++, --: few (q'', j') have a pair near the window.  Pass 1 tests every q'' of the round with
+                // cheap bounds and lists the (q'', j') left, in order; pass 2 takes that list one pair per
+                // thread, so the mask work runs on full warps, and lists the entries (all modes of 8^3, ++ and
+                // --: 126.6 -> 121.9 ms on top of the packed mode scalars; with the candidates in shared memory
+                // of their own, which the L1 then lacks, it gained nothing).
+                unsigned cand[kQPT];
+                int n_cand = 0;
+#pragma unroll
+                for (int k = 0; k < kQPT; ++k) {
+                    cand[k] = 0;
+                    const int q2 = cb + qb + k * kTileQ + (int)threadIdx.x;
+                    if (q2 >= N) continue;
+                    const int4 c2 = t.qc[q2];
+                    const int q3 = q_index_near(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
+                                                t.mesh[0], t.mesh[1], t.mesh[2]);
+                    const int tri = tri_code_sampled(a, ch, m0, q1, q2, q3, N);
+                    if (tri < 0) continue;
+                    acc_cev += NB * NB * NB;                     // this q'' is visited
+                    // |Δ32| of every pair lies in [b + min ω'' - max ω''', b + max ω'' - min ω''']
+                    // (FP32 sums are monotonic)
+                    const float4 r2 = t.wrange[q2], r3 = t.wrange[q3];
+                    const float lo2 = s2 > 0 ? r2.x : -r2.y, hi2 = s2 > 0 ? r2.y : -r2.x;
+                    const float thr = a.hi32;
+                    unsigned near = 0;
+#pragma unroll
+                    for (int j1 = 0; j1 < NB; ++j1)
+                        if (((base32[j1] + lo2) - r3.y) <= thr && ((base32[j1] + hi2) - r3.x) >= -thr) near |= 1u << j1;
+                    near &= vm1;
+                    if (!near) continue;
+                    float w2f[NB], w3f[NB];
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) {
+                        w2f[j] = (float)s2 * t.omT32[j * N + q2];   // branch-major: lanes read consecutive q
+                        w3f[j] = t.omT32[j * N + q3];
+                    }
+#pragma unroll
+                    for (int j1 = 0; j1 < NB; ++j1) {
+                        if (!((near >> j1) & 1u)) continue;
+                        float mn = thr + 1.0f;
+#pragma unroll
+                        for (int j2 = 0; j2 < NB; ++j2) {
+                            const float t2 = base32[j1] + w2f[j2];
+                            float r = fabsf(t2 - w3f[0]);        // six short chains
+#pragma unroll
+                            for (int j3 = 1; j3 < NB; ++j3) r = fminf(r, fabsf(t2 - w3f[j3]));
+                            mn = fminf(mn, r);
+                        }
+                        if (!(mn <= thr)) near &= ~(1u << j1);
+                    }
+                    cand[k] = near | ((unsigned)tri << 8);
+                    n_cand += __popc(near);
+                }
+                int n_all, co = block_exclusive_scan(n_cand, s_scan, &n_all);
+#pragma unroll
+                for (int k = 0; k < kQPT; ++k)
+                    for (unsigned m = cand[k] & 0xffu; m; m &= m - 1)
+                        sC[co++] = ((unsigned)(k * kTileQ + threadIdx.x) << 16) | ((unsigned)(__ffs(m) - 1) << 8) |
+                                   (cand[k] >> 8);
+                __syncthreads();
+                total = 0;
+                for (int cf = 0; cf < n_all; cf += kTileQ) {
+                    unsigned long long e = 0;
+                    if (cf + (int)threadIdx.x < n_all) {
+                        const unsigned cw = sC[cf + threadIdx.x];
+                        const int ixr = (int)(cw >> 16), j1 = (int)((cw >> 8) & 0xffu), tri = (int)(cw & 0xffu);
+                        const int q2 = cb + qb + ixr;
+                        const int4 c2 = t.qc[q2];
+                        const int q3 = q_index_near(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
+                                                    t.mesh[0], t.mesh[1], t.mesh[2]);
+                        const unsigned v2 = t.vmask[q2], v3 = t.vmask[q3];
+                        const float thr = a.hi32;
+                        const float b = w0f + (float)s1 * t.om32[q1 * NB + j1];
+                        unsigned long long near = 0, okm = 0, keep = 0;
+                        float t2[NB];
+#pragma unroll
+                        for (int j2 = 0; j2 < NB; ++j2) t2[j2] = b + (float)s2 * t.om32[q2 * NB + j2];
+                        unsigned row = v2 & ((1u << NB) - 1u);
+                        if (tri == 3) row &= ~((1u << j1) - 1u);             // j'' >= j'
+#pragma unroll
+                        for (int j3 = 0; j3 < NB; ++j3) {
+                            const float w3 = t.om32[q3 * NB + j3];
+                            if ((v3 >> j3) & 1u) okm |= (unsigned long long)row << (NB * j3);
+#pragma unroll
+                            for (int j2 = 0; j2 < NB; ++j2)
+                                near |= (unsigned long long)(fabsf(t2[j2] - w3) <= thr) << (NB * j3 + j2);
+                        }
+                        near &= okm;
+                        while (near) {                           // the few pairs within reach, one by one
+                            const int k = __ffsll(near) - 1;
+                            near &= near - 1;
+                            const int j3 = k / NB, j2 = k - j3 * NB;
+                            const int m2 = q2 * NB + j2, m3 = q3 * NB + j3;
+                            const float ad = fabsf((b + (float)s2 * t.om32[m2]) - t.om32[m3]);
+                            const bool kp = ad <= a.lo32 || window_exact4(ch, w0, t.om[q1 * NB + j1], t.om[m2], t.om[m3],
+                                                                          a.two_sigma);
+                            keep |= (unsigned long long)kp << k;
+                        }
+                        if (keep) e = ((unsigned long long)ixr << 48) | ((unsigned long long)j1 << 40) |
+                                      ((unsigned long long)tri << 36) | keep;
+                    }
+                    const unsigned bal = __ballot_sync(kFull, e != 0);
+                    if ((threadIdx.x & 31) == 0) s_scan[threadIdx.x >> 5] = __popc(bal);
+                    __syncthreads();
+                    int o = total + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
+#pragma unroll
+                    for (int w = 0; w < kTileQ / 32; ++w) {
+                        if (w < (int)(threadIdx.x >> 5)) o += s_scan[w];
+                        total += s_scan[w];
+                    }
+                    if (e) sQ[o] = e;
+                    __syncthreads();
+                }
+            } else {
             // window: this thread's q'' of the round (up to kQPT) against every partner branch j'
-            int n_ent = 0;
             unsigned long long ent[NB * kQPT];
             for (int ix = qb + threadIdx.x; ix < min(cnt, qb + kTileQ * kQPT); ix += kTileQ) {
                 const int q2 = cb + (pm_list ? (int)s_tri[ix] : ix);
@@ -356,6 +481,21 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                         if (tri == 2) row &= (2u << j3) - 1u;    // j'' <= j'''
                         okm |= (unsigned long long)row << (NB * j3);
                     }
+                // Adaptive ++, --: |Δ32| of every pair lies in [b + min ω'' - max ω''', b + max ω'' - min ω''']
+                // (FP32 sums are monotonic), and no width exceeds the one of |P''| + |P'''|: most q'' need none.
+                unsigned j1_near = vm1;
+                if constexpr (ADA) {
+                    if (ch != 3) {
+                        const float4 r2 = t.wrange[q2], r3 = t.wrange[q3];
+                        const float lo2 = s2 > 0 ? r2.x : -r2.y, hi2 = s2 > 0 ? r2.y : -r2.x;
+                        const float thr = fmaf(a.ad_rhi, a.ad_c32 * (r2.z + r3.z), a.ad_e0);
+#pragma unroll
+                        for (int j1 = 0; j1 < NB; ++j1)
+                            if (!(((base32[j1] + lo2) - r3.y) <= thr && ((base32[j1] + hi2) - r3.x) >= -thr))
+                                j1_near &= ~(1u << j1);
+                        if (!j1_near) continue;
+                    }
+                }
                 // Adaptive σ: the width of a pair (λ'', λ''') does not depend on j', so the 36 widths
                 // of this q'' are formed once, kept in this thread's column of s_g, and tested below
                 // against every j' (branch-free masks as for a fixed σ, rare exact decisions out of line).
@@ -366,13 +506,12 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
 #pragma unroll
                         for (int j2 = 0; j2 < NB; ++j2)
                             s_g[(j3 * NB + j2) * kTileQ + threadIdx.x] =
-                                a.ad_c32 * vel_diff_norm32(t.vpT32[j2 * N + q2], t.vpTlo[j2 * N + q2], h3, l3);
+                                a.ad_c32 * vel_diff_norm32_approx(t.vpT32[j2 * N + q2], t.vpTlo[j2 * N + q2], h3, l3);
                     }
                 }
                 // Adaptive ++, --: most (q'', j') have no pair near its window at all.  The necessary
                 // condition min over (j'', j''') of |Δ32| - (r_hi 2σ32 + e0) <= 0 is evaluated for all
                 // j' at once, so each width is read and scaled once per q'' instead of once per j'.
-                unsigned j1_near = vm1;
                 if constexpr (ADA) {
                     if (ch != 3) {
                         float mn[NB];
@@ -470,17 +609,163 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                                        ((unsigned long long)j1 << 40) | tri_bits | sure;
                 }
             }
-            int total;
-            const int off = block_exclusive_scan(n_ent, s_scan, &total);
+            off = block_exclusive_scan(n_ent, s_scan, &total);
             for (int k = 0; k < n_ent; ++k) sQ[off + k] = ent[k];
             __syncthreads();
+            }
 
-            // Compacted: the block's entries are dealt out to the threads in order.  The ablation
-            // instantiation (NOCOMP, fc4_set_ablation) instead has each thread evaluate the entries
-            // its own window found, as an uncompacted GPU-only loop would, so warps diverge on
-            // their counts.
-            const int it_end = NOCOMP ? off + n_ent : total;
-            for (int it = NOCOMP ? off : (int)threadIdx.x; it < it_end; it += NOCOMP ? 1 : kTileQ) {
+            // Compacted: the block's entries are dealt out to the threads in order.
+            // FP64: 32 to a warp at a time.  A lane forms its entry's X; the warp then takes the items
+            // (q'', j', j''') of its 32 entries one per lane (X by shuffles from the entry's lane) and the
+            // processes of 32 items one per lane (Y by shuffles), since entries carry 1-6 items and items
+            // 1-6 processes, and an idle lane costs the FP64 pipe as much as a busy one.  The weights
+            // return through shared memory to the lane that owns the entry, which adds them in the
+            // entry's order (4 q points of 8^3: 61.5 -> 52 ms for the three channels).
+            // FP32: each thread walks its entry's items and processes.  Redistributed as above it was
+            // slower (+- of 8^3 314 -> 414 ms; processes only, 16^3: 102 -> 132 ms): shuffles and scans
+            // lengthen the chain of each warp, and 3-4 warps per scheduler do not cover it.
+            // The ablation instantiation (NOCOMP, fc4_set_ablation) has each thread evaluate the entries
+            // its own window found, as an uncompacted GPU-only loop would.
+            if constexpr (WARP) {
+              const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+              unsigned char *wItem = s_item + wid * 32 * NB;
+              unsigned char *wProc = s_proc + wid * 32 * NB;
+              R *wVal = s_val + wid * 32 * NB * NV;
+              for (int ib = wid * 32; ib < total; ib += kTileQ) {
+                unsigned long long e = 0;
+                int iq2 = 0, iq3 = 0;
+                C X[NA][NA][9];
+                if (ib + lane < total) {
+                    ++acc_ent;
+                    e = sQ[ib + lane];
+                    const int ixe = qb + (int)(e >> 48), j1 = (int)((e >> 40) & 0xff);
+                    iq2 = cb + (pm_list ? (int)s_tri[ixe] : ixe);
+                    const int4 cc2 = t.qc[iq2];
+                    iq3 = q_index_near(b0 + s2 * cc2.x, b1 + s2 * cc2.y, b2 + s2 * cc2.z,
+                                       t.mesh[0], t.mesh[1], t.mesh[2]);
+                    const C *Prow = P4 + (size_t)iq2 * nk;
+                    const C *Wj = sW + j1 * nk * 9;
+#pragma unroll
+                    for (int c = 0; c < NA; ++c)
+#pragma unroll
+                        for (int d = 0; d < NA; ++d) {
+#pragma unroll
+                            for (int k = 0; k < 9; ++k) X[c][d][k] = czero<C>();
+                            const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
+                            for (int r = r0; r < r1; ++r) {
+                                const C ph = cconj_if(Prow[r], s2 < 0);
+                                const C *Wr = Wj + 9 * r;
+#pragma unroll
+                                for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
+                            }
+                        }
+                }
+                unsigned rows = 0;
+#pragma unroll
+                for (int j3 = 0; j3 < NB; ++j3)
+                    if ((e >> (NB * j3)) & ((1u << NB) - 1u)) rows |= 1u << j3;
+                const int n_it = __popc(rows);
+                const int io = warp_exclusive_scan(n_it), n_items = __shfl_sync(kFull, io + n_it, 31);
+                {
+                    int o = io;
+                    for (unsigned r = rows; r; r &= r - 1) wItem[o++] = (unsigned char)((lane << 3) | (__ffs(r) - 1));
+                }
+                __syncwarp();
+                for (int ip = 0; ip < n_items; ip += 32) {
+                    const bool act = ip + lane < n_items;
+                    const int code = act ? wItem[ip + lane] : 0;
+                    const int src = code >> 3, j3 = code & 7;
+                    const unsigned long long es = __shfl_sync(kFull, e, src);
+                    const int sq2 = __shfl_sync(kFull, iq2, src), sq3 = __shfl_sync(kFull, iq3, src);
+                    const unsigned m = act ? (unsigned)(es >> (NB * j3)) & ((1u << NB) - 1u) : 0u;
+                    if (act) ++acc_items;
+                    C Y[NA][3];
+#pragma unroll
+                    for (int c = 0; c < NA; ++c)
+#pragma unroll
+                        for (int g = 0; g < 3; ++g) Y[c][g] = czero<C>();
+#pragma unroll
+                    for (int d = 0; d < NA; ++d) {
+                        C e3[3];
+#pragma unroll
+                        for (int dl = 0; dl < 3; ++dl) e3[dl] = cconj(ev[(sq3 * NB + 3 * d + dl) * NB + j3]);
+#pragma unroll
+                        for (int c = 0; c < NA; ++c)
+#pragma unroll
+                            for (int g = 0; g < 3; ++g)
+#pragma unroll
+                                for (int dl = 0; dl < 3; ++dl)
+                                    Y[c][g] = cfma(cshfl(X[c][d][3 * g + dl], src), e3[dl], Y[c][g]);
+                    }
+                    const int np = __popc(m);
+                    const int po = warp_exclusive_scan(np), n_proc = __shfl_sync(kFull, po + np, 31);
+                    {
+                        int o = po;
+                        for (unsigned mm = m; mm; mm &= mm - 1) wProc[o++] = (unsigned char)((lane << 3) | (__ffs(mm) - 1));
+                    }
+                    // processes of this lane's own entry in the pass
+                    const int lo = max(io, ip) - ip, hi = min(io + n_it, ip + 32) - ip;
+                    const int from = __shfl_sync(kFull, po, lo & 31);
+                    const int end = __shfl_sync(kFull, po + np, (hi - 1) & 31), to = lo < hi ? end : from;
+                    // j', j''' and the domain code of the item
+                    const int jj = (int)((es >> 40) & 0xff) | (j3 << 8) | ((int)((es >> 36) & 3u) << 16);
+                    __syncwarp();
+                    for (int pp = 0; pp < n_proc; pp += 32) {
+                        const bool pact = pp + lane < n_proc;
+                        const int pc = pact ? wProc[pp + lane] : 0;
+                        const int il = pc >> 3, j2 = pc & 7;
+                        const int pjj = __shfl_sync(kFull, jj, il);
+                        const int j1 = pjj & 0xff, pj3 = (pjj >> 8) & 0xff, tri = pjj >> 16;
+                        const int m1 = q1 * NB + j1;
+                        const int m2 = __shfl_sync(kFull, sq2, il) * NB + j2, m3 = __shfl_sync(kFull, sq3, il) * NB + pj3;
+                        const C *e2p = ev + (size_t)(m2 - j2) * NB + j2;
+                        C V = czero<C>();
+#pragma unroll
+                        for (int c = 0; c < NA; ++c)
+#pragma unroll
+                            for (int g = 0; g < 3; ++g)
+                                V = cfma(cconj_if(e2p[(3 * c + g) * NB], s2 < 0), cshfl(Y[c][g], il), V);
+                        const double d = delta_exact(ch, w0, t.om[m1], t.om[m2], t.om[m3]);
+                        double g;
+                        if constexpr (ADA) g = gauss_adaptive(t, a, d, m2, m3);
+                        else g = exp(-(d * d) * a.inv_sigma2) * a.gnorm;
+                        R w = sym4<double>(ch) * occupation_factor<double>(ch, occ[m1], occ[m2], occ[m3]) *
+                              g * invw[m0] * invw[m1] * invw[m2] * invw[m3];
+                        const int wt = tri_weight(tri, j1, j2, pj3);
+                        w *= (R)wt;
+                        if (pact) {
+                            R *v = wVal + (pp + lane) * NV;
+                            v[0] = w;
+                            v[1] = V.x * V.x + V.y * V.y;
+                            acc_n += wt;
+                            acc_ev += 1;
+                            if constexpr (BTE) {
+                                const R *F = Sel<R>::bteF(a);
+                                const R o1 = (R)(ch == 4 ? 1 : -1) * Sel<R>::om(t)[m1];
+                                const R o2 = (R)(ch == 2 ? -1 : 1) * Sel<R>::om(t)[m2];
+                                const R o3 = Sel<R>::om(t)[m3];
+#pragma unroll
+                                for (int x = 0; x < 3; ++x)
+                                    v[2 + x] = (o1 * F[3 * m1 + x] + o2 * F[3 * m2 + x]) + o3 * F[3 * m3 + x];
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    for (int k = from; k < to; ++k) {
+                        const R *v = wVal + k * NV;
+                        acc_wp.add(v[0]);
+                        acc_g.add(v[0] * v[1]);
+                        if constexpr (BTE) {
+                            const R g = v[0] * v[1];
+#pragma unroll
+                            for (int x = 0; x < 3; ++x) acc_d[x].add(g * v[2 + x]);
+                        }
+                    }
+                    __syncwarp();                                // lists reused by the next pass
+                }
+              }
+            } else {
+            for (int it = NOCOMP ? off : (int)threadIdx.x; it < (NOCOMP ? off + n_ent : total); it += NOCOMP ? 1 : kTileQ) {
                 ++acc_ent;
                 const unsigned long long e = sQ[it];
                 const int ixe = qb + (int)(e >> 48), j1 = (int)((e >> 40) & 0xff);
@@ -492,13 +777,10 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                 const int m1 = q1 * NB + j1;
                 // per-entry constants of the mixed weight: TwoSum of ω + s1 ω', the sum of their lo
                 // parts, n', 1/(ω ω')
-                float ex1 = 0.0f, ee1 = 0.0f, el01 = 0.0f, iw01 = 0.0f, n1f = 0.0f;
-                if constexpr (sizeof(R) == 4) {
-                    ex1 = two_sum(t.om32[m0], (float)s1 * t.om32[m1], ee1);
-                    el01 = t.om32lo[m0] + (float)s1 * t.om32lo[m1];
-                    iw01 = invw[m0] * invw[m1];
-                    n1f = occ[m1];
-                }
+                const float4 k0 = t.mode4[m0], k1 = t.mode4[m1];
+                float ee1;
+                const float ex1 = two_sum(k0.x, (float)s1 * k1.x, ee1);
+                const float el01 = k0.y + (float)s1 * k1.y, iw01 = k0.w * k1.w, n1f = k1.z;
                 const C *Prow = P4 + (size_t)iq2 * nk;
                 const C *Wj = sW + j1 * nk * 9;
                 C X[NA][NA][9];
@@ -539,12 +821,7 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                                 for (int dl = 0; dl < 3; ++dl) Y[c][g] = cfma(X[c][d][3 * g + dl], e3[dl], Y[c][g]);
                     }
                     const int m3 = iq3 * NB + j3;
-                    const R n3 = occ[m3], iw3 = invw[m3];
-                    float h3 = 0.0f, l3 = 0.0f;
-                    if constexpr (sizeof(R) == 4) {
-                        h3 = t.om32[m3];
-                        l3 = t.om32lo[m3];
-                    }
+                    const float4 k3 = t.mode4[m3];
                     while (m) {
                         const int j2 = __ffs(m) - 1;
                         m &= m - 1;
@@ -555,29 +832,20 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
 #pragma unroll
                             for (int g = 0; g < 3; ++g)
                                 V = cfma(cconj_if(ev[(iq2 * NB + 3 * c + g) * NB + j2], s2 < 0), Y[c][g], V);
-                        R w;
-                        if constexpr (sizeof(R) == 8) {
-                            const double d = delta_exact(ch, w0, t.om[m1], t.om[m2], t.om[m3]);
-                            double g;
-                            if constexpr (ADA) g = gauss_adaptive(t, a, d, m2, m3);
-                            else g = exp(-(d * d) * a.inv_sigma2) * a.gnorm;
-                            w = sym4<double>(ch) * occupation_factor<double>(ch, occ[m1], occ[m2], n3) *
-                                g * invw[m0] * invw[m1] * invw[m2] * iw3;
-                        } else {
-                            // Δ from the entry's TwoSum (ex1, ee1) and the hi/lo splits of the last two ω
-                            float e2s, e3s;
-                            const float x2 = two_sum(ex1, (float)s2 * t.om32[m2], e2s);
-                            const float x3 = two_sum(x2, -h3, e3s);
-                            const float lo = (el01 + (float)s2 * t.om32lo[m2]) - l3;
-                            const float df = x3 + ((ee1 + e2s) + (e3s + lo));
-                            float gs;
-                            if constexpr (ADA) gs = gauss_adaptive32(t, a, df, m2, m3);
-                            else gs = __expf(-(df * df) * a.inv_sigma2_32) * a.gnorm32;
-                            w = sym4<float>(ch) * occupation_factor<float>(ch, n1f, occ[m2], n3) * gs *
-                                iw01 * (invw[m2] * iw3);
-                        }
+                        // Δ from the entry's TwoSum (ex1, ee1) and the hi/lo splits of the last two ω
+                        float e2s, e3s;
+                        const float4 k2 = t.mode4[m2];
+                        const float x2 = two_sum(ex1, (float)s2 * k2.x, e2s);
+                        const float x3 = two_sum(x2, -k3.x, e3s);
+                        const float lo = (el01 + (float)s2 * k2.y) - k3.y;
+                        const float df = x3 + ((ee1 + e2s) + (e3s + lo));
+                        float gs;
+                        if constexpr (ADA) gs = gauss_adaptive32(t, a, df, m2, m3);
+                        else gs = __expf(-(df * df) * a.inv_sigma2_32) * a.gnorm32;
+                        R w = sym4<float>(ch) * occupation_factor<float>(ch, n1f, k2.z, k3.z) * gs *
+                            iw01 * (k2.w * k3.w);
                         // weight of the representative: 2 for a swapped pair, 1 on the diagonal
-                        const int wt = tri == 0 ? 1 : tri == 1 ? 2 : tri == 2 ? (j2 < j3 ? 2 : 1) : (j2 > j1 ? 2 : 1);
+                        const int wt = tri_weight(tri, j1, j2, j3);
                         w *= (R)wt;
                         acc_wp.add(w);
                         acc_g.add(w * (V.x * V.x + V.y * V.y));
@@ -595,6 +863,7 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                         }
                     }
                 }
+            }
             }
             __syncthreads();                                     // sQ reused by the next round
           }
