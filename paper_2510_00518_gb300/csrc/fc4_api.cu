@@ -60,6 +60,8 @@ struct fc4_ctx {
     std::map<void *, size_t> alloc_bytes;  // size of each allocation (entries of freed ones are stale)
     std::vector<int> perm4;                 // device cluster slot -> input cluster index
     std::vector<int> swap12, swap23;        // input cluster -> the cluster with legs 1,2 (2,3) swapped
+    std::vector<int> swap12_3;              // third order: the cluster with legs 1, 2 swapped (-1: none)
+    bool sym12_3 = false;                   // Φ3 invariant under that swap (3ph- domain)
     bool sym12 = false, sym23 = false;      // Φ4 invariant under those swaps (triangular domains)
     std::vector<double> om_host;            // current ω (for the prefilter bound)
     double vmax = 0.0;                      // max |v| over modes (adaptive prefilter bound)
@@ -256,6 +258,23 @@ void check_sym4(fc4_ctx *c, const double *phi) {
     c->sym23 = ok(c->swap23, false);
 }
 
+// The same for Φ3 and legs 1, 2 (the domain of 3ph-).
+void check_sym3(fc4_ctx *c, const double *phi) {
+    double mx = 0.0;
+    for (size_t k = 0; k < 27 * (size_t)c->nc3; ++k) mx = std::max(mx, std::fabs(phi[k]));
+    c->sym12_3 = true;
+    for (int i = 0; i < c->nc3 && c->sym12_3; ++i) {
+        const int j = c->swap12_3[i];
+        if (j < 0 || c->swap12_3[j] != i) { c->sym12_3 = false; break; }       // (a repeated cluster: no pairing)
+        for (int al = 0; al < 3; ++al)
+            for (int x = 0; x < 3; ++x)
+                for (int y = 0; y < 3; ++y)
+                    if (!(std::fabs(phi[27 * (size_t)i + (al * 3 + x) * 3 + y] - phi[27 * (size_t)j + (al * 3 + y) * 3 + x]) <=
+                          1e-12 * mx))
+                        c->sym12_3 = false;
+    }
+}
+
 // Prefilter thresholds: |Δ32 - Δ64| <= 13 u ω_max (u = 2^-24; three roundings of the inputs'
 // partial sums plus four input roundings); margin 32 u ω_max, doubled to cover the rounding of
 // the thresholds themselves.
@@ -294,7 +313,7 @@ void set_window(const fc4_ctx *c, fc4::RateArgs &a, bool adaptive, double sigma_
     a.spin_limit = c->timeout_cycles;
     a.err = c->dev_err;
     a.n_kernels = const_cast<long long *>(&c->n_launches);
-    a.tri = (c->sym23 ? 1 : 0) | (c->sym12 && !adaptive ? 2 : 0);
+    a.tri = (c->sym23 ? 1 : 0) | (c->sym12 && !adaptive ? 2 : 0) | (c->sym12_3 ? 4 : 0);
     a.no_compact = c->no_compact;
     a.sample_all = c->sample_all;
     a.sample_threshold = c->sample_threshold;
@@ -490,6 +509,22 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         t.c3_r12 = d_r12;
         t.c3_ism = d_im;
         t.phi3 = c->phi3;
+        {   // leg-swap partner of every cluster
+            using CK = std::array<int, 9>;
+            std::map<CK, int> id;
+            auto key = [&](int i, int l1, int l2) {
+                const int *a = phi3->atoms + 3 * i, *R = phi3->cells + 6 * i;
+                return CK{a[0], a[1 + l1], a[1 + l2], R[3 * l1], R[3 * l1 + 1], R[3 * l1 + 2], R[3 * l2], R[3 * l2 + 1],
+                          R[3 * l2 + 2]};
+            };
+            for (int i = 0; i < c->nc3; ++i) id.emplace(key(i, 0, 1), i);
+            c->swap12_3.assign(c->nc3, -1);
+            for (int i = 0; i < c->nc3; ++i) {
+                auto f = id.find(key(i, 1, 0));
+                if (f != id.end()) c->swap12_3[i] = f->second;
+            }
+            if (c->nc3) check_sym3(c, phi3->phi);
+        }
         // key = (leg-1 atom, leg-2 atom, R1 - R2), as the 4ph keys below
         using Key = std::tuple<int, int, int, int>;
         std::map<Key, std::vector<int>> by_key;
@@ -915,9 +950,17 @@ fc4_status rates_call(fc4_ctx *c, double T_K, int sigma_adaptive, double sigma_v
             // a channel without clusters launches nothing: its a.n_part[ch] stays 0, so the
             // reduction reads no partials and writes Γ = WP = 0 and count 0 for it
             if (ch < 2 ? c->nc3 == 0 : c->nc4 == 0) continue;
-            if (ch < 2) {
+            if (ch < 2) {                   // both 3ph channels in one launch, unless each is timed
+                const int both = channel_mask & 3;
+                if (!c->timing && both == 3 && ch == 1) continue;
                 Timed tm(c, ch, s);
-                FC4_CUDA(c, fc4::launch_rates3(c->t, a, ch, fp64, s));
+                FC4_CUDA(c, fc4::launch_rates3(c->t, a, c->timing ? 1 << ch : both, s));
+                continue;
+            }
+            if (!per_mode && !bte_F && !c->timing) {       // general kernel: its channels in one launch
+                const int rest = channel_mask & 0b11100;
+                if ((rest & ((1 << ch) - 1)) == 0)
+                    FC4_CUDA(c, fc4::launch_rates4_general(c->t, a, rest, fp64, c->block_threads, s));
                 continue;
             }
             const int s1 = ch == 4 ? -1 : 1;
@@ -1169,6 +1212,7 @@ fc4_status fc4_update_anharmonic(fc4_ctx *c, const double *phi3, const double *p
     if (!c) return fail(nullptr, FC4_ERR_INVALID, "ctx is NULL");
     FC4_CUDA(c, cudaDeviceSynchronize());
     if (phi4) c->w_s1 = 0;
+    if (phi3 && c->nc3) check_sym3(c, phi3);
     if (phi3 && c->nc3)
         FC4_CUDA(c, cudaMemcpy(c->phi3, phi3, 27 * (size_t)c->nc3 * sizeof(double), cudaMemcpyHostToDevice));
     if (phi4 && c->nc4) {
@@ -1420,9 +1464,11 @@ extern "C" fc4_status fc4_rates_static(fc4_ctx *c, double T_K, double sigma_valu
         // A channel without clusters launches nothing: its a.n_part[ch] stays 0, so the reduction
         // reads no partials and writes Γ = WP = 0 and count 0 for it.
         if (ch < 2 ? c->nc3 == 0 : c->nc4 == 0) continue;
-        if (ch < 2) FC4_CUDA(c, fc4::launch_rates3(c->t, a, ch, fp64, s));
-        else FC4_CUDA(c, fc4::launch_rates4(c->t, a, ch, fp64, c->block_threads, s));
+        if (ch < 2) {
+            if (ch == 0 || !(channel_mask & 1)) FC4_CUDA(c, fc4::launch_rates3(c->t, a, channel_mask & 3, s));
+        }
     }
+    if (c->nc4) FC4_CUDA(c, fc4::launch_rates4_general(c->t, a, channel_mask & 0b11100, fp64, c->block_threads, s));
     FC4_CUDA(c, fc4::launch_reduce(c->t, a, channel_mask, unit_c3(), unit_c4(), gamma_out, wp_out,
                                    counts_out, nullptr, s));
     return FC4_OK;
@@ -1611,8 +1657,7 @@ extern "C" fc4_status fc4_batch_rates(fc4_batch *b, double T_K, double sigma_val
     for (int i = 0; i < n; ++i) {
         fc4_ctx *c = b->ctx[i];
         if (!nms[i] || !c->nc3) continue;
-        for (int ch = 0; ch < 2; ++ch)
-            if ((channel_mask >> ch) & 1) FC4_BCUDA(b, fc4::launch_rates3(c->t, args[i], ch, 0, s));
+        FC4_BCUDA(b, fc4::launch_rates3(c->t, args[i], channel_mask & 3, s));
     }
     // work list: contexts grouped by cell size (largest first), meshes from the largest down
     std::vector<int> order(n);

@@ -120,14 +120,17 @@ struct RateArgs {
     const float *bte_F32;
     double *part_d;
     int tri;                     // triangular 4ph domain allowed: bit 0 +- (Φ4 symmetric in legs 2, 3),
-                                 // bit 1 ++ and -- (legs 1, 2; fixed σ only)
+                                 // bit 1 ++ and -- (legs 1, 2; fixed σ only); bit 2 3ph- (Φ3, legs 1, 2)
 };
 
 // launchers (stream-ordered; return cudaGetLastError())
 // each rate launcher records in a.n_part[ch] how many partial slots per mode it writes
-cudaError_t launch_rates3(const Tables &t, RateArgs &a, int ch, int fp64, cudaStream_t s);
+// the three-phonon channels of mask (bit 0 3ph+, bit 1 3ph-) in one launch
+cudaError_t launch_rates3(const Tables &t, RateArgs &a, int mask, cudaStream_t s);
 cudaError_t launch_rates4(const Tables &t, RateArgs &a, int ch, int fp64, int threads,
                           cudaStream_t s);
+// the general kernel over the 4ph channels of mask (bits 2..4) in one launch
+cudaError_t launch_rates4_general(const Tables &t, RateArgs &a, int mask, int fp64, int threads, cudaStream_t s);
 // tensor-core +- path (k_rates4_tc.cu): availability for a context, and its launch over a mode chunk
 bool tc_supported(const Tables &t);
 cudaError_t launch_rates4_tc(const Tables &t, const RateArgs &a, int ch, int mode0, int nm, const float2 *w,

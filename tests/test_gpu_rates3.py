@@ -1,5 +1,6 @@
-"""Three-phonon kernel at the edges of its spans of 128 partner points and of its queue rounds of
-128 processes, and for every branch grouping of its window, against the FP64 oracle.
+"""Three-phonon kernels at the edges of their spans of partner points (512 for cells of up to two
+atoms) and of their rounds of 128 points or processes, for every branch grouping of the window and with
+a Φ3 that has no leg-exchange symmetry, against the FP64 oracle.
 
 Counts are exact.  Γ and WP are sums whose terms have both signs once the window is wide (at (1, 1, 127)
 with σ = 4 THz a soft mode's terms cancel 6800-fold), so the FP64 bar of 1e-10 applies to the sum of
@@ -68,7 +69,7 @@ def _check(system, mesh, q, sigma, adaptive):
     e.close()
 
 
-@pytest.mark.parametrize("mesh", [(1, 1, 1), (1, 1, 127), (8, 4, 4), (3, 43, 1), (16, 16, 1), (1, 1, 256)])
+@pytest.mark.parametrize("mesh", [(1, 1, 1), (1, 1, 127), (8, 4, 4), (3, 43, 1), (16, 16, 1), (1, 1, 256), (8, 8, 8), (8, 8, 9)])
 @pytest.mark.parametrize("sigma,adaptive", [(0.1, False), (4.0, False), (1.0, True)])
 def test_span_and_queue_edges(mesh, sigma, adaptive):
     n = int(np.prod(mesh))
@@ -91,3 +92,23 @@ def test_branch_groupings(atoms):
         c = supercell_crystal(base, atoms // 2, np.linspace(12.0, 90.0, atoms))
         p2, p3, p4 = morse_ifcs(c, seed=1)
     _check((c, p2, p3, p4), (5, 3, 9), [0, 77][:2 if atoms < 6 else 1], 0.5 if atoms > 2 else 2.0, False)
+
+
+def test_broken_leg_exchange_takes_the_rectangle():
+    """3ph- evaluates one process of a swapped pair only where Φ3 is symmetric in legs 1 and 2."""
+    c, p2, p3, p4 = morse_system(seed=3)
+    e = make_engine((c, p2, p3, p4), (4, 4, 4))
+    e.rates(300.0, 0.3, 3)
+    st = e.stats()
+    assert st["evaluated"][0] == st["kept"][0] and st["evaluated"][1] < st["kept"][1]
+    e.close()
+    p3.phi[5, 7] += 0.3 * np.abs(p3.phi).max()
+    _check((c, p2, p3, p4), (4, 4, 4), [0, 9], 0.3, False)
+    e = make_engine((c, p2, p3, p4), (4, 4, 4))
+    e.rates(300.0, 0.3, 3)
+    st = e.stats()
+    assert np.array_equal(st["evaluated"][:2], st["kept"][:2])
+    e.update_anharmonic(phi3=morse_system(seed=3)[2].phi)
+    e.rates(300.0, 0.3, 3)
+    assert e.stats()["evaluated"][1] < st["kept"][1]
+    e.close()
