@@ -24,7 +24,7 @@ constexpr float kInvSqrtPiF = 0.56418958354775628695f;
 
 // 2σ of the pair (ma, mb) in FP32 (prefilter)
 __device__ __forceinline__ float two_sigma32(const Tables &t, const RateArgs &a, int ma, int mb) {
-    return a.ad_c32 * vel_diff_norm32(t.vp32[ma], t.vp32lo[ma], t.vp32[mb], t.vp32lo[mb]);
+    return a.ad_c32 * vel_diff_norm32_approx(t.vp32[ma], t.vp32lo[ma], t.vp32[mb], t.vp32lo[mb]);
 }
 
 // exact FP64 σ of the pair (ma, mb)
@@ -86,7 +86,7 @@ static __device__ __noinline__ unsigned window_adaptive4_row(const Tables &t, co
         if (!((v2 >> j2) & 1u)) continue;
         const int m2 = q2 * NB + j2;
         const float ad = fabsf((base32 + (float)s2 * t.om32[m2]) - w3);
-        const float g32 = a.ad_c32 * vel_diff_norm32(t.vp32[m2], t.vp32lo[m2], h3, l3);
+        const float g32 = a.ad_c32 * vel_diff_norm32_approx(t.vp32[m2], t.vp32lo[m2], h3, l3);
         const int w = window_adaptive32(a, ad, g32);
         if (w == 2 || (w == 1 && window_exact_adaptive(t, a, ch, m0, m1, m2, m3, m2, m3))) keep |= 1u << j2;
     }

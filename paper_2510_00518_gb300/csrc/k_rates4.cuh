@@ -128,7 +128,12 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
     const unsigned v2 = t.vmask[q2], v3 = t.vmask[q3];
     const int q1 = m1 / NB, j1 = m1 - q1 * NB;
     const int tri = tri_code_sampled(a, ch, m0, q1, q2, q3, t.N);
-    if (tri < 0) {
+    // no pair of the point can reach the window: FP32 sums are monotonic, and no width exceeds the one of
+    // |P''| + |P'''|
+    const float4 r2 = t.wrange[q2], r3 = t.wrange[q3];
+    const float thr = ADA ? fmaf(a.ad_rhi, a.ad_c32 * (r2.z + r3.z), a.ad_e0) : a.hi32;
+    const bool out = (base32 + (s2 > 0 ? r2.x : -r2.y)) - r3.y > thr || (base32 + (s2 > 0 ? r2.y : -r2.x)) - r3.x < -thr;
+    if (tri < 0 || out) {
 #pragma unroll
         for (int j3 = 0; j3 < NB; ++j3) mask[j3] = 0u;
         return 0;
@@ -642,12 +647,12 @@ template <typename R, int NA> constexpr int general_blocks() { return sizeof(R) 
 
 template <typename R, int NA, bool ADA>
 __global__ void __launch_bounds__(128, general_blocks<R, NA>())
-rates4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int ch) {
-    rates4_unit<R, NA, ADA>(t, a, ch, blockIdx.x);
+rates4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int channels) {
+    rates4_unit<R, NA, ADA>(t, a, (channels >> (4 * blockIdx.y)) & 15, blockIdx.x);
 }
 
 template <typename R, int NA, bool ADA>
-cudaError_t launch4(const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s) {
+cudaError_t launch4(const Tables &t, const RateArgs &a, int channels, int threads, cudaStream_t s) {
     const size_t smem = GeneralSmem<R, NA>::bytes(t);
     cudaError_t e = cudaFuncSetAttribute(rates4_kernel<R, NA, ADA>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -655,7 +660,8 @@ cudaError_t launch4(const Tables &t, const RateArgs &a, int ch, int threads, cud
     const long long units = (long long)a.n_modes * t.N;
     if (units > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if (units == 0) return cudaSuccess;
-    rates4_kernel<R, NA, ADA><<<(unsigned)units, threads, smem, s>>>(t, a, ch);
+    const int n_ch = channels >> 8 ? 3 : channels >> 4 ? 2 : 1;
+    rates4_kernel<R, NA, ADA><<<dim3((unsigned)units, n_ch), threads, smem, s>>>(t, a, channels);
     e = cudaGetLastError();
     if (e == cudaSuccess && a.n_kernels) ++*a.n_kernels;
     return e;
@@ -675,16 +681,18 @@ size_t general_smem_atoms(int na, const Tables &t) {
 // Dispatch over the atom count NA..HI (instantiations split across translation units so that they
 // compile in parallel; ADA selects the adaptive-σ window and Gaussian at compile time so that the
 // fixed-σ kernels carry none of its registers).
+// channels: up to three channels, four bits each from the first down, run by one launch (their blocks
+// fill each other's last wave).
 template <typename R, bool ADA, int NA, int HI>
-cudaError_t launch4_atoms(int na, const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s) {
-    if (na == NA) return launch4<R, NA, ADA>(t, a, ch, threads, s);
-    if constexpr (NA < HI) return launch4_atoms<R, ADA, NA + 1, HI>(na, t, a, ch, threads, s);
+cudaError_t launch4_atoms(int na, const Tables &t, const RateArgs &a, int channels, int threads, cudaStream_t s) {
+    if (na == NA) return launch4<R, NA, ADA>(t, a, channels, threads, s);
+    if constexpr (NA < HI) return launch4_atoms<R, ADA, NA + 1, HI>(na, t, a, channels, threads, s);
     else return cudaErrorInvalidValue;
 }
 
 // general-kernel launchers, one per translation unit: precision x adaptive x atoms 1-4 / 5-8
 #define FC4_GENERAL_LAUNCHER(name) \
-    cudaError_t name(int na, const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s);
+    cudaError_t name(int na, const Tables &t, const RateArgs &a, int channels, int threads, cudaStream_t s);
 FC4_GENERAL_LAUNCHER(launch4_d_1_4)
 FC4_GENERAL_LAUNCHER(launch4_d_5_8)
 FC4_GENERAL_LAUNCHER(launch4_f_1_4)

@@ -4,8 +4,8 @@
 
 namespace fc4 {
 
-cudaError_t launch4_ad_d_5_8(int na, const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s) {
-    return launch4_atoms<double, true, 5, 8>(na, t, a, ch, threads, s);
+cudaError_t launch4_ad_d_5_8(int na, const Tables &t, const RateArgs &a, int channels, int threads, cudaStream_t s) {
+    return launch4_atoms<double, true, 5, 8>(na, t, a, channels, threads, s);
 }
 
 }  // namespace fc4

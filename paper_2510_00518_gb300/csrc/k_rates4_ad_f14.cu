@@ -4,8 +4,8 @@
 
 namespace fc4 {
 
-cudaError_t launch4_ad_f_1_4(int na, const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s) {
-    return launch4_atoms<float, true, 1, 4>(na, t, a, ch, threads, s);
+cudaError_t launch4_ad_f_1_4(int na, const Tables &t, const RateArgs &a, int channels, int threads, cudaStream_t s) {
+    return launch4_atoms<float, true, 1, 4>(na, t, a, channels, threads, s);
 }
 
 }  // namespace fc4

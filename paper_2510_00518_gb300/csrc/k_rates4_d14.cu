@@ -4,8 +4,8 @@
 
 namespace fc4 {
 
-cudaError_t launch4_d_1_4(int na, const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s) {
-    return launch4_atoms<double, false, 1, 4>(na, t, a, ch, threads, s);
+cudaError_t launch4_d_1_4(int na, const Tables &t, const RateArgs &a, int channels, int threads, cudaStream_t s) {
+    return launch4_atoms<double, false, 1, 4>(na, t, a, channels, threads, s);
 }
 
 // The tiled kernel (k_rates4_tile.cuh) serves cells of <= 2 atoms whose tile fits in shared
@@ -35,16 +35,28 @@ cudaError_t launch_rates4(const Tables &t, RateArgs &a, int ch, int fp64, int th
         if (ad) return fp64 ? launch4_tile_ad_d(na, t, a, ch, s) : launch4_tile_ad_f(na, t, a, ch, s);
         return fp64 ? launch4_tile_d(na, t, a, ch, s) : launch4_tile_f(na, t, a, ch, s);
     }
-    a.n_part[ch] = t.N;
+    return launch_rates4_general(t, a, 1 << ch, fp64, threads, s);
+}
+
+cudaError_t launch_rates4_general(const Tables &t, RateArgs &a, int mask, int fp64, int threads, cudaStream_t s) {
+    const int na = t.n_atoms;
+    const bool ad = a.adaptive != 0;
+    int channels = 0, n = 0;
+    for (int ch : {3, 2, 4})                    // the dense channel's blocks first
+        if ((mask >> ch) & 1) {
+            a.n_part[ch] = t.N;
+            channels |= ch << (4 * n++);
+        }
+    if (!n) return cudaSuccess;
     if (threads <= 0) threads = 128;
     if (threads % 32 || threads > 256) return cudaErrorInvalidValue;
     const bool lo = na <= 4;
     if (ad) {
-        if (fp64) return lo ? launch4_ad_d_1_4(na, t, a, ch, threads, s) : launch4_ad_d_5_8(na, t, a, ch, threads, s);
-        return lo ? launch4_ad_f_1_4(na, t, a, ch, threads, s) : launch4_ad_f_5_8(na, t, a, ch, threads, s);
+        if (fp64) return lo ? launch4_ad_d_1_4(na, t, a, channels, threads, s) : launch4_ad_d_5_8(na, t, a, channels, threads, s);
+        return lo ? launch4_ad_f_1_4(na, t, a, channels, threads, s) : launch4_ad_f_5_8(na, t, a, channels, threads, s);
     }
-    if (fp64) return lo ? launch4_d_1_4(na, t, a, ch, threads, s) : launch4_d_5_8(na, t, a, ch, threads, s);
-    return lo ? launch4_f_1_4(na, t, a, ch, threads, s) : launch4_f_5_8(na, t, a, ch, threads, s);
+    if (fp64) return lo ? launch4_d_1_4(na, t, a, channels, threads, s) : launch4_d_5_8(na, t, a, channels, threads, s);
+    return lo ? launch4_f_1_4(na, t, a, channels, threads, s) : launch4_f_5_8(na, t, a, channels, threads, s);
 }
 
 }  // namespace fc4

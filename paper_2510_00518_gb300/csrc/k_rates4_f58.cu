@@ -4,8 +4,8 @@
 
 namespace fc4 {
 
-cudaError_t launch4_f_5_8(int na, const Tables &t, const RateArgs &a, int ch, int threads, cudaStream_t s) {
-    return launch4_atoms<float, false, 5, 8>(na, t, a, ch, threads, s);
+cudaError_t launch4_f_5_8(int na, const Tables &t, const RateArgs &a, int channels, int threads, cudaStream_t s) {
+    return launch4_atoms<float, false, 5, 8>(na, t, a, channels, threads, s);
 }
 
 cudaError_t launch4_batch_f_5_8(int na, const int4 *items, int n_items, int *counter, size_t smem,
