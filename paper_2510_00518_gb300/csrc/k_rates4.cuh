@@ -439,10 +439,14 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                                     for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
                                 }
                             }
-#pragma unroll 1
-                        for (int j3 = 0; j3 < NB; ++j3) {
+                        unsigned rows = 0;                          // each lane goes through its own items
+#pragma unroll
+                        for (int j3 = 0; j3 < NB; ++j3)
+                            if ((unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u)) rows |= 1u << j3;
+                        while (rows) {
+                            const int j3 = __ffs(rows) - 1;
+                            rows &= rows - 1;
                             unsigned m = (unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u);
-                            if (!m) continue;
                             ++acc_items;
                             C Y[NA][3];
 #pragma unroll

@@ -207,8 +207,6 @@ rates4_tc_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
     const int row = tid & (kTcRows - 1), wg = tid >> 7;         // TMEM lane = row; warpgroup
     constexpr int nj = 2;                                       // partner branches per warpgroup: g, g + 3
     const float2 *ev = t.ev32;
-    const float *occ = t.occ32;
-    const float *invw = t.invw32;
     const long long spins = a.spin_limit > 0 ? a.spin_limit : 2000000000ll;   // ~1 s
     const uint32_t mbar = smem_u32(&s_mbar);
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
@@ -481,11 +479,10 @@ rates4_tc_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
                     if (!e) continue;
                     ++acc_ent;
                     const int m1 = q1 * NB + j1;
+                    const float4 k0 = t.mode4[m0], k1 = t.mode4[m1];
                     float ee1;
-                    const float ex1 = two_sum(t.om32[m0], (float)s1 * t.om32[m1], ee1);
-                    const float el01 = t.om32lo[m0] + (float)s1 * t.om32lo[m1];
-                    const float iw01 = invw[m0] * invw[m1];
-                    const float n1f = occ[m1];
+                    const float ex1 = two_sum(k0.x, (float)s1 * k1.x, ee1);
+                    const float el01 = k0.y + (float)s1 * k1.y, iw01 = k0.w * k1.w, n1f = k1.z;
                     float2 X[NA][NA][9];
 #pragma unroll
                     for (int c = 0; c < NA; ++c)
@@ -494,10 +491,14 @@ rates4_tc_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
 #pragma unroll
                             for (int k = 0; k < 9; ++k)
                                 X[c][d][k] = make_float2(xr[c * NA + d][2 * k] * xscale, xr[c * NA + d][2 * k + 1] * xscale);
-#pragma unroll 1
-                    for (int j3 = 0; j3 < NB; ++j3) {
+                    unsigned rows = 0;                           // each lane goes through its own items
+#pragma unroll
+                    for (int j3 = 0; j3 < NB; ++j3)
+                        if ((unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u)) rows |= 1u << j3;
+                    while (rows) {
+                        const int j3 = __ffs(rows) - 1;
+                        rows &= rows - 1;
                         unsigned m = (unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u);
-                        if (!m) continue;
                         ++acc_items;
                         float2 Y[NA][3];
 #pragma unroll
@@ -517,8 +518,7 @@ rates4_tc_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
                                     for (int dl = 0; dl < 3; ++dl) Y[c][g] = cfma(X[c][d][3 * g + dl], e3[dl], Y[c][g]);
                         }
                         const int m3 = iq3 * NB + j3;
-                        const float n3 = occ[m3], iw3 = invw[m3];
-                        const float h3 = t.om32[m3], l3 = t.om32lo[m3];
+                        const float4 k3 = t.mode4[m3];
                         while (m) {
                             const int j2 = __ffs(m) - 1;
                             m &= m - 1;
@@ -530,15 +530,16 @@ rates4_tc_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
                                 for (int g = 0; g < 3; ++g)
                                     V = cfma(cconj_if(ev[(iq2 * NB + 3 * c + g) * NB + j2], s2 < 0), Y[c][g], V);
                             float e2s, e3s;
-                            const float x2 = two_sum(ex1, (float)s2 * t.om32[m2], e2s);
-                            const float x3 = two_sum(x2, -h3, e3s);
-                            const float lo = (el01 + (float)s2 * t.om32lo[m2]) - l3;
+                            const float4 k2 = t.mode4[m2];
+                            const float x2 = two_sum(ex1, (float)s2 * k2.x, e2s);
+                            const float x3 = two_sum(x2, -k3.x, e3s);
+                            const float lo = (el01 + (float)s2 * k2.y) - k3.y;
                             const float df = x3 + ((ee1 + e2s) + (e3s + lo));
                             float gs;
                             if constexpr (ADA) gs = gauss_adaptive32(t, a, df, m2, m3);
                             else gs = __expf(-(df * df) * a.inv_sigma2_32) * a.gnorm32;
-                            const float w = sym4<float>(ch) * occupation_factor<float>(ch, n1f, occ[m2], n3) * gs *
-                                            iw01 * (invw[m2] * iw3);
+                            const float w = sym4<float>(ch) * occupation_factor<float>(ch, n1f, k2.z, k3.z) * gs *
+                                            iw01 * (k2.w * k3.w);
                             const int wt = tri_weight(tri, j1, j2, j3);
                             acc_wp.add(w * (float)wt);
                             acc_g.add((w * (float)wt) * (V.x * V.x + V.y * V.y));

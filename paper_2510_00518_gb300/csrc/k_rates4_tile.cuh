@@ -798,10 +798,16 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                             for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
                         }
                     }
-#pragma unroll 1
-                for (int j3 = 0; j3 < NB; ++j3) {
+                // each lane goes through its own items: the warp takes as many steps as the entry with the most
+                // items has, not one per j''' that any entry has
+                unsigned rows = 0;
+#pragma unroll
+                for (int j3 = 0; j3 < NB; ++j3)
+                    if ((unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u)) rows |= 1u << j3;
+                while (rows) {
+                    const int j3 = __ffs(rows) - 1;
+                    rows &= rows - 1;
                     unsigned m = (unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u);
-                    if (!m) continue;
                     ++acc_items;
                     C Y[NA][3];
 #pragma unroll
