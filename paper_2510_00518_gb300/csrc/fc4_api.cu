@@ -166,6 +166,31 @@ int4 phase_vec(const int R[3], const int mesh[3], int L) {
                      mod_i((long long)R[2] * (L / mesh[2]), L), 0);
 }
 
+// The FP64 order of the keys of each group and where its pairs begin (fc4_kernels.h, perm4); key_r holds
+// (group, dR) of the sorted keys.
+void pair_keys(const std::vector<std::array<int, 4>> &keys, int n_groups, std::vector<int> &perm, std::vector<int> &pairs) {
+    perm.clear();
+    pairs.assign(n_groups, 0);
+    size_t k = 0;
+    for (int g = 0; g < n_groups; ++g) {
+        std::map<std::array<int, 4>, int> id;
+        const size_t k0 = k;
+        for (; k < keys.size() && keys[k][0] == g; ++k) id[keys[k]] = (int)k;
+        std::vector<int> mirrored;
+        for (size_t i = k0; i < k; ++i) {
+            const std::array<int, 4> m{g, -keys[i][1], -keys[i][2], -keys[i][3]};
+            const auto f = id.find(m);
+            if (f == id.end() || f->second == (int)i) perm.push_back((int)i);
+            else if ((int)i < f->second) {
+                mirrored.push_back((int)i | 1 << 28);
+                mirrored.push_back(f->second | 2 << 28);
+            }
+        }
+        pairs[g] = (int)perm.size();
+        perm.insert(perm.end(), mirrored.begin(), mirrored.end());
+    }
+}
+
 fc4_status check_ifc(const fc4_ifc *f, int order, int n_atoms, bool required, const char *name) {
     if (!f) {
         if (required) return fail(nullptr, FC4_ERR_INVALID, std::string(name) + " is NULL");
@@ -534,8 +559,10 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         }
         std::vector<int> k_start(1, 0), k_idx, g_start((size_t)na * na + 1, 0);
         std::vector<int4> kr;
+        std::vector<std::array<int, 4>> kv3;
         for (const auto &kv : by_key) {
             const int d[3] = {std::get<1>(kv.first), std::get<2>(kv.first), std::get<3>(kv.first)};
+            kv3.push_back({std::get<0>(kv.first), d[0], d[1], d[2]});
             kr.push_back(phase_vec(d, mesh, L));
             k_idx.insert(k_idx.end(), kv.second.begin(), kv.second.end());
             k_start.push_back((int)k_idx.size());
@@ -551,6 +578,13 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         FC4_TRY(upload(c, &d_gs, g_start));
         FC4_TRY(upload(c, &d_kr, kr));
         FC4_TRY(dalloc(c, &d_P3, (size_t)N * kr.size()));
+        std::vector<int> perm, pairs;
+        pair_keys(kv3, na * na, perm, pairs);
+        int *d_perm, *d_pairs;
+        FC4_TRY(upload(c, &d_perm, perm));
+        FC4_TRY(upload(c, &d_pairs, pairs));
+        t.perm3 = d_perm;
+        t.pairs3 = d_pairs;
         t.k3_start = d_ks;
         t.k3_idx = d_ki;
         t.grp3_start = d_gs;
@@ -663,6 +697,16 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         FC4_TRY(upload(c, &d_ks, key_start));
         FC4_TRY(upload(c, &d_ko, key_order));
         t.key_order = d_ko;
+        std::vector<std::array<int, 4>> kv4;
+        for (int k = 0; k < nk; ++k)
+            kv4.push_back({std::get<0>(keys[k]), std::get<1>(keys[k]), std::get<2>(keys[k]), std::get<3>(keys[k])});
+        std::vector<int> perm, pairs;
+        pair_keys(kv4, na * na, perm, pairs);
+        int *d_perm, *d_pairs;
+        FC4_TRY(upload(c, &d_perm, perm));
+        FC4_TRY(upload(c, &d_pairs, pairs));
+        t.perm4 = d_perm;
+        t.pairs4 = d_pairs;
         FC4_TRY(upload(c, &d_kbs, kb_start));
         FC4_TRY(upload(c, &d_kbi, kb_idx));
         FC4_TRY(upload(c, &d_kr, kr));

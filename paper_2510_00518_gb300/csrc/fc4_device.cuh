@@ -46,6 +46,47 @@ template <typename C> __device__ __forceinline__ double cabs2(C a) {
     return (double)a.x * (double)a.x + (double)a.y * (double)a.y;
 }
 
+// FP64 key sums Σ_r P_r^s W_r.  The phases of the keys dR and -dR are conjugate, so with θ = q.dR
+//   P W_dR + P* W_-dR = cos θ A + sin θ B,  A = W_dR + W_-dR,  B = i (W_dR - W_-dR),
+// four real multiply-adds a component pair instead of eight; A and B take the places of the two W.
+constexpr int kKeyMask = (1 << 28) - 1;
+
+// entry p of the FP64 order from the values w[key * stride]
+template <typename C>
+__device__ __forceinline__ C paired_value(const int *perm, int p, const C *w, int stride) {
+    const int e = perm[p], r = e & kKeyMask;
+    C x = w[(size_t)r * stride];
+    if (e >> 28 == 1) {
+        const C y = w[(size_t)(perm[p + 1] & kKeyMask) * stride];
+        x.x += y.x;
+        x.y += y.y;
+    } else if (e >> 28 == 2) {
+        const C y = w[(size_t)(perm[p - 1] & kKeyMask) * stride];
+        x = cmake(x.y - y.y, y.x - x.x);                       // i (y - x)
+    }
+    return x;
+}
+
+// X[k] = Σ over the keys of one group: entries [p0, pp) singly, [pp, p1) in pairs; P: phases by key,
+// W [p][9] in the FP64 order, s the sign of the phase
+template <typename C, typename R>
+__device__ __forceinline__ void paired_sum(const int *perm, int p0, int pp, int p1, const C *P, const C *W, R s, C (&X)[9]) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) X[k] = czero<C>();
+    for (int p = p0; p < pp; ++p) {
+        C ph = P[perm[p] & kKeyMask];
+        ph.y *= s;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) X[k] = cfma(ph, W[9 * p + k], X[k]);
+    }
+    for (int p = pp; p < p1; p += 2) {
+        C ph = P[perm[p] & kKeyMask];
+        ph.y *= s;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) X[k] = crfma(ph.y, W[9 * p + 9 + k], crfma(ph.x, W[9 * p + k], X[k]));
+    }
+}
+
 // ------------------------------------------------------------------------------ mesh
 
 __device__ __forceinline__ int mod_pos(int x, int n) {

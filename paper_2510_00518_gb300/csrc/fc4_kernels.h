@@ -54,6 +54,7 @@ struct Tables {
     const int *k3_start;         // [n_keys3 + 1] range in k3_idx of each key
     const int *k3_idx;           // [nc3] clusters grouped by key, ascending within a key
     const int *grp3_start;       // [n_atoms * n_atoms + 1] key range of group b * n_atoms + c
+    const int *perm3, *pairs3;   // FP64 order of the keys (see perm4), [n_keys3] and [n_atoms * n_atoms]
     const double2 *P3;           // [N][n_keys3] exp(i q.(R1 - R2)) of each key
     // fourth order: clusters sorted by key; keys sorted by (leg-2 atom, leg-3 atom) group
     int nc4, n_keys;
@@ -65,6 +66,10 @@ struct Tables {
     const double *phi4;          // [nc4][81]
     const float *phi4_32;
     const int *key_start;        // [n_keys + 1] cluster range of each key
+    // FP64 order of the keys within each group: the keys without a mirror key (-dR), then the pairs
+    // (dR, -dR) side by side from pairs4[group] on; an entry is key | 1 << 28 (first of a pair) or
+    // key | 2 << 28 (second)
+    const int *perm4, *pairs4;
     const int *key_order;        // [n_keys] keys from the most clusters down (the W kernel's columns)
     const int *kb_start;         // [n_keys * n_atoms + 1] range in kb_idx of (key r, leg-1 atom b)
     const int *kb_idx;           // [nc4] clusters grouped by (r, b), ascending within a group

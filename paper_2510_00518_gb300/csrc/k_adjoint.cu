@@ -255,7 +255,7 @@ adj4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
 // phase_c K_r(c)b(c) to 27 numbers a cluster in registers, and expands them by e_λ(aα) into the mode's
 // gradient slice at the end.
 //
-// Bound: FP64.  Per entry 612 + 72 items complex multiply-adds, per (λ, q') 17000 for the fold (the
+// Bound: FP64.  Per entry 396 + 72 items complex multiply-adds (mirror keys paired), per (λ, q') 17000 for the fold (the
 // block-per-mode kernel above takes 1020 an item and 220000 a (λ, q')).  Where Φ4 has the leg-exchange
 // symmetry only one process of each swapped pair is evaluated (self-swapped ones with weight 1/2) and
 // sum_slices_kernel adds the gradient of the swapped legs.  κ and its gradient for all modes of a 4^3
@@ -286,9 +286,11 @@ adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
     const double gl = dLdG[(size_t)ch * a.n_modes + ms] * cst;
     const unsigned vm1 = t.vmask[q1];
     for (int k = threadIdx.x; k < NB * nk * 9; k += kAdjThreads) {
-        sW[k] = H[k];
-        H[k] = czero<C>();
+        const int j = k / (nk * 9), rem = k - j * (nk * 9);
+        sW[k] = paired_value(t.perm4, rem / 9, (const C *)H + j * (nk * 9) + rem % 9, 9);
     }
+    __syncthreads();                                             // the whole of W is read
+    for (int k = threadIdx.x; k < NB * nk * 9; k += kAdjThreads) H[k] = czero<C>();
     if ((q0 == 0 && j0 < 3) || gl == 0.0 || !vm1) return;
     const int4 c0 = t.qc[q0], c1 = t.qc[q1];
     const int b0 = c0.x + s1 * c1.x, b1 = c0.y + s1 * c1.y, b2 = c0.z + s1 * c1.z;
@@ -361,17 +363,9 @@ adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
 #pragma unroll
                 for (int c = 0; c < NA; ++c)
 #pragma unroll
-                    for (int d = 0; d < NA; ++d) {
-#pragma unroll
-                        for (int k = 0; k < 9; ++k) X[c][d][k] = czero<C>();
-                        const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
-                        for (int r = r0; r < r1; ++r) {
-                            const C ph = cconj_if(Prow[r], s2 < 0);
-                            const C *Wr = Wj + 9 * r;
-#pragma unroll
-                            for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
-                        }
-                    }
+                    for (int d = 0; d < NA; ++d)
+                        paired_sum(t.perm4, t.grp_start[c * NA + d], t.pairs4[c * NA + d], t.grp_start[c * NA + d + 1], Prow, Wj,
+                                   (double)s2, X[c][d]);
                 const C *e2row = t.ev + (size_t)iq2 * NB * NB, *e3row = t.ev + (size_t)iq3 * NB * NB;
                 const double w01 = (ch == 4 ? 1.0 / 6.0 : 0.5) * gl * t.invw[m0] * t.invw[m1];
                 const double w1 = t.om[m1], n1 = t.occ[m1];
@@ -426,24 +420,41 @@ adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
                 }
             }
             __syncthreads();
-            // H_r[j'][γδ] += Σ P_r^s2 Z[c_r γ, d_r δ] over this batch, j' by j', in queue order
+            // H_r[j'][γδ] += Σ P_r^s2 Z[c_r γ, d_r δ] over this batch, j' by j', in queue order; of a pair of
+            // mirror keys the first collects Σ cos θ Z and the second Σ s2 sin θ Z
             for (int k = threadIdx.x; k < nk * 9; k += kAdjThreads) {
-                const int r = k / 9, gd = k - 9 * r, g = gd / 3, dl = gd - 3 * g;
+                const int p = k / 9, gd = k - 9 * p, g = gd / 3, dl = gd - 3 * g;
+                const int e = t.perm4[p], kind = e >> 28, r = e & kKeyMask;
+                const int rp = kind == 2 ? t.perm4[p - 1] & kKeyMask : r;        // the key whose phase it takes
                 int grp = 0;
                 while (t.grp_start[grp + 1] <= r) ++grp;
                 const C *Z = sZ + ((3 * (grp / NA) + g) * NB + 3 * (grp % NA) + dl) * kAdjLd;
                 for (int i = 0; i < n;) {
                     const int j1 = s_j1[i];
-                    C h = H[(j1 * nk) * 9 + k];
-                    for (; i < n && s_j1[i] == j1; ++i) {
-                        const C ph = cconj_if(t.P4[(size_t)s_q2[i] * nk + r], s2 < 0);
-                        h = cfma(ph, Z[i], h);
+                    C h = H[(j1 * nk + r) * 9 + gd];
+                    if (kind == 0) {
+                        for (; i < n && s_j1[i] == j1; ++i)
+                            h = cfma(cconj_if(t.P4[(size_t)s_q2[i] * nk + rp], s2 < 0), Z[i], h);
+                    } else {
+                        for (; i < n && s_j1[i] == j1; ++i) {
+                            const C ph = t.P4[(size_t)s_q2[i] * nk + rp];
+                            h = crfma(kind == 1 ? ph.x : s2 * ph.y, Z[i], h);
+                        }
                     }
-                    H[(j1 * nk) * 9 + k] = h;
+                    H[(j1 * nk + r) * 9 + gd] = h;
                 }
             }
             __syncthreads();
         }
+    }
+    // pairs: H_dR = A + i B, H_-dR = A - i B
+    for (int k = threadIdx.x; k < NB * nk * 9; k += kAdjThreads) {
+        const int j = k / (nk * 9), rem = k - j * (nk * 9), p = rem / 9, gd = rem - 9 * p;
+        if (t.perm4[p] >> 28 != 1) continue;
+        C *x = H + (j * nk + (t.perm4[p] & kKeyMask)) * 9 + gd, *y = H + (j * nk + (t.perm4[p + 1] & kKeyMask)) * 9 + gd;
+        const C A = *x, B = *y;
+        *x = cmake(A.x - B.y, A.y + B.x);
+        *y = cmake(A.x + B.y, A.y - B.x);
     }
 }
 

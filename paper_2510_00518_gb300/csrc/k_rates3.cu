@@ -12,7 +12,8 @@
 //
 // Bound: the FP64 pipe (64 FP32 operations per FP64 one on this GPU); cluster by cluster a process took
 // 1274 complex multiply-adds.  Cells of up to two atoms (rates3_pair_kernel) list the points (λ, q') with a
-// kept process, form T[bβ][cγ] = Σ_r P_r G_r[βγ] once per point (306 for the diamond cell) and take the
+// kept process, form T[bβ][cγ] = Σ_r P_r G_r[βγ] once per point (198 for the diamond cell,
+// mirror keys paired) and take the
 // 2-3 processes of a point at 42 each, on full warps.  Larger cells (rates3_kernel) evaluate a process
 // per thread at 9 n_keys + 12 groups each (their T does not fit in registers).  3ph- is evaluated on half of
 // its pairs where Φ3 allows it, and both channels share a launch.  All modes of 12^3 (2 x 9.5e6
@@ -39,7 +40,8 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     using C = double2;
     const int N = t.N, nk = t.n_keys3;
     extern __shared__ __align__(16) unsigned char smem[];
-    C *sG = reinterpret_cast<C *>(smem);                        // [nk][9]
+    C *sG = reinterpret_cast<C *>(smem);                        // [nk][9], in the FP64 key order
+    C *sG0 = sG + nk * 9;                                       // [nk][9], by key
     __shared__ unsigned long long s_list[kSpan3Pair];           // points: q' - qlo, domain code, kept (j', j'')
     __shared__ unsigned short s_proc[kR3Threads * NB * NB];     // per warp: processes (lane, j', j'') of 32 points
     __shared__ C se0[NB];
@@ -59,7 +61,10 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     if (!(p.q0 == 0 && p.j0 < 3)) {
         for (int k = threadIdx.x; k < NB; k += kR3Threads) se0[k] = t.ev[(p.q0 * NB + k) * NB + p.j0];
         __syncthreads();
-        three_G(t, p, se0, sG);                // ordered before its use by the scans' barriers
+        three_G(t, p, se0, sG0);
+        __syncthreads();
+        for (int k = threadIdx.x; k < nk * 9; k += kR3Threads)     // ordered before its use by the scans' barriers
+            sG[k] = paired_value(t.perm3, k / 9, sG0 + k % 9, 9);
         int total = 0;
         for (int qb = qlo; qb < qhi; qb += kR3Threads) {
             const int q1 = qb + threadIdx.x;
@@ -128,17 +133,9 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
 #pragma unroll
                 for (int b = 0; b < NA; ++b)
 #pragma unroll
-                    for (int c = 0; c < NA; ++c) {
-#pragma unroll
-                        for (int k = 0; k < 9; ++k) T[b][c][k] = czero<C>();
-                        const int r0 = t.grp3_start[b * NA + c], r1 = t.grp3_start[b * NA + c + 1];
-                        for (int r = r0; r < r1; ++r) {
-                            const C ph = cconj_if(P[r], p.s < 0);
-                            const C *G = sG + 9 * r;
-#pragma unroll
-                            for (int k = 0; k < 9; ++k) T[b][c][k] = cfma(ph, G[k], T[b][c][k]);
-                        }
-                    }
+                    for (int c = 0; c < NA; ++c)
+                        paired_sum(t.perm3, t.grp3_start[b * NA + c], t.pairs3[b * NA + c], t.grp3_start[b * NA + c + 1], P, sG,
+                                   (double)p.s, T[b][c]);
             }
             const unsigned long long kept = e & ((1ull << (NB * NB)) - 1ull);
             const int np = __popcll(kept);
@@ -280,7 +277,7 @@ static cudaError_t launch3(const Tables &t, RateArgs &a, int mask, cudaStream_t 
     for (int ch = 0; ch < 2; ++ch)
         if ((mask >> ch) & 1) a.n_part[ch] = n_span;
     if (a.n_modes == 0 || !mask) return cudaSuccess;
-    const size_t smem = sizeof(double2) * (size_t)t.n_keys3 * 9 +
+    const size_t smem = sizeof(double2) * (size_t)t.n_keys3 * 9 * (NA <= 2 ? 2 : 1) +
                         (NA <= 2 ? 0 : sizeof(unsigned) * (size_t)kR3Threads * (jb3(NB) * NB + 1));
     if ((long long)a.n_modes * n_span > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     void (*kern)(Tables, RateArgs, int, int);

@@ -8,8 +8,8 @@
 // exact FP64 Δ), compacts the (q'', j', masks) entries with a block scan, and evaluates them:
 //   X[c,d][γδ] = Σ_{r in (c,d)} P_r^s2 W_r[γδ] once per entry, Y = X e*''' per j''' (36 MACs).
 // FP64 holds X too (2 blocks of 255 registers per SM): its pipe issues a warp operation every ~19
-// clocks and SM, so what counts is the 306 + 36 items complex multiply-adds of an entry, against 408
-// an item key by key; 4 q points of 8^3 went from 239 to 71.5 ms.
+// clocks and SM, so what counts is the 198 + 36 items complex multiply-adds of an entry (306 + 36 items
+// without the pairing of mirror keys), against 408 an item key by key.
 // The same window decision, weights and accumulation as the general kernel (k_rates4.cuh).
 #pragma once
 #include "k_rates4.cuh"
@@ -299,7 +299,14 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
         const float w0f = t.om32[m0];
         {                                                        // W of (λ, q') for every j'
             const C *src = wall + (size_t)unit * (NB * nk * 9);
-            for (int k = threadIdx.x; k < NB * nk * 9; k += kTileQ) sW[k] = src[k];
+            if constexpr (sizeof(R) == 8) {
+                for (int k = threadIdx.x; k < NB * nk * 9; k += kTileQ) {
+                    const int j = k / (nk * 9), rem = k - j * (nk * 9);
+                    sW[k] = paired_value(t.perm4, rem / 9, src + j * (nk * 9) + rem % 9, 9);
+                }
+            } else {
+                for (int k = threadIdx.x; k < NB * nk * 9; k += kTileQ) sW[k] = src[k];
+            }
         }
         float base32[NB];
 #pragma unroll
@@ -648,17 +655,9 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
 #pragma unroll
                     for (int c = 0; c < NA; ++c)
 #pragma unroll
-                        for (int d = 0; d < NA; ++d) {
-#pragma unroll
-                            for (int k = 0; k < 9; ++k) X[c][d][k] = czero<C>();
-                            const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
-                            for (int r = r0; r < r1; ++r) {
-                                const C ph = cconj_if(Prow[r], s2 < 0);
-                                const C *Wr = Wj + 9 * r;
-#pragma unroll
-                                for (int k = 0; k < 9; ++k) X[c][d][k] = cfma(ph, Wr[k], X[c][d][k]);
-                            }
-                        }
+                        for (int d = 0; d < NA; ++d)
+                            paired_sum(t.perm4, t.grp_start[c * NA + d], t.pairs4[c * NA + d], t.grp_start[c * NA + d + 1], Prow, Wj,
+                                       (R)s2, X[c][d]);
                 }
                 unsigned rows = 0;
 #pragma unroll
