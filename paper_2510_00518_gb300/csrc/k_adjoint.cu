@@ -370,10 +370,14 @@ adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
                 const double w01 = (ch == 4 ? 1.0 / 6.0 : 0.5) * gl * t.invw[m0] * t.invw[m1];
                 const double w1 = t.om[m1], n1 = t.occ[m1];
                 bool started = false;
-#pragma unroll 1
-                for (int j3 = 0; j3 < NB; ++j3) {
+                unsigned rows = 0;                               // each lane goes through its own items
+#pragma unroll
+                for (int j3 = 0; j3 < NB; ++j3)
+                    if ((unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u)) rows |= 1u << j3;
+                while (rows) {
+                    const int j3 = __ffs(rows) - 1;
+                    rows &= rows - 1;
                     unsigned m = (unsigned)(e >> (NB * j3)) & ((1u << NB) - 1u);
-                    if (!m) continue;
                     C Y[NB], yb[NB];
 #pragma unroll
                     for (int k = 0; k < NB; ++k) Y[k] = yb[k] = czero<C>();

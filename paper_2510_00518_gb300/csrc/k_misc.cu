@@ -284,20 +284,19 @@ cudaError_t launch_phase_tables(const Tables &t, int n_keys, const int4 *key_r, 
 struct int5 { int a, b, c, d, e; };
 
 // One warp per (channel, mode): lane l sums q' = l, l + 32, ... in order, then a fixed
-// butterfly; Γ = C / N^k * Σ, WP = Σ / N^k (k = 1 for 3ph, 2 for 4ph).
+// butterfly; Γ = (C / N^k) Σ, WP = (1 / N^k) Σ (k = 1 for 3ph, 2 for 4ph; c3, c4 and norm3, norm4).
 __global__ void reduce_kernel(int n_modes, int ld, int N, int5 n_part, int channel_mask, double c3, double c4,
-                              double scale4,
+                              double norm3, double norm4, double scale4,
                               const double *part_g, const double *part_wp, const long long *part_n,
                               const long long *part_items, const long long *part_ent, const long long *part_ev,
                               const long long *part_cev, double *gamma, double *wp, long long *counts,
                               unsigned long long *stats, const int *err) {
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (w >= 5 * n_modes) return;
     const int ch = w / n_modes, ms = w - ch * n_modes;
     double g = 0.0, p = 0.0;
     long long n = 0, it = 0, en = 0, ev = 0, cv = 0;
-    if ((channel_mask >> ch) & 1) {
+    if (w < 5 * n_modes && ((channel_mask >> ch) & 1)) {
         const size_t base = ((size_t)ch * n_modes + ms) * N;
         const int np = ch == 0 ? n_part.a : ch == 1 ? n_part.b : ch == 2 ? n_part.c : ch == 3 ? n_part.d : n_part.e;
         for (int q = lane; q < np; q += 32) {
@@ -320,15 +319,23 @@ __global__ void reduce_kernel(int n_modes, int ld, int N, int5 n_part, int chann
             cv += __shfl_xor_sync(kFull, cv, o);
         }
     }
-    if (lane == 0 && stats) {
-        atomicAdd(stats + 5 * ch, (unsigned long long)n);       // integer sums: order-independent
-        atomicAdd(stats + 5 * ch + 1, (unsigned long long)it);
-        atomicAdd(stats + 5 * ch + 2, (unsigned long long)en);
-        atomicAdd(stats + 5 * ch + 3, (unsigned long long)ev);
-        atomicAdd(stats + 5 * ch + 4, (unsigned long long)cv);
+    if (stats) {                                     // integer sums: order-independent
+        __shared__ unsigned long long s_stats[25];
+        if (threadIdx.x < 25) s_stats[threadIdx.x] = 0;
+        __syncthreads();
+        if (lane == 0 && w < 5 * n_modes) {
+            const long long v[5] = {n, it, en, ev, cv};
+#pragma unroll
+            for (int k = 0; k < 5; ++k)
+                if (v[k]) atomicAdd(s_stats + 5 * ch + k, (unsigned long long)v[k]);
+        }
+        __syncthreads();
+        if (threadIdx.x < 25 && s_stats[threadIdx.x]) atomicAdd(stats + threadIdx.x, s_stats[threadIdx.x]);
     }
+    if (w >= 5 * n_modes) return;
     if (lane == 0) {
-        const double norm = ch < 2 ? (double)N : (double)N * (double)N;
+        // an FP64 division by one lane takes as long as the warp's sums: the host divides
+        const double norm = ch < 2 ? norm3 : norm4;
         const double cst = ch < 2 ? c3 : c4;
         if (ch >= 2 && scale4 != 1.0) {              // sampling estimate: inverse inclusion probability
             g *= scale4;
@@ -336,8 +343,8 @@ __global__ void reduce_kernel(int n_modes, int ld, int N, int5 n_part, int chann
         }
         // a rate kernel whose bounded wait expired leaves incomplete partials: poison Γ
         if (err && *err) g = __longlong_as_double(0x7ff8000000000000ll);
-        gamma[(size_t)ch * ld + ms] = g * cst / norm;
-        if (wp) wp[(size_t)ch * ld + ms] = p / norm;
+        gamma[(size_t)ch * ld + ms] = g * cst;
+        if (wp) wp[(size_t)ch * ld + ms] = p * norm;
         if (counts) counts[(size_t)ch * ld + ms] = n;
     }
 }
@@ -349,9 +356,10 @@ cudaError_t launch_reduce(const Tables &t, const RateArgs &a, int channel_mask, 
     if (threads == 0) return cudaSuccess;
     int5 np;
     np.a = a.n_part[0]; np.b = a.n_part[1]; np.c = a.n_part[2]; np.d = a.n_part[3]; np.e = a.n_part[4];
+    const double N = t.N;
     reduce_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
-        a.n_modes, a.out_ld > 0 ? a.out_ld : a.n_modes, t.N, np, channel_mask, c3, c4,
-        a.sample_all ? 1.0 : a.sample_scale, a.part_g, a.part_wp, a.part_n, a.part_items, a.part_ent,
+        a.n_modes, a.out_ld > 0 ? a.out_ld : a.n_modes, t.N, np, channel_mask, c3 / N, c4 / (N * N), 1.0 / N,
+        1.0 / (N * N), a.sample_all ? 1.0 : a.sample_scale, a.part_g, a.part_wp, a.part_n, a.part_items, a.part_ent,
         a.part_ev, a.part_cev, gamma, wp, counts, stats, a.err);
     return cudaGetLastError();
 }
