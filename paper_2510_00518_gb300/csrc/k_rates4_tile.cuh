@@ -377,13 +377,14 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                         w2f[j] = (float)s2 * t.omT32[j * N + q2];   // branch-major: lanes read consecutive q
                         w3f[j] = t.omT32[j * N + q3];
                     }
-#pragma unroll
+#pragma unroll 1
                     for (int j1 = 0; j1 < NB; ++j1) {
                         if (!((near >> j1) & 1u)) continue;
+                        const float b1 = w0f + (float)s1 * t.om32[q1 * NB + j1];
                         float mn = thr + 1.0f;
 #pragma unroll
                         for (int j2 = 0; j2 < NB; ++j2) {
-                            const float t2 = base32[j1] + w2f[j2];
+                            const float t2 = b1 + w2f[j2];
                             float r = fabsf(t2 - w3f[0]);        // six short chains
 #pragma unroll
                             for (int j3 = 1; j3 < NB; ++j3) r = fminf(r, fabsf(t2 - w3f[j3]));
@@ -790,6 +791,7 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
 #pragma unroll
                         for (int k = 0; k < 9; ++k) X[c][d][k] = czero<C>();
                         const int r0 = t.grp_start[c * NA + d], r1 = t.grp_start[c * NA + d + 1];
+#pragma unroll 2
                         for (int r = r0; r < r1; ++r) {
                             const C ph = cconj_if(Prow[r], s2 < 0);
                             const C *Wr = Wj + 9 * r;
