@@ -74,20 +74,30 @@ __device__ __forceinline__ bool pair_sampled(const RateArgs &a, int m0, int q1, 
     return (z ^ (z >> 31)) < a.sample_threshold;
 }
 
-// Window row of one (q'', λ''') for the four-phonon channels with adaptive σ: bit j'' set iff kept.
+// Window row of one (q'', λ''') for the four-phonon channels with adaptive σ: bit j'' set iff kept.  thr
+// bounds the window of every pair of the two points, so only the branches of |Δ32| <= thr have their width
+// formed (each lane goes through its own).  The tables are branch-major: neighbouring lanes hold neighbouring
+// points.
 template <int NB>
 static __device__ __noinline__ unsigned window_adaptive4_row(const Tables &t, const RateArgs &a, int ch, int s2,
-                                                             float base32, int m0, int m1, int q2, int m3,
-                                                             unsigned v2) {
-    const float w3 = t.om32[m3];
-    const float4 h3 = t.vp32[m3], l3 = t.vp32lo[m3];
-    unsigned keep = 0;
-    for (int j2 = 0; j2 < NB; ++j2) {
-        if (!((v2 >> j2) & 1u)) continue;
-        const int m2 = q2 * NB + j2;
-        const float ad = fabsf((base32 + (float)s2 * t.om32[m2]) - w3);
-        const float g32 = a.ad_c32 * vel_diff_norm32_approx(t.vp32[m2], t.vp32lo[m2], h3, l3);
+                                                             float base32, int m0, int m1, int q2, int q3,
+                                                             int j3, unsigned v2, float thr) {
+    const size_t N = t.N, i3 = j3 * N + q3;
+    const float w3 = t.omT32[i3];
+    unsigned near = 0, keep = 0;
+#pragma unroll
+    for (int j2 = 0; j2 < NB; ++j2)
+        near |= (unsigned)(fabsf((base32 + (float)s2 * t.omT32[j2 * N + q2]) - w3) <= thr) << j2;
+    near &= v2;
+    if (!near) return 0u;
+    const float4 h3 = t.vpT32[i3], l3 = t.vpTlo[i3];
+    for (; near; near &= near - 1) {
+        const int j2 = __ffs(near) - 1;
+        const size_t i2 = j2 * N + q2;
+        const float ad = fabsf((base32 + (float)s2 * t.omT32[i2]) - w3);
+        const float g32 = a.ad_c32 * vel_diff_norm32_approx(t.vpT32[i2], t.vpTlo[i2], h3, l3);
         const int w = window_adaptive32(a, ad, g32);
+        const int m2 = q2 * NB + j2, m3 = q3 * NB + j3;
         if (w == 2 || (w == 1 && window_exact_adaptive(t, a, ch, m0, m1, m2, m3, m2, m3))) keep |= 1u << j2;
     }
     return keep;

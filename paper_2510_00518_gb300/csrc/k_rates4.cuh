@@ -4,15 +4,15 @@
 // The paper (Algorithms 3-4) enumerates the kept processes on the CPU, ships index lists to
 // the GPU and evaluates V per process.  Here the same work is fused and factored so that the
 // dense parts are shared.  One thread block owns a unit (λ = (q, j), q') and loops over the
-// partner branch j'.  With q''' = q + s1 q' + s2 q'', the phase of a cluster factorises as
-//   exp(i(s1 q'.R1 + s2 q''.R2 - q'''.R3)) = exp(-i q.R3) exp(i s1 q'.(R1 - R3)) exp(i s2 q''.(R2 - R3)),
+// partner branch j'.  With q@3@ = q + s1 q' + s2 q'', the phase of a cluster factorises as
+//   exp(i(s1 q'.R1 + s2 q''.R2 - q@3@.R3)) = exp(-i q.R3) exp(i s1 q'.(R1 - R3)) exp(i s2 q''.(R2 - R3)),
 // so with a "key" r = (leg-2 atom c, leg-3 atom d, R2 - R3) the element is
-//   V = Σ_r P_r(q'')^s2 Σ_γδ W_r[γδ] e^s2_λ''(cγ) e*_λ'''(dδ),
+//   V = Σ_r P_r(q'')^s2 Σ_γδ W_r[γδ] e^s2_λ''(cγ) e*_λ@3@(dδ),
 //   W_r[γδ] = Σ_{clusters in r} exp(-i q.R3 + i s1 q'.(R1 - R3)) / sqrt(m) Σ_αβ Φ[αβγδ] e_λ(aα) e^s1_λ'(bβ),
 // W built once per (λ, q', j') in shared memory.  Partners q'' are enumerated one per thread,
 // the window is tested with an FP32 prefilter of proven error bound (ambiguous cases are
-// decided by the exact FP64 Δ), kept (q'', j''', j''-mask) items are compacted in order by a
-// block scan, and each item computes Y[cγ] = Σ_r P_r Σ_δ W_r[γδ] e*_λ'''(dδ) once for all its
+// decided by the exact FP64 Δ), kept (q'', j@3@, j''-mask) items are compacted in order by a
+// block scan, and each item computes Y[cγ] = Σ_r P_r Σ_δ W_r[γδ] e*_λ@3@(dδ) once for all its
 // j'' (V = Σ_cγ e^s2_λ''(cγ) Y[cγ]).
 #pragma once
 #include <algorithm>
@@ -76,7 +76,7 @@ __device__ __forceinline__ float two_sum(float a, float b, float &e) {
     return s;
 }
 
-// Δ = ω + s1 ω' + s2 ω'' - ω''' from hi/lo FP32 splits of each ω (|error| ~ 2^-44 ω_max): the
+// Δ = ω + s1 ω' + s2 ω'' - ω@3@ from hi/lo FP32 splits of each ω (|error| ~ 2^-44 ω_max): the
 // Gaussian's argument in the mixed path without FP64 instructions.
 __device__ __forceinline__ float delta_comp(float h0, float l0, float h1, float l1, float h2, float l2,
                                             float h3, float l3, int s1, int s2) {
@@ -89,8 +89,8 @@ __device__ __forceinline__ float delta_comp(float h0, float l0, float h1, float 
 }
 
 // Triangular domain of a (q', q'') pair (partner-swap symmetry of the summand): -1 the pair is the
-// swap of one evaluated elsewhere; 0 no symmetry used (weight 1); 1 weight 2; 2 +- with q'' = q'''
-// (keep j'' <= j'''); 3 ++ / -- with q'' = q' (keep j'' >= j').
+// swap of one evaluated elsewhere; 0 no symmetry used (weight 1); 1 weight 2; 2 +- with q'' = q@3@
+// (keep j'' <= j@3@); 3 ++ / -- with q'' = q' (keep j'' >= j').
 __device__ __forceinline__ int tri_code(const RateArgs &a, int ch, int q1, int q2, int q3) {
     if (ch == 3) {
         if (!(a.tri & 1)) return 0;
@@ -101,7 +101,7 @@ __device__ __forceinline__ int tri_code(const RateArgs &a, int ch, int q1, int q
 }
 
 // tri_code of a (q', q'') pair of mode m0 under the sampling estimate: a representative stands for
-// its own pair and, off the diagonal (code 1), for its swapped pair ((λ, q', q''') for +-,
+// its own pair and, off the diagonal (code 1), for its swapped pair ((λ, q', q@3@) for +-,
 // (λ, q'', q') for ++ and --); it keeps weight 2 when both are in the sample, becomes weight 1
 // (code 0) when one is, and is skipped (-1) when neither is.
 __device__ __forceinline__ int tri_code_sampled(const RateArgs &a, int ch, int m0, int q1, int q2, int q3, int N) {
@@ -118,7 +118,7 @@ __device__ __forceinline__ int tri_weight(int tri, int j1, int j2, int j3) {
     return tri == 0 ? 1 : tri == 1 ? 2 : tri == 2 ? (j2 < j3 ? 2 : 1) : (j2 > j1 ? 2 : 1);
 }
 
-// Window masks of one q'': bit j'' of mask[j'''] is set iff the process is kept (restricted to the
+// Window masks of one q'': bit j'' of mask[j@3@] is set iff the process is kept (restricted to the
 // triangular domain).  FP32 prefilter with the proven bound; candidates inside the band are
 // decided by the exact FP64 Δ.
 template <int NB, bool ADA>
@@ -138,14 +138,14 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
         for (int j3 = 0; j3 < NB; ++j3) mask[j3] = 0u;
         return 0;
     }
-    // branch pairs of the domain: j'' <= j''' (tri 2) or j'' >= j' (tri 3)
+    // branch pairs of the domain: j'' <= j@3@ (tri 2) or j'' >= j' (tri 3)
     auto dom = [&](int j3) -> unsigned {
         return tri == 2 ? (2u << j3) - 1u : tri == 3 ? ~((1u << j1) - 1u) : ~0u;
     };
     if constexpr (ADA) {
         int n = 0;
         for (int j3 = 0; j3 < NB; ++j3) {
-            mask[j3] = ((v3 >> j3) & 1u) ? window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3 * NB + j3, v2) & dom(j3)
+            mask[j3] = ((v3 >> j3) & 1u) ? window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3, j3, v2, thr) & dom(j3)
                                          : 0u;
             n += (mask[j3] != 0);
         }
@@ -154,8 +154,8 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
     float t2[NB], w3f[NB];
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
-        t2[j] = base32 + (float)s2 * t.om32[q2 * NB + j];
-        w3f[j] = t.om32[q3 * NB + j];
+        t2[j] = base32 + (float)s2 * t.omT32[(size_t)j * t.N + q2];
+        w3f[j] = t.omT32[(size_t)j * t.N + q3];
     }
     int n = 0;
 #pragma unroll
@@ -179,7 +179,7 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
     return n;
 }
 
-// One row of the window of (λ, λ'; q''): bit j'' set iff the process with λ''' = (q3, j3) is kept,
+// One row of the window of (λ, λ'; q''): bit j'' set iff the process with λ@3@ = (q3, j3) is kept,
 // restricted to the triangular domain.  A row none of whose |Δ32| can reach the window (FP32 sums are
 // monotonic in ω''; lo2, hi2: range of s2 ω'' over the participating branches; thr bounds the window of
 // every pair) is decided without looking at its pairs.
@@ -187,22 +187,22 @@ template <int NB, bool ADA>
 __device__ __forceinline__ unsigned window_row(const Tables &t, const RateArgs &a, int ch, int s2, float base32,
                                                int m0, int m1, int j1, double w0, int q2, int q3, unsigned v2,
                                                int j3, int tri, float lo2, float hi2, float thr) {
-    const float w3 = t.om32[q3 * NB + j3];
+    const float w3 = t.omT32[(size_t)j3 * t.N + q3];
     if ((base32 + lo2) - w3 > thr || (base32 + hi2) - w3 < -thr) return 0u;
     const unsigned dom = tri == 2 ? (2u << j3) - 1u : tri == 3 ? ~((1u << j1) - 1u) : ~0u;
     if constexpr (ADA) {
-        return window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3 * NB + j3, v2) & dom;
+        return window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3, j3, v2, thr) & dom;
     } else {
         unsigned near = 0;
 #pragma unroll
         for (int j2 = 0; j2 < NB; ++j2)
-            near |= (unsigned)(fabsf((base32 + (float)s2 * t.om32[q2 * NB + j2]) - w3) <= a.hi32) << j2;
+            near |= (unsigned)(fabsf((base32 + (float)s2 * t.omT32[(size_t)j2 * t.N + q2]) - w3) <= a.hi32) << j2;
         near &= v2 & dom;
         unsigned m = 0;
         while (near) {
             const int j2 = __ffs(near) - 1;
             near &= near - 1;
-            const float ad = fabsf((base32 + (float)s2 * t.om32[q2 * NB + j2]) - w3);
+            const float ad = fabsf((base32 + (float)s2 * t.omT32[(size_t)j2 * t.N + q2]) - w3);
             if (ad <= a.lo32 || window_exact4(ch, w0, t.om[m1], t.om[q2 * NB + j2], t.om[q3 * NB + j3], a.two_sigma))
                 m |= 1u << j2;
         }
@@ -238,7 +238,8 @@ struct GeneralSmem {
     C *W, *Ph, *E, *e0, *Con;
     unsigned long long *Q;         // X route: entries (q'', masks) [kQChunk]
     unsigned short *ent;           // else: entries (q'') [kQChunk]
-    unsigned *mask;                // [NB][kSubBatch] kept j'' per (j''', entry of the sub-batch)
+    unsigned *found;               // bit per q'' of the chunk
+    unsigned *mask;                // [NB][kSubBatch] kept j'' per (j@3@, entry of the sub-batch)
     unsigned long long *item;      // [kSubBatch * NB]
     R *proc;                       // [128 * NB][2] weight and |V|^2 of a pass' processes
     int n_con;                     // clusters per piece
@@ -250,7 +251,7 @@ struct GeneralSmem {
     }
     __host__ __device__ static size_t bytes(const Tables &t) {
         size_t b = sizeof(C) * ((size_t)t.n_keys * 9 + t.nc4 + NA * NA * 9 + NB + (NB & 1)) + buffer_bytes() +
-                   (XROUTE ? 0 : sizeof(unsigned short) * kQChunk);
+                   (XROUTE ? 0 : sizeof(unsigned short) * kQChunk + kQChunk / 8);
         return (b + 15) & ~size_t(15);
     }
     __device__ __forceinline__ GeneralSmem(unsigned char *smem, const Tables &t) {
@@ -267,6 +268,7 @@ struct GeneralSmem {
         proc = reinterpret_cast<R *>(item + kSubBatch * NB);
         mask = reinterpret_cast<unsigned *>(proc + 2 * 128 * NB);
         ent = reinterpret_cast<unsigned short *>(buf + buffer_bytes());
+        found = reinterpret_cast<unsigned *>(ent + kQChunk);
     }
 };
 
@@ -274,7 +276,7 @@ struct GeneralSmem {
 // the batched persistent kernel, which takes its units from a work list over many contexts).
 //
 // Up to two atoms, X[c,d][γδ] = Σ_r P_r W_r[γδ] is formed once per entry (q'') by the entry's thread, then
-// 36 complex multiply-adds per (q'', j''') item.  Larger cells list their entries, expand them into
+// 36 complex multiply-adds per (q'', j@3@) item.  Larger cells list their entries, expand them into
 // items a sub-batch at a time and take one item per thread: an item's Y (12 n_keys complex multiply-
 // adds) is the bulk of the work, and entries carry 1 to nb of them.  The weights of a pass go
 // through shared memory to the entry's owner thread, which adds them in order, so Γ's bits are those
@@ -453,7 +455,7 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                             for (int c = 0; c < NA; ++c)
 #pragma unroll
                                 for (int g = 0; g < 3; ++g) Y[c][g] = czero<C>();
-                            // Y[cγ] = Σ_dδ X[c,d][γδ] e*_λ'''(dδ)
+                            // Y[cγ] = Σ_dδ X[c,d][γδ] e*_λ@3@(dδ)
 #pragma unroll
                             for (int d = 0; d < NA; ++d) {
                                 C e3[3];
@@ -506,19 +508,25 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                                                                          z.v2, j3, z.tri, z.lo2, z.hi2, z.thr)
                                                    : 0u;
                     };
-                    unsigned found = 0;                             // bit i: this thread's i-th q'' is an entry
-                    int i = 0;
-                    for (int q2 = qb + threadIdx.x; q2 < qe; q2 += blockDim.x, ++i) {
+                    // which q'' are entries: three rows of one q'' a thread at a time, those of
+                    // a found one left out (a stale read of its bit costs the rows, no more)
+                    for (int k = threadIdx.x; k < kQChunk / 32; k += blockDim.x) sm.found[k] = 0;
+                    __syncthreads();
+                    for (int k = threadIdx.x; k < (qe - qb) * NA; k += blockDim.x) {
+                        const int jg = 3 * (k / (qe - qb)), o = k % (qe - qb), q2 = qb + o;
                         const Point z = point(q2);
                         if (z.tri < 0) continue;
-                        acc_cev += NB * NB;                         // visited
-#pragma unroll 1
-                        for (int j3 = 0; j3 < NB; ++j3)
-                            if (row(z, q2, j3)) {
-                                found |= 1u << i;
-                                break;
-                            }
+                        acc_cev += 3 * NB;                          // visited
+                        if ((reinterpret_cast<volatile unsigned *>(sm.found)[o >> 5] >> (o & 31)) & 1u) continue;
+                        if (row(z, q2, jg) || row(z, q2, jg + 1) || row(z, q2, jg + 2))
+                            atomicOr(&sm.found[o >> 5], 1u << (o & 31));
                     }
+                    __syncthreads();
+                    // the list, in the order of a thread per q'' (its first, second, ... q'')
+                    unsigned found = 0;
+                    int i = 0;
+                    for (int o = threadIdx.x; o < qe - qb; o += blockDim.x, ++i)
+                        found |= ((sm.found[o >> 5] >> (o & 31)) & 1u) << i;
                     int off = block_exclusive_scan(__popc(found), s_scan, &total);
                     for (; found; found &= found - 1)
                         sm.ent[off++] = (unsigned short)((__ffs(found) - 1) * blockDim.x + threadIdx.x);
@@ -526,21 +534,23 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
 
                     const int sub = blockDim.x % kSubBatch ? 32 : kSubBatch;
                     for (int eb = 0; eb < total; eb += sub) {
-                        // expand: the entry's owner (the thread it % blockDim of the whole list) lists its items
+                        // expand: the rows of the sub-batch over all threads, then the entry's owner (the thread
+                        // it % blockDim of the whole list) lists its items
+                        const int n_sub = min(sub, total - eb);
+                        for (int k = threadIdx.x; k < n_sub * NB; k += blockDim.x) {
+                            const int j3 = k / n_sub, o = k - j3 * n_sub, eq2 = qb + sm.ent[eb + o];
+                            sm.mask[j3 * kSubBatch + o] = row(point(eq2), eq2, j3);
+                        }
+                        __syncthreads();
                         const int mine = (int)threadIdx.x - eb % (int)blockDim.x;     // slot in the sub-batch
-                        const bool own = mine >= 0 && mine < sub && eb + mine < total;
+                        const bool own = mine >= 0 && mine < n_sub;
                         int n_it = 0, q2 = 0, tri = 0;
                         if (own) {
                             ++acc_ent;
                             q2 = qb + sm.ent[eb + mine];
-                            const Point z = point(q2);
-                            tri = z.tri;
+                            tri = point(q2).tri;
 #pragma unroll 1
-                            for (int j3 = 0; j3 < NB; ++j3) {
-                                const unsigned m = row(z, q2, j3);
-                                sm.mask[j3 * kSubBatch + mine] = m;
-                                n_it += m != 0;
-                            }
+                            for (int j3 = 0; j3 < NB; ++j3) n_it += sm.mask[j3 * kSubBatch + mine] != 0;
                         }
                         int n_items;
                         const int it0 = block_exclusive_scan(n_it, s_scan, &n_items), it1 = it0 + n_it;
@@ -570,7 +580,7 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                                 const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
                                                        t.mesh[0], t.mesh[1], t.mesh[2]);
                                 const C *P = P4 + (size_t)iq2 * t.n_keys;
-                                // Y[cγ] = Σ_d Σ_{r in (c,d)} P_r^s2 Σ_δ W_r[γδ] e*_λ'''(dδ)
+                                // Y[cγ] = Σ_d Σ_{r in (c,d)} P_r^s2 Σ_δ W_r[γδ] e*_λ@3@(dδ)
                                 C Y[NA][3];
 #pragma unroll
                                 for (int c = 0; c < NA; ++c) {
