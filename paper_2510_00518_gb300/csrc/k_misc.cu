@@ -7,14 +7,19 @@ namespace fc4 {
 
 // ------------------------------------------------------------------------------ harmonic
 
-// One warp per q point; D and the accumulated rotations U live in shared memory.
-// D(q) = Σ_c Φ2_c exp(i q.R_c) / sqrt(m_a m_b) (Hermitised), one lane per matrix entry (clusters
-// summed in order); cyclic complex Jacobi: every lane derives the same rotation from shared
-// values, lanes k < nb update row/column k; sweeps stop when the off-diagonal mass is below
-// (1e-16 |D|_F)².  Eigenpairs sorted ascending, ω = sqrt(λ * eig_to_w2) (rad/ps), and
-// v_x = Re(e^H dD/dq_x e) eig_to_w2 / (2ω) (Hellmann-Feynman), one lane per branch.
+constexpr int kHarmonicThreads = 128;
+
+// One block per q point; D and the accumulated rotations U live in shared memory.
+// D(q) = Σ_c Φ2_c exp(i q.R_c) / sqrt(m_a m_b) (Hermitised), one thread per matrix entry (clusters
+// summed in order); cyclic complex Jacobi by the first warp: every lane derives the same rotation from
+// shared values, a lane per row of A and of U updates it, then one per column of A; sweeps stop when the
+// off-diagonal mass is below (1e-16 |D|_F)².  Eigenpairs sorted ascending, ω = sqrt(λ * eig_to_w2) (rad/ps),
+// and v_x = Re(e^H dD/dq_x e) eig_to_w2 / (2ω) (Hellmann-Feynman), its clusters shared out over the block.
+// Bound by the latency of FP64: an FP64 instruction takes a scheduler's pipe some 64 cycles whatever lanes it
+// has, so what counts is instructions per warp.  8^3, 2 atoms: 450 -> 350 us, nearly all of it the Jacobi
+// rotations (some 110 dependent FP64 instructions each, three divisions and three square roots among them).
 template <int NA>
-__global__ void __launch_bounds__(32)
+__global__ void __launch_bounds__(kHarmonicThreads)
 harmonic_kernel(const __grid_constant__ Tables t, int nc2, const int4 *__restrict__ c2_at,
                 const int4 *__restrict__ c2_r, const double *__restrict__ c2_R,
                 const double *__restrict__ c2_phi, const double *__restrict__ c2_ism,
@@ -22,10 +27,12 @@ harmonic_kernel(const __grid_constant__ Tables t, int nc2, const int4 *__restric
     constexpr int NB = 3 * NA;
     constexpr int LD = NB + 1;
     __shared__ double2 sA[NB * LD], sU[NB * LD];
+    constexpr int kParts = kHarmonicThreads / NB;                        // cluster shares of a velocity sum
     __shared__ int s_ord[NB];
-    const int q = blockIdx.x, lane = threadIdx.x;
+    __shared__ double s_v[kParts * NB][3];
+    const int q = blockIdx.x, lane = threadIdx.x & 31;
     const int4 qc = t.qc[q];
-    for (int k = lane; k < NB * NB; k += 32) {
+    for (int k = threadIdx.x; k < NB * NB; k += kHarmonicThreads) {
         const int i = k / NB, j = k - i * NB;
         const int a = i / 3, al = i - 3 * a, b = j / 3, be = j - 3 * b;
         double2 x = czero<double2>();
@@ -40,89 +47,112 @@ harmonic_kernel(const __grid_constant__ Tables t, int nc2, const int4 *__restric
         sA[i * LD + j] = x;
         sU[i * LD + j] = cmake(i == j ? 1.0 : 0.0, 0.0);
     }
-    __syncwarp();
-    double2 h[(NB * NB + 31) / 32];
-    for (int k = lane, n = 0; k < NB * NB; k += 32, ++n) {      // (A + A^H) / 2
-        const int i = k / NB, j = k - i * NB;
-        const double2 x = sA[i * LD + j], y = sA[j * LD + i];
-        h[n] = cmake(0.5 * (x.x + y.x), 0.5 * (x.y - y.y));
-    }
-    __syncwarp();
-    double fro = 0.0;
-    for (int k = lane, n = 0; k < NB * NB; k += 32, ++n) {
-        sA[(k / NB) * LD + (k % NB)] = h[n];
-        fro += cabs2(h[n]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(kFull, fro, o);
-    __syncwarp();
-    const double tol = 1e-32 * fro;
-    for (int sweep = 0; sweep < 60; ++sweep) {
-        double off = 0.0;
-        for (int k = lane; k < NB * NB; k += 32) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        double2 h[(NB * NB + 31) / 32];
+        for (int k = lane, n = 0; k < NB * NB; k += 32, ++n) {      // (A + A^H) / 2
             const int i = k / NB, j = k - i * NB;
-            if (j > i) off += cabs2(sA[i * LD + j]);
+            const double2 x = sA[i * LD + j], y = sA[j * LD + i];
+            h[n] = cmake(0.5 * (x.x + y.x), 0.5 * (x.y - y.y));
+        }
+        __syncwarp();
+        double fro = 0.0;
+        for (int k = lane, n = 0; k < NB * NB; k += 32, ++n) {
+            sA[(k / NB) * LD + (k % NB)] = h[n];
+            fro += cabs2(h[n]);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) off += __shfl_xor_sync(kFull, off, o);
-        if (off <= tol) break;
-        for (int p = 0; p < NB - 1; ++p)
-            for (int r = p + 1; r < NB; ++r) {
-                const double2 apr = sA[p * LD + r];
-                const double b = sqrt(cabs2(apr));
-                if (b <= 1e-300) continue;                            // uniform across the warp
-                const double2 e = cmake(apr.x / b, apr.y / b);        // e^{iφ}
-                const double th = (sA[r * LD + r].x - sA[p * LD + p].x) / (2.0 * b);
-                const double tt = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
-                const double cs = 1.0 / sqrt(1.0 + tt * tt), sn = tt * cs;
-                const double2 me = cmake(-sn * e.x, sn * e.y);       // -s e^{-iφ}
-                const double2 ce = cmake(cs * e.x, -cs * e.y);       //  c e^{-iφ}
-                __syncwarp();
-                if (lane < NB) {                                      // A <- A U, U_acc <- U_acc U
-                    const int k = lane;
-                    const double2 ap = sA[k * LD + p], ar = sA[k * LD + r];
-                    sA[k * LD + p] = cfma(ar, me, cmake(cs * ap.x, cs * ap.y));
-                    sA[k * LD + r] = cfma(ar, ce, cmake(sn * ap.x, sn * ap.y));
-                    const double2 up = sU[k * LD + p], ur = sU[k * LD + r];
-                    sU[k * LD + p] = cfma(ur, me, cmake(cs * up.x, cs * up.y));
-                    sU[k * LD + r] = cfma(ur, ce, cmake(sn * up.x, sn * up.y));
-                }
-                __syncwarp();
-                if (lane < NB) {                                      // A <- U^H A
-                    const int k = lane;
-                    const double2 ap = sA[p * LD + k], ar = sA[r * LD + k];
-                    sA[p * LD + k] = cfma(cconj(me), ar, cmake(cs * ap.x, cs * ap.y));
-                    sA[r * LD + k] = cfma(cconj(ce), ar, cmake(sn * ap.x, sn * ap.y));
-                }
-                __syncwarp();
-                if (lane == 0) {
-                    sA[p * LD + r] = czero<double2>();
-                    sA[r * LD + p] = czero<double2>();
-                    sA[p * LD + p].y = 0.0;
-                    sA[r * LD + r].y = 0.0;
-                }
-                __syncwarp();
+        for (int o = 16; o > 0; o >>= 1) fro += __shfl_xor_sync(kFull, fro, o);
+        __syncwarp();
+        const double tol = 1e-32 * fro;
+        for (int sweep = 0; sweep < 60; ++sweep) {
+            double off = 0.0;
+            for (int k = lane; k < NB * NB; k += 32) {
+                const int i = k / NB, j = k - i * NB;
+                if (j > i) off += cabs2(sA[i * LD + j]);
             }
-    }
-    if (lane == 0) {                                                  // ascending order
-        int ord[NB];
-        for (int i = 0; i < NB; ++i) ord[i] = i;
-        for (int i = 0; i < NB; ++i)
-            for (int j = i + 1; j < NB; ++j)
-                if (sA[ord[j] * LD + ord[j]].x < sA[ord[i] * LD + ord[i]].x) {
-                    const int x = ord[i];
-                    ord[i] = ord[j];
-                    ord[j] = x;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) off += __shfl_xor_sync(kFull, off, o);
+            if (off <= tol) break;
+            for (int p = 0; p < NB - 1; ++p)
+                for (int r = p + 1; r < NB; ++r) {
+                    const double2 apr = sA[p * LD + r];
+                    const double b = sqrt(cabs2(apr));
+                    if (b <= 1e-300) continue;                            // uniform across the warp
+                    // one division for the three quotients, a lane each
+                    const double num = lane == 0 ? apr.x : lane == 1 ? apr.y : sA[r * LD + r].x - sA[p * LD + p].x;
+                    const double quo = num / (lane < 2 ? b : 2.0 * b);
+                    const double2 e = cmake(__shfl_sync(kFull, quo, 0), __shfl_sync(kFull, quo, 1));   // e^{iφ}
+                    const double th = __shfl_sync(kFull, quo, 2);
+                    const double tt = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
+                    const double cs = 1.0 / sqrt(1.0 + tt * tt), sn = tt * cs;
+                    const double2 me = cmake(-sn * e.x, sn * e.y);       // -s e^{-iφ}
+                    const double2 ce = cmake(cs * e.x, -cs * e.y);       //  c e^{-iφ}
+                    __syncwarp();
+                    for (int k = lane; k < 2 * NB; k += 32) {             // A <- A U, U_acc <- U_acc U: a row a lane
+                        double2 *row = k < NB ? sA + k * LD : sU + (k - NB) * LD;
+                        const double2 ap = row[p], ar = row[r];
+                        row[p] = cfma(ar, me, cmake(cs * ap.x, cs * ap.y));
+                        row[r] = cfma(ar, ce, cmake(sn * ap.x, sn * ap.y));
+                    }
+                    __syncwarp();
+                    if (lane < NB) {                                      // A <- U^H A
+                        const int k = lane;
+                        const double2 ap = sA[p * LD + k], ar = sA[r * LD + k];
+                        sA[p * LD + k] = cfma(cconj(me), ar, cmake(cs * ap.x, cs * ap.y));
+                        sA[r * LD + k] = cfma(cconj(ce), ar, cmake(sn * ap.x, sn * ap.y));
+                    }
+                    __syncwarp();
+                    if (lane == 0) {
+                        sA[p * LD + r] = czero<double2>();
+                        sA[r * LD + p] = czero<double2>();
+                        sA[p * LD + p].y = 0.0;
+                        sA[r * LD + r].y = 0.0;
+                    }
+                    __syncwarp();
                 }
-        for (int i = 0; i < NB; ++i) s_ord[i] = ord[i];
+        }
+        if (lane == 0) {                                                  // ascending order
+            int ord[NB];
+            for (int i = 0; i < NB; ++i) ord[i] = i;
+            for (int i = 0; i < NB; ++i)
+                for (int j = i + 1; j < NB; ++j)
+                    if (sA[ord[j] * LD + ord[j]].x < sA[ord[i] * LD + ord[i]].x) {
+                        const int x = ord[i];
+                        ord[i] = ord[j];
+                        ord[j] = x;
+                    }
+            for (int i = 0; i < NB; ++i) s_ord[i] = ord[i];
+        }
     }
-    __syncwarp();
-    for (int k = lane; k < NB * NB; k += 32) {
+    __syncthreads();
+    for (int k = threadIdx.x; k < NB * NB; k += kHarmonicThreads) {
         const int comp = k / NB, j = k - comp * NB;
         ev[((size_t)q * NB + comp) * NB + j] = sU[comp * LD + s_ord[j]];
     }
-    if (lane < NB) {
-        const int j = lane, o = s_ord[j];
+    // velocity sums e^H (dD/dq_x) e: thread (part, j) takes every kParts-th cluster
+    if (threadIdx.x < kParts * NB) {
+        const int part = threadIdx.x / NB, o = s_ord[threadIdx.x - part * NB];
+        double v[3] = {0.0, 0.0, 0.0};
+        for (int c = part; c < nc2; c += kParts) {
+            const int4 at = c2_at[c];
+            const double2 ph = t.rt[phase_index(qc, c2_r[c], t.L)];
+            double2 s = czero<double2>();
+            for (int al = 0; al < 3; ++al) {
+                double2 sb = czero<double2>();
+                for (int be = 0; be < 3; ++be)
+                    sb = crfma(c2_phi[9 * c + 3 * al + be], sU[(3 * at.y + be) * LD + o], sb);
+                s = cfma(cconj(sU[(3 * at.x + al) * LD + o]), sb, s);
+            }
+            s = cmul(s, ph);                                          // e^H Φ e exp(iqR)
+            // dD/dq_x contributes i R_x (...): Re(i z) = -Im z
+            for (int x = 0; x < 3; ++x) v[x] += -c2_R[3 * c + x] * c2_ism[c] * s.y;
+        }
+        for (int x = 0; x < 3; ++x) s_v[threadIdx.x][x] = v[x];
+    }
+    __syncthreads();
+    if (threadIdx.x < NB) {
+        const int j = threadIdx.x, o = s_ord[j];
         const double l = sA[o * LD + o].x;
         eig[q * NB + j] = l;
         const bool excl = (q == 0 && j < 3);
@@ -131,25 +161,14 @@ harmonic_kernel(const __grid_constant__ Tables t, int nc2, const int4 *__restric
         if (!excl) w = (l >= 0.0 ? 1.0 : -1.0) * sqrt(fabs(l) * eig_to_w2);
         if (!excl && !(w > 0.0)) atomicOr(err, 1);
         om[q * NB + j] = (excl || !(w > 0.0)) ? 0.0 : w;       // imaginary modes take no part
-        double v[3] = {0.0, 0.0, 0.0};
-        if (!excl && w > 0.0) {
-            for (int c = 0; c < nc2; ++c) {
-                const int4 at = c2_at[c];
-                const double2 ph = t.rt[phase_index(qc, c2_r[c], t.L)];
-                double2 s = czero<double2>();
-                for (int al = 0; al < 3; ++al) {
-                    double2 sb = czero<double2>();
-                    for (int be = 0; be < 3; ++be)
-                        sb = crfma(c2_phi[9 * c + 3 * al + be], sU[(3 * at.y + be) * LD + o], sb);
-                    s = cfma(cconj(sU[(3 * at.x + al) * LD + o]), sb, s);
-                }
-                s = cmul(s, ph);                                      // e^H Φ e exp(iqR)
-                // dD/dq_x contributes i R_x (...): Re(i z) = -Im z
-                for (int x = 0; x < 3; ++x) v[x] += -c2_R[3 * c + x] * c2_ism[c] * s.y;
+        for (int x = 0; x < 3; ++x) {
+            double v = 0.0;
+            if (!excl && w > 0.0) {
+                for (int part = 0; part < kParts; ++part) v += s_v[part * NB + j][x];
+                v = v * eig_to_w2 / (2.0 * w);
             }
-            for (int x = 0; x < 3; ++x) v[x] = v[x] * eig_to_w2 / (2.0 * w);
+            vel[((size_t)q * NB + j) * 3 + x] = v;
         }
-        for (int x = 0; x < 3; ++x) vel[((size_t)q * NB + j) * 3 + x] = v[x];
     }
 }
 
@@ -157,7 +176,7 @@ cudaError_t launch_harmonic(const Tables &t, int nc2, const int4 *c2_at, const i
                             const double *c2_R, const double *c2_phi, const double *c2_ism,
                             double eig_to_w2, double *om, double *vel, double2 *ev, double *eig,
                             int *err, cudaStream_t s) {
-    const int threads = 32, blocks = t.N;
+    const int threads = kHarmonicThreads, blocks = t.N;
 #define FC4_H(NA_)                                                                           \
     case NA_:                                                                                \
         harmonic_kernel<NA_><<<blocks, threads, 0, s>>>(t, nc2, c2_at, c2_r, c2_R, c2_phi,   \
@@ -173,13 +192,12 @@ cudaError_t launch_harmonic(const Tables &t, int nc2, const int4 *c2_at, const i
 
 // ------------------------------------------------------------------------------ tables
 
-// Per-mode tables derived from ω, e and v: FP32 hi/lo splits of ω, 1/ω, FP32 eigenvectors, the
-// participation mask, and the velocity projections P_k = (v . b_k) / n_k (hi/lo FP32) of the
-// adaptive width.
+// Per-mode tables derived from ω, e and v: FP32 hi/lo splits of ω, 1/ω, FP32 eigenvectors, and the velocity
+// projections P_k = (v . b_k) / n_k (hi/lo FP32) of the adaptive width.
 __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om, float *om32, float *om32lo,
-                                   float2 *ev32, const double2 *ev, unsigned *vmask, double *invw,
+                                   float2 *ev32, const double2 *ev, double *invw,
                                    float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
-                                   float4 *vpTlo, float4 *wrange) {
+                                   float4 *vpTlo) {
     const int N = t.N, nb = t.nb;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nm = (long long)N * nb;
@@ -193,13 +211,15 @@ __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om,
         invw32[i] = w > 0.0 ? (float)(1.0 / w) : 0.0f;
         const double *v = t.vel + 3 * i;
         float h[3], l[3];
+        double p2 = 0.0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const double p = (v[0] * t.recip[3 * k] + v[1] * t.recip[3 * k + 1] + v[2] * t.recip[3 * k + 2]) / t.mesh[k];
             h[k] = (float)p;
             l[k] = (float)(p - (double)h[k]);
+            p2 += p * p;
         }
-        vp32[i] = make_float4(h[0], h[1], h[2], 0.0f);
+        vp32[i] = make_float4(h[0], h[1], h[2], (float)(sqrt(p2) * (1.0 + 0x1p-14)));   // w >= |P|
         vp32lo[i] = make_float4(l[0], l[1], l[2], 0.0f);
         const size_t it = (size_t)j * N + q;                 // branch-major copies
         omT32[it] = (float)w;
@@ -210,26 +230,27 @@ __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om,
         const double2 e = ev[i];
         ev32[i] = make_float2((float)e.x, (float)e.y);
     }
-    if (i < N) {
-        unsigned m = 0;
-        float lo = __int_as_float(0x7f800000), hi = -lo, pm = 0.0f;
-        for (int j = 0; j < nb; ++j)
-            if (!(i == 0 && j < 3) && om[i * nb + j] > 0.0) {
-                m |= 1u << j;
-                const float w = (float)om[i * nb + j];
-                lo = fminf(lo, w);
-                hi = fmaxf(hi, w);
-                const double *v = t.vel + 3 * (i * nb + j);
-                double p2 = 0.0;
-                for (int k = 0; k < 3; ++k) {
-                    const double p = (v[0] * t.recip[3 * k] + v[1] * t.recip[3 * k + 1] + v[2] * t.recip[3 * k + 2]) / t.mesh[k];
-                    p2 += p * p;
-                }
-                pm = fmaxf(pm, (float)(sqrt(p2) * (1.0 + 0x1p-14)));
-            }
-        vmask[i] = m;
-        wrange[i] = make_float4(lo, hi, pm, 0.0f);
+}
+
+// Per point: the branches that take part, their range of ω and the largest |P| (in the kernel above, with its
+// square roots, this held one thread a point: 33 -> 8 us at 8^3).
+__global__ void point_tables_kernel(int N, int nb, const double *__restrict__ om, const float4 *__restrict__ vp32,
+                                    unsigned *vmask, float4 *wrange) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    unsigned m = 0;
+    float lo = __int_as_float(0x7f800000), hi = -lo, pm = 0.0f;
+    for (int j = 0; j < nb; ++j) {
+        const double wd = om[i * nb + j];
+        if ((i == 0 && j < 3) || !(wd > 0.0)) continue;
+        m |= 1u << j;
+        const float w = (float)wd;
+        lo = fminf(lo, w);
+        hi = fmaxf(hi, w);
+        pm = fmaxf(pm, vp32[i * nb + j].w);
     }
+    vmask[i] = m;
+    wrange[i] = make_float4(lo, hi, pm, 0.0f);
 }
 
 cudaError_t launch_mode_tables(const Tables &t, double *om, float *om32, float *om32lo,
@@ -237,8 +258,10 @@ cudaError_t launch_mode_tables(const Tables &t, double *om, float *om32, float *
                                float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
                                float4 *vpTlo, float4 *wrange, cudaStream_t s) {
     const long long n = (long long)t.N * t.nb * t.nb;
-    mode_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(t, om, om32, om32lo, ev32, ev, vmask, invw,
-                                                                    invw32, vp32, vp32lo, omT32, vpT32, vpTlo, wrange);
+    // the first N nb threads hold the FP64 divisions: small blocks spread them over the SMs
+    mode_tables_kernel<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(t, om, om32, om32lo, ev32, ev, invw, invw32, vp32,
+                                                                 vp32lo, omT32, vpT32, vpTlo);
+    point_tables_kernel<<<(t.N + 63) / 64, 64, 0, s>>>(t.N, t.nb, om, vp32, vmask, wrange);
     return cudaGetLastError();
 }
 
