@@ -57,6 +57,9 @@ struct fc4_ctx {
     long long n_launches = 0;
     double volume = 0.0;
     std::vector<void *> owned;
+    char *slab = nullptr;                   // current slab of fc4_init: used [0, lo) and [hi, kSlab)
+    size_t slab_lo = 0, slab_hi = 0, slab_sent = 0;
+    std::vector<char> slab_host;            // contents of [0, lo); those up to slab_sent are on the device
     std::map<void *, size_t> alloc_bytes;  // size of each allocation (entries of freed ones are stale)
     std::vector<int> perm4;                 // device cluster slot -> input cluster index
     std::vector<int> swap12, swap23;        // input cluster -> the cluster with legs 1,2 (2,3) swapped
@@ -149,12 +152,88 @@ cudaError_t dalloc(fc4_ctx *c, T **p, size_t n) {
     return e;
 }
 
+// fc4_init's arrays up to kSlab / 4 bytes come from slabs of kSlab bytes: uploaded ones from the bottom, in
+// order, so that those of a slab go over in one copy before the first kernel that reads them; others from the
+// top.  Some seventy arrays were an allocation (6-19 us), a free (6-17 us) and half of them a copy (8-12 us)
+// each: 8^3, 2 atoms, fc4_init 1370 -> 970 us (350 of them the harmonic solution), fc4_destroy 690 -> 490 us.
+constexpr size_t kSlab = (size_t)2 << 20;
+
+cudaError_t flush_uploads(fc4_ctx *c) {
+    if (c->slab_lo == c->slab_sent) return cudaSuccess;
+    const cudaError_t e = cudaMemcpy(c->slab + c->slab_sent, c->slab_host.data() + c->slab_sent,
+                                     c->slab_lo - c->slab_sent, cudaMemcpyHostToDevice);
+    c->slab_sent = c->slab_lo;
+    return e;
+}
+
+// room for bytes (a multiple of 256) in the slab
+cudaError_t slab_room(fc4_ctx *c, size_t bytes) {
+    if (c->slab && c->slab_hi - c->slab_lo >= bytes) return cudaSuccess;
+    cudaError_t e = flush_uploads(c);
+    if (e != cudaSuccess) return e;
+    e = dalloc(c, &c->slab, kSlab);
+    c->slab_lo = c->slab_sent = 0;
+    c->slab_hi = e == cudaSuccess ? kSlab : 0;
+    c->slab_host.clear();
+    return e;
+}
+
+size_t slab_bytes(size_t n, size_t size) { return (std::max<size_t>(1, n) * size + 255) & ~(size_t)255; }
+
+// an array that lives as long as the context (fc4_init only; other arrays are freed and grown: dalloc)
+template <typename T>
+cudaError_t place(fc4_ctx *c, T **p, size_t n) {
+    const size_t bytes = slab_bytes(n, sizeof(T));
+    if (bytes > kSlab / 4) return dalloc(c, p, n);
+    const cudaError_t e = slab_room(c, bytes);
+    *p = nullptr;
+    if (e != cudaSuccess) return e;
+    c->slab_hi -= bytes;
+    *p = reinterpret_cast<T *>(c->slab + c->slab_hi);
+    return cudaSuccess;
+}
+
+// the same with contents; valid on the device after flush_uploads
 template <typename T>
 cudaError_t upload(fc4_ctx *c, T **p, const std::vector<T> &h) {
-    cudaError_t e = dalloc(c, p, h.size());
+    const size_t bytes = slab_bytes(h.size(), sizeof(T));
+    if (bytes > kSlab / 4) {
+        const cudaError_t e = dalloc(c, p, h.size());
+        return e != cudaSuccess ? e : cudaMemcpy(*p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
+    }
+    const cudaError_t e = slab_room(c, bytes);
+    *p = nullptr;
     if (e != cudaSuccess) return e;
-    if (!h.empty()) e = cudaMemcpy(*p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
-    return e;
+    c->slab_host.resize(c->slab_lo + bytes);
+    if (!h.empty()) std::memcpy(c->slab_host.data() + c->slab_lo, h.data(), h.size() * sizeof(T));
+    *p = reinterpret_cast<T *>(c->slab + c->slab_lo);
+    c->slab_lo += bytes;
+    return cudaSuccess;
+}
+
+// The seven partial arrays of need entries each, in one allocation (of seven: 39 + 67 us each at 63 MB).
+cudaError_t grow_partials(fc4_ctx *c, size_t need) {
+    static_assert(sizeof(double) == 8 && sizeof(long long) == 8, "one element size");
+    if (c->part_g) {
+        cudaFree(c->part_g);
+        c->owned.erase(std::find(c->owned.begin(), c->owned.end(), (void *)c->part_g));
+    }
+    c->part_wp = nullptr;
+    c->part_n = c->part_items = c->part_ent = c->part_ev = c->part_cev = nullptr;
+    c->part_cap = 0;
+    const cudaError_t e = dalloc(c, &c->part_g, 7 * need);
+    if (e != cudaSuccess) {
+        c->part_g = nullptr;
+        return e;
+    }
+    c->part_wp = c->part_g + need;
+    c->part_n = reinterpret_cast<long long *>(c->part_wp + need);
+    c->part_items = c->part_n + need;
+    c->part_ent = c->part_items + need;
+    c->part_ev = c->part_ent + need;
+    c->part_cev = c->part_ev + need;
+    c->part_cap = need;
+    return cudaSuccess;
 }
 
 int gcd_i(int a, int b) { return b ? gcd_i(b, a % b) : a; }
@@ -577,7 +656,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         FC4_TRY(upload(c, &d_ki, k_idx));
         FC4_TRY(upload(c, &d_gs, g_start));
         FC4_TRY(upload(c, &d_kr, kr));
-        FC4_TRY(dalloc(c, &d_P3, (size_t)N * kr.size()));
+        FC4_TRY(place(c, &d_P3, (size_t)N * kr.size()));
         std::vector<int> perm, pairs;
         pair_keys(kv3, na * na, perm, pairs);
         int *d_perm, *d_pairs;
@@ -589,6 +668,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         t.k3_idx = d_ki;
         t.grp3_start = d_gs;
         t.P3 = d_P3;
+        FC4_TRY(flush_uploads(c));
         FC4_TRY(fc4::launch_phase_tables(t, t.n_keys3, d_kr, d_P3, nullptr, 0));
     }
 
@@ -632,12 +712,14 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         std::vector<Key> keys;
         for (auto &kv : key_id) { kv.second = nk++; keys.push_back(kv.first); }
         t.n_keys = nk;
+        std::vector<int> kid(c->nc4);                 // key of each cluster
+        for (int i = 0; i < c->nc4; ++i) kid[i] = key_id[ck[i]];
         c->perm4.resize(c->nc4);
         std::iota(c->perm4.begin(), c->perm4.end(), 0);
         std::stable_sort(c->perm4.begin(), c->perm4.end(),
-                         [&](int x, int y) { return key_id[ck[x]] < key_id[ck[y]]; });
+                         [&](int x, int y) { return kid[x] < kid[y]; });
         std::vector<int> key_start(nk + 1, 0);
-        for (int i = 0; i < c->nc4; ++i) key_start[key_id[ck[i]] + 1]++;
+        for (int i = 0; i < c->nc4; ++i) key_start[kid[i] + 1]++;
         for (int k = 0; k < nk; ++k) key_start[k + 1] += key_start[k];
         for (int g = 0; g <= na * na; ++g) t.grp_start[g] = nk;
         for (int k = nk - 1; k >= 0; --k) t.grp_start[std::get<0>(keys[k])] = k;
@@ -667,14 +749,14 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         // the clusters of each (key, leg-1 atom), in cluster order: the W kernels' phase fold
         std::vector<int> kb_start((size_t)nk * na + 1, 0), kb_idx(c->nc4);
         for (int s = 0; s < c->nc4; ++s) {
-            const int r = key_id[ck[c->perm4[s]]];
+            const int r = kid[c->perm4[s]];
             kb_start[(size_t)r * na + at[s].y + 1]++;
         }
         for (size_t g = 0; g < (size_t)nk * na; ++g) kb_start[g + 1] += kb_start[g];
         {
             std::vector<int> fill(kb_start.begin(), kb_start.end() - 1);
             for (int s = 0; s < c->nc4; ++s) {
-                const int r = key_id[ck[c->perm4[s]]];
+                const int r = kid[c->perm4[s]];
                 kb_idx[fill[(size_t)r * na + at[s].y]++] = s;
             }
         }
@@ -722,7 +804,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
             FC4_TRY(upload(c, &c->swap12_dev, s12));
             FC4_TRY(upload(c, &c->swap23_dev, s23));
         }
-        FC4_TRY(dalloc(c, &c->adj_tmp, 81 * (size_t)std::max(1, c->nc4)));
+        FC4_TRY(place(c, &c->adj_tmp, 81 * (size_t)std::max(1, c->nc4)));
         t.c4_at = d_at;
         t.c4_r3 = d_r3;
         t.c4_r13 = d_r13;
@@ -735,40 +817,41 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         t.kb_idx = d_kbi;
         double2 *d_P4;
         float2 *d_P4_32;
-        FC4_TRY(dalloc(c, &d_P4, (size_t)N * nk));
-        FC4_TRY(dalloc(c, &d_P4_32, (size_t)N * nk));
+        FC4_TRY(place(c, &d_P4, (size_t)N * nk));
+        FC4_TRY(place(c, &d_P4_32, (size_t)N * nk));
         t.P4 = d_P4;
         t.P4_32 = d_P4_32;
+        FC4_TRY(flush_uploads(c));
         FC4_TRY(fc4::launch_phase_tables(t, nk, d_kr, d_P4, d_P4_32, 0));
     }
 
     // modes: device harmonic solve
     const size_t nm = (size_t)N * nb;
-    FC4_TRY(dalloc(c, &c->om, nm));
-    FC4_TRY(dalloc(c, &c->vel, 3 * nm));
-    FC4_TRY(dalloc(c, &c->eig, nm));
-    FC4_TRY(dalloc(c, &c->ev, nm * nb));
-    FC4_TRY(dalloc(c, &c->ev32, nm * nb));
-    FC4_TRY(dalloc(c, &c->om32, nm));
-    FC4_TRY(dalloc(c, &c->om32lo, nm));
-    FC4_TRY(dalloc(c, &c->invw, nm));
-    FC4_TRY(dalloc(c, &c->invw32, nm));
-    FC4_TRY(dalloc(c, &c->occ, nm));
-    FC4_TRY(dalloc(c, &c->occ32, nm));
-    FC4_TRY(dalloc(c, &c->vmask, (size_t)N));
-    FC4_TRY(dalloc(c, &c->vp32, nm));
-    FC4_TRY(dalloc(c, &c->vp32lo, nm));
-    FC4_TRY(dalloc(c, &c->omT32, nm));
-    FC4_TRY(dalloc(c, &c->vpT32, nm));
-    FC4_TRY(dalloc(c, &c->vpTlo, nm));
-    FC4_TRY(dalloc(c, &c->wrange, (size_t)N));
-    FC4_TRY(dalloc(c, &c->mode4, nm));
-    FC4_TRY(dalloc(c, &c->err, 1));
+    FC4_TRY(place(c, &c->om, nm));
+    FC4_TRY(place(c, &c->vel, 3 * nm));
+    FC4_TRY(place(c, &c->eig, nm));
+    FC4_TRY(place(c, &c->ev, nm * nb));
+    FC4_TRY(place(c, &c->ev32, nm * nb));
+    FC4_TRY(place(c, &c->om32, nm));
+    FC4_TRY(place(c, &c->om32lo, nm));
+    FC4_TRY(place(c, &c->invw, nm));
+    FC4_TRY(place(c, &c->invw32, nm));
+    FC4_TRY(place(c, &c->occ, nm));
+    FC4_TRY(place(c, &c->occ32, nm));
+    FC4_TRY(place(c, &c->vmask, (size_t)N));
+    FC4_TRY(place(c, &c->vp32, nm));
+    FC4_TRY(place(c, &c->vp32lo, nm));
+    FC4_TRY(place(c, &c->omT32, nm));
+    FC4_TRY(place(c, &c->vpT32, nm));
+    FC4_TRY(place(c, &c->vpTlo, nm));
+    FC4_TRY(place(c, &c->wrange, (size_t)N));
+    FC4_TRY(place(c, &c->mode4, nm));
+    FC4_TRY(place(c, &c->err, 1));
     FC4_TRY(cudaMemset(c->err, 0, sizeof(int)));
-    FC4_TRY(dalloc(c, &c->dev_err, 1));
+    FC4_TRY(place(c, &c->dev_err, 1));
     FC4_TRY(cudaMemset(c->dev_err, 0, sizeof(int)));
-    FC4_TRY(dalloc(c, &c->kappa_part, 9 * (size_t)fc4::kKappaBlocks));
-    FC4_TRY(dalloc(c, &c->kappa_counter, 1));
+    FC4_TRY(place(c, &c->kappa_part, 9 * (size_t)fc4::kKappaBlocks));
+    FC4_TRY(place(c, &c->kappa_counter, 1));
     FC4_TRY(cudaMemset(c->kappa_counter, 0, sizeof(unsigned)));
     t.om = c->om;
     t.om32 = c->om32;
@@ -796,6 +879,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         FC4_TRY(upload(c, &d_R, c2_R));
         FC4_TRY(upload(c, &d_phi, c2_phi));
         FC4_TRY(upload(c, &d_ism, c2_ism));
+        FC4_TRY(flush_uploads(c));
         FC4_TRY(fc4::launch_harmonic(t, c->nc2, d_at, d_r, d_R, d_phi, d_ism, kEigToW2, c->om, c->vel,
                                      c->ev, c->eig, c->err, 0));
     }
@@ -809,6 +893,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     if (refresh_modes(c) != FC4_OK) return bail(FC4_ERR_CUDA);
     FC4_TRY(cudaDeviceSynchronize());
 #undef FC4_TRY
+    std::vector<char>().swap(c->slab_host);
     *out = c;
     return FC4_OK;
 }
@@ -927,22 +1012,7 @@ fc4_status rates_call(fc4_ctx *c, double T_K, int sigma_adaptive, double sigma_v
         chunk = std::max<size_t>(1, std::min(chunk, w_cap(c) / per_mode));
     }
     const size_t need = (size_t)5 * chunk * N;
-    if (need > c->part_cap) {
-        for (void *p : {(void *)c->part_g, (void *)c->part_wp, (void *)c->part_n, (void *)c->part_items,
-                        (void *)c->part_ent, (void *)c->part_ev, (void *)c->part_cev})
-            if (p) { cudaFree(p); c->owned.erase(std::find(c->owned.begin(), c->owned.end(), p)); }
-        c->part_g = c->part_wp = nullptr;
-        c->part_n = c->part_items = c->part_ent = c->part_ev = c->part_cev = nullptr;
-        c->part_cap = 0;
-        FC4_CUDA(c, dalloc(c, &c->part_g, need));
-        FC4_CUDA(c, dalloc(c, &c->part_wp, need));
-        FC4_CUDA(c, dalloc(c, &c->part_n, need));
-        FC4_CUDA(c, dalloc(c, &c->part_items, need));
-        FC4_CUDA(c, dalloc(c, &c->part_ent, need));
-        FC4_CUDA(c, dalloc(c, &c->part_ev, need));
-        FC4_CUDA(c, dalloc(c, &c->part_cev, need));
-        c->part_cap = need;
-    }
+    if (need > c->part_cap) FC4_CUDA(c, grow_partials(c, need));
     if (bte_F) {                          // BTE partials [5][chunk][N][3] and the FP32 copy of F
         if (3 * need > c->part_d_cap) {
             if (c->part_d) { cudaFree(c->part_d); c->owned.erase(std::find(c->owned.begin(), c->owned.end(), (void *)c->part_d)); }
@@ -1649,22 +1719,7 @@ extern "C" fc4_status fc4_batch_rates(fc4_batch *b, double T_K, double sigma_val
             c->modes_on_device.clear();
         }
         const size_t need = (size_t)5 * nm * N;
-        if (need > c->part_cap) {
-            for (void *p : {(void *)c->part_g, (void *)c->part_wp, (void *)c->part_n, (void *)c->part_items,
-                            (void *)c->part_ent, (void *)c->part_ev, (void *)c->part_cev})
-                if (p) { cudaFree(p); c->owned.erase(std::find(c->owned.begin(), c->owned.end(), p)); }
-            c->part_g = c->part_wp = nullptr;
-            c->part_n = c->part_items = c->part_ent = c->part_ev = c->part_cev = nullptr;
-            c->part_cap = 0;
-            FC4_BCUDA(b, dalloc(c, &c->part_g, need));
-            FC4_BCUDA(b, dalloc(c, &c->part_wp, need));
-            FC4_BCUDA(b, dalloc(c, &c->part_n, need));
-            FC4_BCUDA(b, dalloc(c, &c->part_items, need));
-            FC4_BCUDA(b, dalloc(c, &c->part_ent, need));
-            FC4_BCUDA(b, dalloc(c, &c->part_ev, need));
-            FC4_BCUDA(b, dalloc(c, &c->part_cev, need));
-            c->part_cap = need;
-        }
+        if (need > c->part_cap) FC4_BCUDA(b, grow_partials(c, need));
         if (modes != c->modes_on_device) {
             FC4_BCUDA(b, cudaMemcpyAsync(c->modes, modes.data(), nm * sizeof(int), cudaMemcpyHostToDevice, s));
             c->modes_on_device = modes;
