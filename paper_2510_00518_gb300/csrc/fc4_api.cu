@@ -75,7 +75,7 @@ struct fc4_ctx {
     double2 *ev = nullptr;
     float2 *ev32 = nullptr;
     float4 *vp32 = nullptr, *vp32lo = nullptr;
-    float *omT32 = nullptr;                 // branch-major window copies [nb][N]
+    float *omT32 = nullptr, *pnT32 = nullptr;   // branch-major window copies [nb][N]
     float4 *vpT32 = nullptr, *vpTlo = nullptr, *wrange = nullptr, *mode4 = nullptr;
     unsigned *vmask = nullptr;
     int *err = nullptr;
@@ -293,7 +293,7 @@ fc4_status check_ifc(const fc4_ifc *f, int order, int n_atoms, bool required, co
 fc4_status refresh_modes(fc4_ctx *c) {
     FC4_CUDA(c, fc4::launch_mode_tables(c->t, c->om, c->om32, c->om32lo, c->ev32, c->ev, c->vmask,
                                         c->invw, c->invw32, c->vp32, c->vp32lo, c->omT32, c->vpT32, c->vpTlo,
-                                        c->wrange, 0));
+                                        c->pnT32, c->wrange, 0));
     const size_t nm = (size_t)c->t.N * c->t.nb;
     c->om_host.assign(nm, 0.0);
     FC4_CUDA(c, cudaMemcpy(c->om_host.data(), c->om, nm * sizeof(double), cudaMemcpyDeviceToHost));
@@ -844,6 +844,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     FC4_TRY(place(c, &c->omT32, nm));
     FC4_TRY(place(c, &c->vpT32, nm));
     FC4_TRY(place(c, &c->vpTlo, nm));
+    FC4_TRY(place(c, &c->pnT32, nm));
     FC4_TRY(place(c, &c->wrange, (size_t)N));
     FC4_TRY(place(c, &c->mode4, nm));
     FC4_TRY(place(c, &c->err, 1));
@@ -865,6 +866,7 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     t.omT32 = c->omT32;
     t.vpT32 = c->vpT32;
     t.vpTlo = c->vpTlo;
+    t.pnT32 = c->pnT32;
     t.wrange = c->wrange;
     t.mode4 = c->mode4;
     t.occ = c->occ;

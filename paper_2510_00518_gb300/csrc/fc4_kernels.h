@@ -33,6 +33,7 @@ struct Tables {
     const float *omT32;          // ω hi
     const float4 *vpT32;         // P hi
     const float4 *vpTlo;         // P lo
+    const float *pnT32;          // |P|, rounded up by 2^-14
     const float4 *wrange;        // [N] over participating branches: min ω, max ω (FP32 hi parts; +inf, -inf if
                                  // none), max |P| (1 + 2^-14)
     double recip[9];             // reciprocal vectors b_k (rows, 1/Å), a_i . b_k = 2π δ_ik
@@ -172,7 +173,7 @@ cudaError_t launch_harmonic(const Tables &t, int nc2, const int4 *c2_at, const i
 cudaError_t launch_mode_tables(const Tables &t, double *om, float *om32, float *om32lo,
                                float2 *ev32, const double2 *ev, unsigned *vmask, double *invw,
                                float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
-                               float4 *vpTlo, float4 *wrange, cudaStream_t s);
+                               float4 *vpTlo, float *pnT32, float4 *wrange, cudaStream_t s);
 cudaError_t launch_occupations(const Tables &t, double hbar_over_kT, double *occ, float *occ32,
                                float4 *mode4, cudaStream_t s);
 // message returned by fc4_last_error(NULL) (errors of calls without a context)

@@ -74,20 +74,23 @@ __device__ __forceinline__ bool pair_sampled(const RateArgs &a, int m0, int q1, 
     return (z ^ (z >> 31)) < a.sample_threshold;
 }
 
-// Window row of one (q'', λ''') for the four-phonon channels with adaptive σ: bit j'' set iff kept.  thr
-// bounds the window of every pair of the two points, so only the branches of |Δ32| <= thr have their width
-// formed (each lane goes through its own).  The tables are branch-major: neighbouring lanes hold neighbouring
-// points.
+// Window row of one (q'', λ''') for the four-phonon channels with adaptive σ: bit j'' set iff kept.  No
+// width exceeds the one of |P''| + |P'''| (pnT32 is rounded up by 2^-14, the bound's own roundings are a few
+// u), so only the branches within that have their width formed, each lane going through its own (three q of
+// 5x5x4, 4 atoms: 18.5 ms with one bound a point, 17.1 with the branch-major tables below, 15.9 with one
+// bound a pair).  The tables are branch-major: neighbouring lanes hold neighbouring points.
 template <int NB>
 static __device__ __noinline__ unsigned window_adaptive4_row(const Tables &t, const RateArgs &a, int ch, int s2,
                                                              float base32, int m0, int m1, int q2, int q3,
-                                                             int j3, unsigned v2, float thr) {
+                                                             int j3, unsigned v2) {
     const size_t N = t.N, i3 = j3 * N + q3;
     const float w3 = t.omT32[i3];
+    const float wide = a.ad_rhi * a.ad_c32, T3 = wide * t.pnT32[i3];
     unsigned near = 0, keep = 0;
 #pragma unroll
     for (int j2 = 0; j2 < NB; ++j2)
-        near |= (unsigned)(fabsf((base32 + (float)s2 * t.omT32[j2 * N + q2]) - w3) <= thr) << j2;
+        near |= (unsigned)(fabsf((base32 + (float)s2 * t.omT32[j2 * N + q2]) - w3) - T3 <=
+                           fmaf(wide, t.pnT32[j2 * N + q2], a.ad_e0)) << j2;
     near &= v2;
     if (!near) return 0u;
     const float4 h3 = t.vpT32[i3], l3 = t.vpTlo[i3];

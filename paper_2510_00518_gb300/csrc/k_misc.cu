@@ -197,7 +197,7 @@ cudaError_t launch_harmonic(const Tables &t, int nc2, const int4 *c2_at, const i
 __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om, float *om32, float *om32lo,
                                    float2 *ev32, const double2 *ev, double *invw,
                                    float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
-                                   float4 *vpTlo) {
+                                   float4 *vpTlo, float *pnT32) {
     const int N = t.N, nb = t.nb;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nm = (long long)N * nb;
@@ -219,10 +219,11 @@ __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om,
             l[k] = (float)(p - (double)h[k]);
             p2 += p * p;
         }
-        vp32[i] = make_float4(h[0], h[1], h[2], (float)(sqrt(p2) * (1.0 + 0x1p-14)));   // w >= |P|
+        vp32[i] = make_float4(h[0], h[1], h[2], 0.0f);
         vp32lo[i] = make_float4(l[0], l[1], l[2], 0.0f);
         const size_t it = (size_t)j * N + q;                 // branch-major copies
         omT32[it] = (float)w;
+        pnT32[it] = (float)(sqrt(p2) * (1.0 + 0x1p-14));     // >= |P|
         vpT32[it] = make_float4(h[0], h[1], h[2], 0.0f);
         vpTlo[it] = make_float4(l[0], l[1], l[2], 0.0f);
     }
@@ -234,7 +235,7 @@ __global__ void mode_tables_kernel(const __grid_constant__ Tables t, double *om,
 
 // Per point: the branches that take part, their range of ω and the largest |P| (in the kernel above, with its
 // square roots, this held one thread a point: 33 -> 8 us at 8^3).
-__global__ void point_tables_kernel(int N, int nb, const double *__restrict__ om, const float4 *__restrict__ vp32,
+__global__ void point_tables_kernel(int N, int nb, const double *__restrict__ om, const float *__restrict__ pnT32,
                                     unsigned *vmask, float4 *wrange) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
@@ -247,7 +248,7 @@ __global__ void point_tables_kernel(int N, int nb, const double *__restrict__ om
         const float w = (float)wd;
         lo = fminf(lo, w);
         hi = fmaxf(hi, w);
-        pm = fmaxf(pm, vp32[i * nb + j].w);
+        pm = fmaxf(pm, pnT32[(size_t)j * N + i]);
     }
     vmask[i] = m;
     wrange[i] = make_float4(lo, hi, pm, 0.0f);
@@ -256,12 +257,12 @@ __global__ void point_tables_kernel(int N, int nb, const double *__restrict__ om
 cudaError_t launch_mode_tables(const Tables &t, double *om, float *om32, float *om32lo,
                                float2 *ev32, const double2 *ev, unsigned *vmask, double *invw,
                                float *invw32, float4 *vp32, float4 *vp32lo, float *omT32, float4 *vpT32,
-                               float4 *vpTlo, float4 *wrange, cudaStream_t s) {
+                               float4 *vpTlo, float *pnT32, float4 *wrange, cudaStream_t s) {
     const long long n = (long long)t.N * t.nb * t.nb;
     // the first N nb threads hold the FP64 divisions: small blocks spread them over the SMs
     mode_tables_kernel<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(t, om, om32, om32lo, ev32, ev, invw, invw32, vp32,
-                                                                 vp32lo, omT32, vpT32, vpTlo);
-    point_tables_kernel<<<(t.N + 63) / 64, 64, 0, s>>>(t.N, t.nb, om, vp32, vmask, wrange);
+                                                                 vp32lo, omT32, vpT32, vpTlo, pnT32);
+    point_tables_kernel<<<(t.N + 63) / 64, 64, 0, s>>>(t.N, t.nb, om, pnT32, vmask, wrange);
     return cudaGetLastError();
 }
 

@@ -145,7 +145,7 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
     if constexpr (ADA) {
         int n = 0;
         for (int j3 = 0; j3 < NB; ++j3) {
-            mask[j3] = ((v3 >> j3) & 1u) ? window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3, j3, v2, thr) & dom(j3)
+            mask[j3] = ((v3 >> j3) & 1u) ? window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3, j3, v2) & dom(j3)
                                          : 0u;
             n += (mask[j3] != 0);
         }
@@ -191,7 +191,7 @@ __device__ __forceinline__ unsigned window_row(const Tables &t, const RateArgs &
     if ((base32 + lo2) - w3 > thr || (base32 + hi2) - w3 < -thr) return 0u;
     const unsigned dom = tri == 2 ? (2u << j3) - 1u : tri == 3 ? ~((1u << j1) - 1u) : ~0u;
     if constexpr (ADA) {
-        return window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3, j3, v2, thr) & dom;
+        return window_adaptive4_row<NB>(t, a, ch, s2, base32, m0, m1, q2, q3, j3, v2) & dom;
     } else {
         unsigned near = 0;
 #pragma unroll

@@ -255,7 +255,7 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     using C = Cplx<R>;
     constexpr int NB = 3 * NA;
     constexpr bool WARP = sizeof(R) == 8 && !NOCOMP;
-    constexpr bool SPARSE = !ADA && kQPT == qpt_of<ADA>(false) && !NOCOMP;
+    constexpr bool SPARSE = kQPT == qpt_of<ADA>(false) && !NOCOMP;
     const int s1 = (ch == 4) ? -1 : 1;
     const int s2 = (ch == 2) ? 1 : -1;
     const int N = t.N, nk = t.n_keys;
@@ -266,7 +266,7 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     // SPARSE: candidates [kTileQ * NB * kQPT] in the upper half of sQ (entry o is written after candidate
     // o + 127 has been read at the latest, so the two lists never meet)
     unsigned *sC = reinterpret_cast<unsigned *>(sQ) + kTileQ * NB * kQPT;
-    float *s_g = reinterpret_cast<float *>(sQ + kTileQ * NB * kQPT);   // adaptive σ: [NB * NB][kTileQ] widths
+    float *s_g = reinterpret_cast<float *>(sQ + kTileQ * NB * kQPT);   // adaptive +-: [NB * NB][kTileQ] widths
     __shared__ int s_scan[32];
     __shared__ double s_red[(BTE ? 5 : 2) * 32];
     __shared__ long long s_redn[5 * 32];
@@ -342,11 +342,15 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
           for (int qb = 0; qb < cnt; qb += kTileQ * kQPT) {
             int total, n_ent = 0, off = 0;
             if constexpr (SPARSE) {
+                const float wide = a.ad_rhi * a.ad_c32;          // adaptive: upper prefilter bound per unit of |ΔP|
                 // ++, --: few (q'', j') have a pair near the window.  Pass 1 tests every q'' of the round with
                 // cheap bounds and lists the (q'', j') left, in order; pass 2 takes that list one pair per
                 // thread, so the mask work runs on full warps, and lists the entries (all modes of 8^3, ++ and
                 // --: 126.6 -> 121.9 ms on top of the packed mode scalars; with the candidates in shared memory
                 // of their own, which the L1 then lacks, it gained nothing).
+                // Adaptive σ: no width exceeds the one of |P''| + |P'''|, and the pairs within that have theirs
+                // formed in pass 2, one by one.  Two q of 16^3, both channels: 106.4 ms with the 36 widths of
+                // every q'' kept in shared memory, 147 with one bound a q'', 90.0 with one a pair.
                 unsigned cand[kQPT];
                 int n_cand = 0;
 #pragma unroll
@@ -364,7 +368,7 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                     // (FP32 sums are monotonic)
                     const float4 r2 = t.wrange[q2], r3 = t.wrange[q3];
                     const float lo2 = s2 > 0 ? r2.x : -r2.y, hi2 = s2 > 0 ? r2.y : -r2.x;
-                    const float thr = a.hi32;
+                    const float thr = ADA ? fmaf(wide, r2.z + r3.z, a.ad_e0) : a.hi32;
                     unsigned near = 0;
 #pragma unroll
                     for (int j1 = 0; j1 < NB; ++j1)
@@ -377,20 +381,26 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                         w2f[j] = (float)s2 * t.omT32[j * N + q2];   // branch-major: lanes read consecutive q
                         w3f[j] = t.omT32[j * N + q3];
                     }
+                    float T2[NB], T3[NB];                            // a pair's window is at most T2 + T3
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) {
+                        T2[j] = ADA ? fmaf(wide, t.pnT32[j * N + q2], a.ad_e0) : 0.0f;
+                        T3[j] = ADA ? wide * t.pnT32[j * N + q3] : 0.0f;
+                    }
 #pragma unroll 1
                     for (int j1 = 0; j1 < NB; ++j1) {
                         if (!((near >> j1) & 1u)) continue;
                         const float b1 = w0f + (float)s1 * t.om32[q1 * NB + j1];
-                        float mn = thr + 1.0f;
+                        float mn = __int_as_float(0x7f800000);
 #pragma unroll
                         for (int j2 = 0; j2 < NB; ++j2) {
                             const float t2 = b1 + w2f[j2];
-                            float r = fabsf(t2 - w3f[0]);        // six short chains
+                            float r = fabsf(t2 - w3f[0]) - T3[0];     // six short chains
 #pragma unroll
-                            for (int j3 = 1; j3 < NB; ++j3) r = fminf(r, fabsf(t2 - w3f[j3]));
-                            mn = fminf(mn, r);
+                            for (int j3 = 1; j3 < NB; ++j3) r = fminf(r, fabsf(t2 - w3f[j3]) - T3[j3]);
+                            mn = fminf(mn, r - T2[j2]);
                         }
-                        if (!(mn <= thr)) near &= ~(1u << j1);
+                        if (!(mn <= (ADA ? 0.0f : thr))) near &= ~(1u << j1);
                     }
                     cand[k] = near | ((unsigned)tri << 8);
                     n_cand += __popc(near);
@@ -413,21 +423,24 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                         const int q3 = q_index_near(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
                                                     t.mesh[0], t.mesh[1], t.mesh[2]);
                         const unsigned v2 = t.vmask[q2], v3 = t.vmask[q3];
-                        const float thr = a.hi32;
                         const float b = w0f + (float)s1 * t.om32[q1 * NB + j1];
                         unsigned long long near = 0, okm = 0, keep = 0;
-                        float t2[NB];
+                        float t2[NB], T2[NB];
 #pragma unroll
-                        for (int j2 = 0; j2 < NB; ++j2) t2[j2] = b + (float)s2 * t.om32[q2 * NB + j2];
+                        for (int j2 = 0; j2 < NB; ++j2) {
+                            t2[j2] = b + (float)s2 * t.om32[q2 * NB + j2];
+                            T2[j2] = ADA ? fmaf(wide, t.pnT32[j2 * N + q2], a.ad_e0) : a.hi32;
+                        }
                         unsigned row = v2 & ((1u << NB) - 1u);
                         if (tri == 3) row &= ~((1u << j1) - 1u);             // j'' >= j'
 #pragma unroll
                         for (int j3 = 0; j3 < NB; ++j3) {
-                            const float w3 = t.om32[q3 * NB + j3];
+                            const float w3 = t.om32[q3 * NB + j3], T3 = ADA ? wide * t.pnT32[j3 * N + q3] : 0.0f;
                             if ((v3 >> j3) & 1u) okm |= (unsigned long long)row << (NB * j3);
 #pragma unroll
                             for (int j2 = 0; j2 < NB; ++j2)
-                                near |= (unsigned long long)(fabsf(t2[j2] - w3) <= thr) << (NB * j3 + j2);
+                                near |= (unsigned long long)((ADA ? fabsf(t2[j2] - w3) - T3 : fabsf(t2[j2] - w3)) <= T2[j2])
+                                        << (NB * j3 + j2);
                         }
                         near &= okm;
                         while (near) {                           // the few pairs within reach, one by one
@@ -436,8 +449,13 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                             const int j3 = k / NB, j2 = k - j3 * NB;
                             const int m2 = q2 * NB + j2, m3 = q3 * NB + j3;
                             const float ad = fabsf((b + (float)s2 * t.om32[m2]) - t.om32[m3]);
-                            const bool kp = ad <= a.lo32 || window_exact4(ch, w0, t.om[q1 * NB + j1], t.om[m2], t.om[m3],
-                                                                          a.two_sigma);
+                            bool kp;
+                            if constexpr (ADA) {
+                                const int w = window_adaptive32(a, ad, two_sigma32(t, a, m2, m3));
+                                kp = w == 2 || (w == 1 && window_exact_adaptive(t, a, ch, m0, q1 * NB + j1, m2, m3, m2, m3));
+                            } else {
+                                kp = ad <= a.lo32 || window_exact4(ch, w0, t.om[q1 * NB + j1], t.om[m2], t.om[m3], a.two_sigma);
+                            }
                             keep |= (unsigned long long)kp << k;
                         }
                         if (keep) e = ((unsigned long long)ixr << 48) | ((unsigned long long)j1 << 40) |
@@ -952,7 +970,7 @@ template <typename R, int NA, bool ADA, bool BTE = false>
 cudaError_t launch4_tile(const Tables &t, const RateArgs &a, int ch, cudaStream_t s) {
     using C = Cplx<R>;
     const bool dense = ch == 3;
-    const size_t smem = tile_smem_bytes<R, NA>(t, qpt_of<ADA>(dense), ADA);
+    const size_t smem = tile_smem_bytes<R, NA>(t, qpt_of<ADA>(dense), ADA && (dense || a.no_compact));
     auto kern = dense ? rates4_tile_kernel<R, NA, ADA, qpt_of<ADA>(true), BTE>
                       : rates4_tile_kernel<R, NA, ADA, qpt_of<ADA>(false), BTE>;
     if constexpr (sizeof(R) == 4 && !BTE)       // ablation switch: mixed precision only
