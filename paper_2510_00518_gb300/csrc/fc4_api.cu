@@ -43,6 +43,8 @@ thread_local std::string g_init_error;
 
 void fc4::set_host_error(const char *msg) { g_init_error = msg; }
 
+constexpr int kKappaEager = 8, kKappaCaptured = 24;   // scratch slots of the κ kernel
+
 struct fc4_ctx {
     fc4::Tables t{};
     int nc2 = 0, nc3 = 0, nc4 = 0;
@@ -85,8 +87,15 @@ struct fc4_ctx {
     long long *part_n = nullptr, *part_items = nullptr, *part_ent = nullptr;
     long long *part_ev = nullptr, *part_cev = nullptr;
     size_t part_cap = 0;
-    double *kappa_part = nullptr;           // block sums of κ [kKappaBlocks][9]
-    unsigned *kappa_counter = nullptr;      // blocks of the κ kernel that are done (0 between calls)
+    // scratch of the κ kernel, one slot a launch in flight (KappaSlot)
+    double *kappa_part = nullptr;           // [slots][kappa_blocks][9]
+    unsigned *kappa_counter = nullptr;      // [slots] blocks that are done (0 between launches)
+    std::mutex kappa_mu;
+    cudaEvent_t kappa_ev[kKappaEager] = {};
+    unsigned kappa_next = 0;
+    int kappa_n_cap = 0;
+    unsigned long long kappa_cap_id[kKappaCaptured] = {};
+    cudaStream_t kappa_cap_s[kKappaCaptured] = {};
     unsigned long long *stats = nullptr;    // [25] kept, items, entries, evaluated, visited per channel
     long long cand[5] = {0, 0, 0, 0, 0};    // candidates per channel of the last call
     int *modes = nullptr;
@@ -851,9 +860,9 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     FC4_TRY(cudaMemset(c->err, 0, sizeof(int)));
     FC4_TRY(place(c, &c->dev_err, 1));
     FC4_TRY(cudaMemset(c->dev_err, 0, sizeof(int)));
-    FC4_TRY(place(c, &c->kappa_part, 9 * (size_t)fc4::kKappaBlocks));
-    FC4_TRY(place(c, &c->kappa_counter, 1));
-    FC4_TRY(cudaMemset(c->kappa_counter, 0, sizeof(unsigned)));
+    FC4_TRY(place(c, &c->kappa_part, 9 * (size_t)fc4::kappa_blocks(t) * (kKappaEager + kKappaCaptured)));
+    FC4_TRY(place(c, &c->kappa_counter, kKappaEager + kKappaCaptured));
+    FC4_TRY(cudaMemset(c->kappa_counter, 0, sizeof(unsigned) * (kKappaEager + kKappaCaptured)));
     t.om = c->om;
     t.om32 = c->om32;
     t.om32lo = c->om32lo;
@@ -935,6 +944,37 @@ namespace {
 
 // κ's prefactor 1/(N V_cell) with v in Å/ps (x 100 m/s) and 1/Γ in ps (x 1e-12 s): W/(m K)
 double kappa_scale(const fc4_ctx *c) { return 1e4 * 1e-12 / ((double)c->t.N * c->volume * 1e-30); }
+
+// A launch of the κ kernel with a scratch slot of its own: launches of a context may overlap on several
+// streams.  Eager launches take kKappaEager slots in turn, each after the slot's last launch; a captured one
+// takes a slot that its stream keeps for that capture (its launches are in order there) and that is never
+// given to another; when those are used up it runs without scratch, on one block.
+template <typename F>
+cudaError_t with_kappa_slot(fc4_ctx *c, cudaStream_t s, F &&launch) {
+    std::lock_guard<std::mutex> lock(c->kappa_mu);
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &st, &id);
+    if (e != cudaSuccess) return e;
+    const size_t size = 9 * (size_t)fc4::kappa_blocks(c->t);
+    if (st != cudaStreamCaptureStatusNone) {
+        int k = 0;
+        while (k < c->kappa_n_cap && (c->kappa_cap_id[k] != id || c->kappa_cap_s[k] != s)) ++k;
+        if (k == kKappaCaptured) return launch(nullptr, nullptr);
+        if (k == c->kappa_n_cap) {
+            c->kappa_cap_id[k] = id;
+            c->kappa_cap_s[k] = s;
+            ++c->kappa_n_cap;
+        }
+        return launch(c->kappa_part + size * (kKappaEager + k), c->kappa_counter + kKappaEager + k);
+    }
+    const unsigned k = c->kappa_next++ % kKappaEager;
+    if (c->kappa_ev[k]) e = cudaStreamWaitEvent(s, c->kappa_ev[k], 0);
+    else e = cudaEventCreateWithFlags(&c->kappa_ev[k], cudaEventDisableTiming);
+    if (e != cudaSuccess) return e;
+    e = launch(c->kappa_part + size * k, c->kappa_counter + k);
+    return e == cudaSuccess ? cudaEventRecord(c->kappa_ev[k], s) : e;
+}
 
 // Cap of the W scratch in bytes: fc4_set_mode_chunk's, or max(4 GiB, a quarter of the device memory).
 size_t w_cap(const fc4_ctx *c) {
@@ -1149,9 +1189,11 @@ fc4_status fc4_kappa_iterative(fc4_ctx *c, double T_K, int sigma_adaptive, doubl
     if (!c->bte_F32) FC4_CUDA(c, dalloc(c, &c->bte_F32, 3 * nm));
     if (!c->bte_kappa) FC4_CUDA(c, dalloc(c, &c->bte_kappa, 9));
     const double xw = kHbar * 1e12 / (kKb * T_K);
+    auto kappa_F = [&](double *part, unsigned *counter) {
+        return fc4::launch_kappa_F(c->t, xw, kKb, c->bte_F, kappa_scale(c), part, counter, c->bte_kappa, s);
+    };
     FC4_CUDA(c, fc4::launch_bte_update(c->t, gamma, channel_mask, nullptr, c->bte_F, c->bte_F32, s));   // F = v / Γ
-    FC4_CUDA(c, fc4::launch_kappa_F(c->t, xw, kKb, c->bte_F, kappa_scale(c), c->kappa_part, c->kappa_counter,
-                                          c->bte_kappa, s));
+    FC4_CUDA(c, with_kappa_slot(c, s, kappa_F));
     double kp[9], kn[9];
     FC4_CUDA(c, cudaMemcpyAsync(kp, c->bte_kappa, sizeof kp, cudaMemcpyDeviceToHost, s));
     FC4_CUDA(c, cudaStreamSynchronize(s));
@@ -1161,8 +1203,7 @@ fc4_status fc4_kappa_iterative(fc4_ctx *c, double T_K, int sigma_adaptive, doubl
                                    nullptr, stream, c->bte_F, c->bte_delta);
         if (st != FC4_OK) return st;
         FC4_CUDA(c, fc4::launch_bte_update(c->t, gamma, channel_mask, c->bte_delta, c->bte_F, c->bte_F32, s));
-        FC4_CUDA(c, fc4::launch_kappa_F(c->t, xw, kKb, c->bte_F, kappa_scale(c), c->kappa_part, c->kappa_counter,
-                                          c->bte_kappa, s));
+        FC4_CUDA(c, with_kappa_slot(c, s, kappa_F));
         FC4_CUDA(c, cudaMemcpyAsync(kn, c->bte_kappa, sizeof kn, cudaMemcpyDeviceToHost, s));
         FC4_CUDA(c, cudaStreamSynchronize(s));
         double dmax = 0.0, kmax = 0.0;
@@ -1228,8 +1269,10 @@ fc4_status fc4_kappa(fc4_ctx *c, double T_K, const double *gamma, int channel_ma
     if (!gamma || !kappa_out) return fail(c, FC4_ERR_INVALID, "NULL buffer");
     if (channel_mask < 0 || channel_mask > 31) return fail(c, FC4_ERR_INVALID, "channel_mask must be in [0, 31]");
     Timed tm(c, 6, (cudaStream_t)stream);
-    FC4_CUDA(c, fc4::launch_kappa(c->t, kHbar * 1e12 / (kKb * T_K), kKb, gamma, channel_mask, kappa_scale(c),
-                                  c->kappa_part, c->kappa_counter, kappa_out, (cudaStream_t)stream));
+    FC4_CUDA(c, with_kappa_slot(c, (cudaStream_t)stream, [&](double *part, unsigned *counter) {
+        return fc4::launch_kappa(c->t, kHbar * 1e12 / (kKb * T_K), kKb, gamma, channel_mask, kappa_scale(c), part, counter,
+                                 kappa_out, (cudaStream_t)stream);
+    }));
     return FC4_OK;
 }
 
@@ -1480,6 +1523,8 @@ void fc4_destroy(fc4_ctx *c) {
         if (c->ev_a[k]) cudaEventDestroy(c->ev_a[k]);
         if (c->ev_b[k]) cudaEventDestroy(c->ev_b[k]);
     }
+    for (cudaEvent_t e : c->kappa_ev)
+        if (e) cudaEventDestroy(e);
     for (void *p : c->owned) cudaFree(p);
     delete c;
 }

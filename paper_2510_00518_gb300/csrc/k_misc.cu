@@ -433,6 +433,12 @@ kappa_kernel(int nm, const double *om, const double *vel, double x_per_w, double
             for (int b = 0; b < 3; ++b) acc[3 * a + b] += c * v[a] * f[b];
     }
     block_sum_multi<9, 1>(acc, none, s_red, s_none);
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) kappa[k] = acc[k] * scale;
+        return;
+    }
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) part[9 * (size_t)blockIdx.x + k] = acc[k];
@@ -460,14 +466,14 @@ int kappa_blocks(const Tables &t) {
 
 cudaError_t launch_kappa(const Tables &t, double hbar_over_kT, double kB, const double *gamma, int mask,
                          double scale, double *part, unsigned *counter, double *kappa, cudaStream_t s) {
-    kappa_kernel<false><<<kappa_blocks(t), kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, gamma,
+    kappa_kernel<false><<<part ? kappa_blocks(t) : 1, kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, gamma,
                                                                   mask, scale, part, counter, kappa);
     return cudaGetLastError();
 }
 
 cudaError_t launch_kappa_F(const Tables &t, double hbar_over_kT, double kB, const double *F, double scale,
                            double *part, unsigned *counter, double *kappa, cudaStream_t s) {
-    kappa_kernel<true><<<kappa_blocks(t), kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, F, 0,
+    kappa_kernel<true><<<part ? kappa_blocks(t) : 1, kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, F, 0,
                                                                  scale, part, counter, kappa);
     return cudaGetLastError();
 }
