@@ -100,6 +100,8 @@ struct fc4_ctx {
     long long cand[5] = {0, 0, 0, 0, 0};    // candidates per channel of the last call
     int *modes = nullptr;
     size_t modes_cap = 0;
+    unsigned char *hbuf = nullptr;         // H of the FP64 adjoint beside W
+    size_t hbuf_bytes = 0, hbuf_tried = 0;
     void *wbuf = nullptr;                  // W scratch of the tiled 4ph path
     size_t wbuf_bytes = 0;
     int w_s1 = 0;                          // sign s1 of the W held for w_modes (0: none)
@@ -1333,6 +1335,25 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
                 st = ensure_wbuf(c, std::max<size_t>(1, std::min((size_t)nm, w_cap(c) / per_mode)) * per_mode);
                 if (st != FC4_OK) return st;
             }
+            // ++ and +- share W where W and H of all modes fit in the cap; without the memory H replaces W
+            const size_t all = (size_t)nm * per_mode;
+            if ((c->last_mask & 0b01100) == 0b01100 && c->wbuf_bytes >= all && 2 * all <= w_cap(c)) {
+                cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+                if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+                if (cap == cudaStreamCaptureStatusNone && c->hbuf_tried < all) {   // once, and not while capturing
+                    c->hbuf_tried = all;
+                    if (c->hbuf) {
+                        cudaFree(c->hbuf);
+                        c->owned.erase(std::find(c->owned.begin(), c->owned.end(), (void *)c->hbuf));
+                    }
+                    c->hbuf_bytes = dalloc(c, &c->hbuf, all) == cudaSuccess ? all : 0;
+                    if (!c->hbuf_bytes) {
+                        c->hbuf = nullptr;
+                        cudaGetLastError();
+                    }
+                }
+                a.hbuf = c->hbuf_bytes >= all ? c->hbuf : nullptr;
+            }
             a.wbuf = c->wbuf;
             a.wbuf_bytes = c->wbuf_bytes;
             c->w_s1 = 0;                    // the W of the last rates call is overwritten
@@ -1347,6 +1368,7 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
         const double cst = ch < 2 ? unit_c3() / N : unit_c4() / (N * N);
         // 3ph: FP64 always; 4ph: FP64 in an FP64 context, else FP32 (FP64 accumulation of the slices)
         const int fp64 = ch < 2 || c->precision == FC4_FP64;
+        a.w_reuse = ch == 3 && ((c->last_mask >> 2) & 1);
         FC4_CUDA(c, fc4::launch_adjoint(c->t, a, ch, dL_dgamma, cst, c->adj_part, fp64, s));
         c->n_launches += 1;
         if (ch < 2) {

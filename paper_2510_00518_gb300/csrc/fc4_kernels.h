@@ -98,6 +98,7 @@ struct RateArgs {
     int n_part[5];               // partial slots written per mode for each channel (<= N)
     void *wbuf;                  // optional scratch for the tiled 4ph path (W per (λ, q')); may be NULL
     size_t wbuf_bytes;
+    void *hbuf;                  // FP64 adjoint: place for H of every mode (else H replaces W)
     int w_reuse;                 // 1: wbuf already holds W of every mode for this channel's sign s1
     // adaptive broadening: σ of a process from the velocities of the two legs its free partner
     // sum moves together (3ph: λ', λ''; 4ph: λ'', λ'''), σ = s |ΔP| / sqrt(6)

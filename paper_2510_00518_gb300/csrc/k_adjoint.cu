@@ -250,7 +250,8 @@ adj4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
 // the entries (q'', j', kept pairs) of its window, j' by j', and takes them 128 at a time, one per thread:
 // X from W, and per item and process V, Ȳ[cγ] = Σ_j'' G conj(V) e^s2_λ'' and Z[cγ,dδ] += Ȳ[cγ] e*_λ'''(dδ)
 // in the thread's column of shared memory; then the owner of each (r, γδ) adds P_r^s2 Z over the
-// entries of a j' and the unit's H[j'][r][γδ] replaces its W in the buffer.  adj4_fold_kernel owns a
+// entries of a j' into the unit's H[j'][r][γδ], which replaces its W unless there is room for both
+// (++ and +- then share W: 4.4 of 92 ms).  adj4_fold_kernel owns a
 // mode: per q' it forms K_rb[βγδ] = Σ_j' e^s1_λ'(bβ) H_r[j'][γδ] once for all clusters and adds
 // phase_c K_r(c)b(c) to 27 numbers a cluster in registers, and expands them by e_λ(aα) into the mode's
 // gradient slice at the end.
@@ -259,13 +260,14 @@ adj4_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
 // block-per-mode kernel above takes 1020 an item and 220000 a (λ, q')).  Where Φ4 has the leg-exchange
 // symmetry only one process of each swapped pair is evaluated (self-swapped ones with weight 1/2) and
 // sum_slices_kernel adds the gradient of the swapped legs.  κ and its gradient for all modes of a 4^3
-// mesh: 634 ms with the block-per-mode kernels for both orders, 121 ms with these.
+// mesh: 634 ms with the block-per-mode kernels for both orders, 121 ms with these as first built, 95 ms with
+// mirror keys paired, lanes taking their own items and the shared W.
 constexpr int kAdjLd = kAdjThreads + 1;
 
 template <int NA, bool ADA>
 __global__ void __launch_bounds__(kAdjThreads, 2)
 adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int ch, int mode0,
-                 const double *__restrict__ dLdG, double cst, double2 *__restrict__ wall) {
+                 const double *__restrict__ dLdG, double cst, const double2 *wall, double2 *hall) {
     using C = double2;
     constexpr int NB = 3 * NA;
     const int s1 = (ch == 4) ? -1 : 1;
@@ -282,12 +284,13 @@ adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
     const int ms = mode0 + ml;
     const int m0 = a.modes[ms];
     const int q0 = m0 / NB, j0 = m0 - q0 * NB;
-    C *H = wall + (size_t)blockIdx.x * (NB * nk * 9);
+    const C *W = wall + (size_t)blockIdx.x * (NB * nk * 9);
+    C *H = hall + (size_t)blockIdx.x * (NB * nk * 9);              // may be W's own place
     const double gl = dLdG[(size_t)ch * a.n_modes + ms] * cst;
     const unsigned vm1 = t.vmask[q1];
     for (int k = threadIdx.x; k < NB * nk * 9; k += kAdjThreads) {
         const int j = k / (nk * 9), rem = k - j * (nk * 9);
-        sW[k] = paired_value(t.perm4, rem / 9, (const C *)H + j * (nk * 9) + rem % 9, 9);
+        sW[k] = paired_value(t.perm4, rem / 9, W + j * (nk * 9) + rem % 9, 9);
     }
     __syncthreads();                                             // the whole of W is read
     for (int k = threadIdx.x; k < NB * nk * 9; k += kAdjThreads) H[k] = czero<C>();
@@ -670,7 +673,9 @@ static cudaError_t launch_adj4_tile(const Tables &t, const RateArgs &a, int ch, 
     const int chunk = (int)std::min<size_t>(a.wbuf_bytes / per_mode, 0x7fffffffu / (unsigned)t.N);
     if (chunk < 1) return cudaErrorInvalidValue;
     const size_t smem = adj4_tile_smem<NA>(t), fsmem = adj4_fold_smem<NA>(t);
-    double2 *w = reinterpret_cast<double2 *>(a.wbuf);
+    // with a place of its own for H, W stays and +- takes the one of ++ (w_reuse)
+    const bool both = a.hbuf && chunk >= a.n_modes;
+    double2 *w = reinterpret_cast<double2 *>(a.wbuf), *h = both ? reinterpret_cast<double2 *>(a.hbuf) : w;
     cudaError_t e = cudaFuncSetAttribute(adj4_tile_kernel<NA, ADA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(adj4_fold_kernel<NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
@@ -678,10 +683,10 @@ static cudaError_t launch_adj4_tile(const Tables &t, const RateArgs &a, int ch, 
     const int n_out = (27 * t.nc4 + kFoldThreads * kFoldAcc - 1) / (kFoldThreads * kFoldAcc);
     for (int m = 0; m < a.n_modes; m += chunk) {
         const int nm = std::min(chunk, a.n_modes - m);
-        e = launch_w4<double, NA>(t, a, ch, m, nm, s);
+        if (!(both && a.w_reuse)) e = launch_w4<double, NA>(t, a, ch, m, nm, s);
         if (e != cudaSuccess) return e;
-        adj4_tile_kernel<NA, ADA><<<(unsigned)((long long)nm * t.N), kAdjThreads, smem, s>>>(t, a, ch, m, dLdG, cst, w);
-        adj4_fold_kernel<NA><<<dim3(nm, n_out), kFoldThreads, fsmem, s>>>(t, a, ch, m, dLdG, w, part);
+        adj4_tile_kernel<NA, ADA><<<(unsigned)((long long)nm * t.N), kAdjThreads, smem, s>>>(t, a, ch, m, dLdG, cst, w, h);
+        adj4_fold_kernel<NA><<<dim3(nm, n_out), kFoldThreads, fsmem, s>>>(t, a, ch, m, dLdG, h, part);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
