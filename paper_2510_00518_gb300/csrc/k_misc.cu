@@ -401,7 +401,8 @@ __device__ __forceinline__ double gamma_total(const double *gamma, int nm, int m
 // κ_ab = scale Σ_λ C_λ v_a f_b, C = k_B x² n (n + 1), over modes with ω > 0: f = v / Γ over modes with
 // Γ > 0 (RTA), or with FIELD the deviation vector F of the iterative BTE.  Every block writes its nine
 // sums to a slot of part, and the block that finishes last adds the slots in block order, so the
-// result does not depend on the order the blocks run in; the counter wraps to 0 by itself.
+// result does not depend on the order the blocks run in; the counter wraps to 0 by itself.  part and
+// counter belong to the launch until it ends; a launch of one block takes none.
 // Bound: FP64 latency and issue (expm1 and the divides are ~100 FP64 operations a mode, one warp
 // operation per ~19 clocks and SM).  κ and its gradient for the 24576 modes of a 16^3 mesh took 406 us
 // with one block of 256 threads, and take 34 us with blocks of 64 on every SM.

@@ -18,7 +18,7 @@
 // per thread at 9 n_keys + 12 groups each (their T does not fit in registers).  3ph- is evaluated on half of
 // its pairs where Φ3 allows it, and both channels share a launch.  All modes of 12^3 (2 x 9.5e6
 // processes): 359 ms for one block per mode and ~11 processes at a time, 70 ms with a process per thread
-// and 28 ms so; eight atoms, one q of 4^3: 55, 13 and 1.7 ms.
+// and 28 ms so, 23.5 with mirror keys paired; eight atoms, one q of 4^3: 55, 13 and 1.7 ms.
 #include "k_rates3.cuh"
 
 namespace fc4 {

@@ -283,7 +283,8 @@ struct GeneralSmem {
 // of a thread that walks its entries alone.
 // Bound: latency of the item work at 3-4 blocks per SM.  One thread per entry walked its items alone (20
 // entries on 128 threads at 4^3) and formed the window three times: one q point of 4^3 with eight
-// atoms 314 -> 26 ms (three channels), three q points of 5x5x4 with four atoms and adaptive σ 68 -> 24 ms.
+// atoms 314 -> 26 ms (three channels), three q points of 5x5x4 with four atoms and adaptive σ 68 -> 24 ms;
+// with the channels in one launch and the window rows shared out, 23 and 16 ms.
 template <typename R, int NA, bool ADA>
 __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, int ch, int unit) {
     using C = Cplx<R>;

@@ -23,7 +23,8 @@ constexpr int kTileQ = 128;
 // pair widths and the per-process width through the same loops: at 128 registers it spilled
 // (~500 bytes), so it runs 3 blocks per SM (168 registers) with 2 and 1 q'' per round; measured on
 // the 16^3 precision workload this took a 5-q batch from 792 to 614 ms, while the fixed-σ kernels
-// lose 1-3 % with either change.
+// lose 1-3 % with either change (the adaptive ++ and --, which now hold no widths, still take 90 ms so and 97
+// at 4 blocks: two q of 16^3).
 constexpr int kQPTSparse = 4, kQPTDense = 2;
 constexpr int kQPTSparseAd = 2, kQPTDenseAd = 1;
 template <bool ADA> constexpr int qpt_of(bool dense) {
@@ -346,7 +347,7 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
                 // ++, --: few (q'', j') have a pair near the window.  Pass 1 tests every q'' of the round with
                 // cheap bounds and lists the (q'', j') left, in order; pass 2 takes that list one pair per
                 // thread, so the mask work runs on full warps, and lists the entries (all modes of 8^3, ++ and
-                // --: 126.6 -> 121.9 ms on top of the packed mode scalars; with the candidates in shared memory
+                // --: 126.6 -> 121.9 ms on top of the packed mode scalars, 112 with the loops as below; with the candidates in shared memory
                 // of their own, which the L1 then lacks, it gained nothing).
                 // Adaptive σ: no width exceeds the one of |P''| + |P'''|, and the pairs within that have theirs
                 // formed in pass 2, one by one.  Two q of 16^3, both channels: 106.4 ms with the 36 widths of
@@ -646,7 +647,8 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
             // processes of 32 items one per lane (Y by shuffles), since entries carry 1-6 items and items
             // 1-6 processes, and an idle lane costs the FP64 pipe as much as a busy one.  The weights
             // return through shared memory to the lane that owns the entry, which adds them in the
-            // entry's order (4 q points of 8^3: 61.5 -> 52 ms for the three channels).
+            // entry's order (4 q points of 8^3: 61.5 -> 52 ms for the three channels; 43 with mirror keys
+            // paired).
             // FP32: each thread walks its entry's items and processes.  Redistributed as above it was
             // slower (+- of 8^3 314 -> 414 ms; processes only, 16^3: 102 -> 132 ms): shuffles and scans
             // lengthen the chain of each warp, and 3-4 warps per scheduler do not cover it.
