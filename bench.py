@@ -268,8 +268,9 @@ def flops_alg(stats, info, nb, adaptive):
     performs (complex multiply-add = 8 flops, real x complex = 4); where the triangular domain
     applies only the visited candidates and the evaluated processes count:
       window          2 per visited candidate (add, subtract; the comparison is not counted);
-                      adaptive σ adds 12 per visited (q'', j'', j''') pair (one sixth of the
-                      candidates): the velocity difference, its norm and the scale
+                      adaptive +- adds 12 per visited (q'', j'', j''') pair (one sixth of the
+                      candidates): the velocity difference, its norm and the scale (++ and --
+                      form few widths)
       W per (λ, q')   Φ~ = Σ_α Φ e_λ: nc4·27·3·4 / 8 (built once per 8 q'), plus the phase
                       fold Ψ_rb = Σ_c phase Φ~: nc4·27·8, plus W = Σ_bβ e' Ψ: nb·n_keys·9·3na·8
       X per entry     n_keys·9·8 (X[c,d] = Σ_r P_r W_r)
@@ -286,7 +287,7 @@ def flops_alg(stats, info, nb, adaptive):
         na = nb // 3
         w = units * (nc4 * 27 * 3 * 4 / 8.0 + nc4 * 27 * 8 + nb * nk * 9 * na * 3 * 8)
         vis = float(stats["visited"][ch])
-        win = 2.0 * vis + (12.0 * vis / nb if adaptive else 0.0)
+        win = 2.0 * vis + (12.0 * vis / nb if adaptive and ch == 3 else 0.0)
         out.append(win + w + stats["entries"][ch] * nk * 72.0 + stats["items"][ch] * nb * nb * 8.0
                    + stats["evaluated"][ch] * (8.0 * nb + 30.0 + (12.0 if adaptive else 0.0)))
     return out
