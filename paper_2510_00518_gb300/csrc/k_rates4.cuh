@@ -608,7 +608,7 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                                     }
                                 }
                                 const int m3 = q3 * NB + j3;
-                                    while (m) {
+                                while (m) {
                                     const int j2 = __ffs(m) - 1;
                                     m &= m - 1;
                                     C V = czero<C>();
