@@ -115,11 +115,11 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
             total += n;
         }
         __syncthreads();
-        // 32 points to a warp (the first warp differs from block to block: each has its own scheduler's
-        // FP64 pipe); a lane forms its point's T, and the processes of the 32 points go one to a lane
+        // 32 points to a warp (the first warp differs from mode to mode, each has its own scheduler's FP64 pipe;
+        // not from block to block: the order of the sums must not depend on the chunk or the subset); a lane forms its point's T, and the processes of the 32 points go one to a lane
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         unsigned short *wProc = s_proc + wid * 32 * NB * NB;
-        for (int pb = ((wid + blockIdx.x) & 3) * 32; pb < total; pb += kR3Threads) {
+        for (int pb = ((wid + p.m0 + span) & 3) * 32; pb < total; pb += kR3Threads) {
             unsigned long long e = 0;
             int iq1 = 0, iq2 = 0;
             C T[NA][NA][9];

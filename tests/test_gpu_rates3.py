@@ -112,3 +112,24 @@ def test_broken_leg_exchange_takes_the_rectangle():
     e.rates(300.0, 0.3, 3)
     assert e.stats()["evaluated"][1] < st["kept"][1]
     e.close()
+
+
+@pytest.mark.parametrize("atoms", [2, 4])
+def test_bits_do_not_depend_on_the_chunk_or_the_subset(atoms):
+    """Γ and WP of a mode to the bit, whatever modes share its chunk or its call, on a mesh whose points fill
+    several warps of a block."""
+    sysm = morse_system(seed=3) if atoms == 2 else \
+        (lambda c: (c,) + morse_ifcs(c, seed=1))(supercell_crystal(diamond_crystal(), 2, np.linspace(12.0, 90.0, 4)))
+    e = make_engine(sysm, (7, 6, 7), inject=False)
+    ref = [x.cpu().numpy() for x in e.rates(300.0, 0.2, 3)]
+    for chunk in (1, 3, 50):
+        e.set_mode_chunk(chunk, 0)
+        for x, y in zip(e.rates(300.0, 0.2, 3), ref):
+            assert np.array_equal(x.cpu().numpy(), y)
+    e.set_mode_chunk(0, 0)
+    nb = 3 * atoms
+    for q in ([5], [293, 17, 100]):
+        rows = modes_of(q, nb)
+        for x, y in zip(e.rates(300.0, 0.2, 3, q_subset=q), ref):
+            assert np.array_equal(x.cpu().numpy(), y[:, rows])
+    e.close()
