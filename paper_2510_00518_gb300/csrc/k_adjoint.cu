@@ -577,9 +577,9 @@ adj3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
     __syncthreads();
     three_G(t, p, se0, sG);
     for (int k = threadIdx.x; k < nk * 9; k += kR3Threads) sH[k] = czero<C>();
-    auto round = [&](int first, int n) {
+    auto round = [&](int qlo, int first, int n) {
         if ((int)threadIdx.x < n) {
-            const ThreeProcess z = three_evaluate<NA, ADA>(t, a, p, 0, sList[first + threadIdx.x], sG);
+            const ThreeProcess z = three_evaluate<NA, ADA>(t, a, p, qlo, sList[first + threadIdx.x], sG);
             const C f = cmake(gl * z.w * z.V.x, -gl * z.w * z.V.y);                     // G conj(V)
             s_q1[threadIdx.x] = z.q1;
 #pragma unroll 1
@@ -601,13 +601,16 @@ adj3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
         }
         __syncthreads();
     };
-    int queued = 0;
-    for (int qb = 0; qb < N; qb += kR3Threads)
-        for (int jb = 0; jb < NB; jb += JB) {
-            queued = three_append<NB, ADA>(t, a, p, 0, qb, N, jb, queued, sList, s_scan);
-            for (; queued >= kR3Threads; queued -= kR3Threads) round(queued - kR3Threads, kR3Threads);
-        }
-    if (queued) round(0, queued);
+    for (int qlo = 0; qlo < N; qlo += kQueueSpan3) {                // the queue is empty between spans
+        const int qhi = min(N, qlo + kQueueSpan3);
+        int queued = 0;
+        for (int qb = qlo; qb < qhi; qb += kR3Threads)
+            for (int jb = 0; jb < NB; jb += JB) {
+                queued = three_append<NB, ADA>(t, a, p, qlo, qb, qhi, jb, queued, sList, s_scan);
+                for (; queued >= kR3Threads; queued -= kR3Threads) round(qlo, queued - kR3Threads, kR3Threads);
+            }
+        if (queued) round(qlo, 0, queued);
+    }
     for (int r = 0; r < nk; ++r) {
         const int i0 = t.k3_start[r], n = (t.k3_start[r + 1] - i0) * 27;
         for (int k = threadIdx.x; k < n; k += kR3Threads) {

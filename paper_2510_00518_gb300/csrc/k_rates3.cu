@@ -208,6 +208,7 @@ template <int NA, bool ADA>
 __global__ void __launch_bounds__(kR3Threads, 4)
 rates3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int mask, int n_span) {
     constexpr int NB = 3 * NA, JB = jb3(NB), kSpan3 = span3(NB);
+    static_assert(kSpan3 <= kQueueSpan3, "a queued process holds q' - qlo in 16 bits");
     const int ch = channel3(mask);
     const int N = t.N;
     extern __shared__ __align__(16) unsigned char smem[];

@@ -10,6 +10,10 @@ constexpr int kR3Threads = 128;
 // partner branches j' tested per compaction (bounds the queue: kR3Threads * (jb3 * nb + 1) entries)
 constexpr int jb3(int nb) { return nb <= 6 ? nb : nb <= 12 ? 3 : 1; }
 
+// A queued process is one word: q' - qlo in its upper 16 bits, j' and j'' in 8 each.  A queue therefore holds
+// partner points [qlo, qlo + kQueueSpan3) only.
+constexpr int kQueueSpan3 = 1 << 16;
+
 // One mode λ = (q0, j0) and channel sign s: q'' = q + s q'.
 struct Three {
     int ch, s, m0, q0, j0;
@@ -40,7 +44,7 @@ __device__ __forceinline__ void three_G(const Tables &t, const Three &p, const d
     }
 }
 
-// Window of the partner points qb + thread (below qhi) and branches jb .. jb + JB - 1 against every
+// Window of the partner points qb + thread (below qhi <= qlo + kQueueSpan3) and branches jb .. jb + JB - 1 against every
 // j'': the kept processes (q' - qlo, j', j'') are appended in order to sList at queued.  Returns the new
 // length.  Ends with a block barrier.
 template <int NB, bool ADA>
