@@ -105,6 +105,7 @@ struct fc4_ctx {
     void *wbuf = nullptr;                  // W scratch of the tiled 4ph path
     size_t wbuf_bytes = 0;
     int w_s1 = 0;                          // sign s1 of the W held for w_modes (0: none)
+    bool w_captured = false;               // a captured call uses wbuf (note_w_use)
     int mode_chunk = 0;                    // modes per chunk of a rates call (0: as many as W allows)
     size_t w_limit = 0;                    // cap of the W buffer in bytes (0: max(4 GiB, HBM / 4))
     int last_chunk = 0;                    // modes per chunk of the last rates call
@@ -985,12 +986,29 @@ size_t w_cap(const fc4_ctx *c) {
     return c->w_limit ? c->w_limit : std::max<size_t>(4ull << 30, total_b / 4);
 }
 
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();                     // the legacy stream while another one captures
+    return true;
+}
+
+// A call on s is about to use the W scratch.  Replays of a captured call rewrite it without the host knowing, and
+// read it without the host ordering what was there, so from the first captured call on no W is carried from one
+// call to the next (each forms its own, once a sign) and the buffers are not freed before the context.
+void note_w_use(fc4_ctx *c, cudaStream_t s) {
+    if (!c->w_captured) c->w_captured = capturing(s);
+    if (c->w_captured) c->w_s1 = 0;
+}
+
 // Grow the W scratch to at least bytes.
 fc4_status ensure_wbuf(fc4_ctx *c, size_t bytes) {
     if (c->wbuf_bytes >= bytes) return FC4_OK;
     if (c->wbuf) {
-        cudaFree(c->wbuf);
-        c->owned.erase(std::find(c->owned.begin(), c->owned.end(), c->wbuf));
+        if (!c->w_captured) {
+            cudaFree(c->wbuf);
+            c->owned.erase(std::find(c->owned.begin(), c->owned.end(), c->wbuf));
+        }
         c->wbuf = nullptr;
         c->wbuf_bytes = 0;
     }
@@ -1071,6 +1089,7 @@ fc4_status rates_call(fc4_ctx *c, double T_K, int sigma_adaptive, double sigma_v
     if (per_mode) {                         // W scratch of the tiled 4ph path
         const fc4_status sw = ensure_wbuf(c, chunk * per_mode);
         if (sw != FC4_OK) return sw;
+        note_w_use(c, s);
     }
     if (modes != c->modes_on_device) {      // unchanged subsets need no copy (stream capture)
         FC4_CUDA(c, cudaMemcpyAsync(c->modes, modes.data(), nm * sizeof(int), cudaMemcpyHostToDevice, s));
@@ -1338,11 +1357,9 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
             // ++ and +- share W where W and H of all modes fit in the cap; without the memory H replaces W
             const size_t all = (size_t)nm * per_mode;
             if ((c->last_mask & 0b01100) == 0b01100 && c->wbuf_bytes >= all && 2 * all <= w_cap(c)) {
-                cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-                if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
-                if (cap == cudaStreamCaptureStatusNone && c->hbuf_tried < all) {   // once, and not while capturing
+                if (!capturing(s) && c->hbuf_tried < all) {        // once, and not while capturing
                     c->hbuf_tried = all;
-                    if (c->hbuf) {
+                    if (c->hbuf && !c->w_captured) {
                         cudaFree(c->hbuf);
                         c->owned.erase(std::find(c->owned.begin(), c->owned.end(), (void *)c->hbuf));
                     }
@@ -1356,6 +1373,7 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
             }
             a.wbuf = c->wbuf;
             a.wbuf_bytes = c->wbuf_bytes;
+            note_w_use(c, s);
             c->w_s1 = 0;                    // the W of the last rates call is overwritten
         }
     }
