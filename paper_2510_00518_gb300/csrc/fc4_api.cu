@@ -1348,12 +1348,22 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
     set_window(c, a, c->last_adaptive, c->last_sigma);
     // FP64 cells of up to two atoms: the tiled adjoint, in chunks of modes whose W fits in the W scratch
     if (c->precision == FC4_FP64 && dphi4 && c->nc4 && (c->last_mask & 0b11100) && fc4::adj4_tiled(c->t)) {
-        const size_t per_mode = fc4::rates4_wbuf_per_mode(c->t, 1);
+        const size_t per_mode = fc4::rates4_wbuf_per_mode(c->t, 1), units = (size_t)c->t.N;
+        size_t modes = 0;                   // modes per chunk
         if (per_mode) {
-            if (c->wbuf_bytes < per_mode) {
-                st = ensure_wbuf(c, std::max<size_t>(1, std::min((size_t)nm, w_cap(c) / per_mode)) * per_mode);
-                if (st != FC4_OK) return st;
-            }
+            // At least kAdjUnits units a chunk where the cap allows it (half a GB for 34 keys), whatever the rates
+            // took: the fold has a block a mode, and chunks of few modes leave the device idle (all modes of 4^3,
+            // 4ph--: 15 ms in one chunk, 21 in chunks of 64 modes, 89 of 8, 173 of 4, 647 mode by mode).
+            constexpr size_t kAdjUnits = 16384;
+            modes = std::max<size_t>(1, std::min({(size_t)nm, w_cap(c) / per_mode, (kAdjUnits + units - 1) / units}));
+            // without the memory: the general adjoint
+            if (!capturing(s) && ensure_wbuf(c, modes * per_mode) != FC4_OK) cudaGetLastError();
+            modes = std::min((size_t)nm, c->wbuf_bytes / per_mode);
+        }
+        // Where the cap leaves many small chunks, the general adjoint, which takes all modes in one launch, is the
+        // faster one: 118 ms there; all modes of 3^3: 32.6 ms against 19 in chunks of 8 and 36 of 4; 24 q of 6^3: 463
+        // against 370 in chunks of 2 (432 units); all modes of 2^3: 5.5 against 5.4 in 12 chunks of 4.
+        if (modes && (modes >= 8 || modes * units >= 512 || (nm + modes - 1) / modes <= 12)) {
             // ++ and +- share W where W and H of all modes fit in the cap; without the memory H replaces W
             const size_t all = (size_t)nm * per_mode;
             if ((c->last_mask & 0b01100) == 0b01100 && c->wbuf_bytes >= all && 2 * all <= w_cap(c)) {
