@@ -298,17 +298,13 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
         const int b0 = c0.x + s1 * c1.x, b1 = c0.y + s1 * c1.y, b2 = c0.z + s1 * c1.z;
         const double w0 = t.om[m0];
         const float w0f = t.om32[m0];
-        {                                                        // W of (λ, q') for every j'
-            const C *src = wall + (size_t)unit * (NB * nk * 9);
-            if constexpr (sizeof(R) == 8) {
-                for (int k = threadIdx.x; k < NB * nk * 9; k += kTileQ) {
-                    const int j = k / (nk * 9), rem = k - j * (nk * 9);
-                    sW[k] = paired_value(t.perm4, rem / 9, src + j * (nk * 9) + rem % 9, 9);
-                }
-            } else {
-                for (int k = threadIdx.x; k < NB * nk * 9; k += kTileQ) sW[k] = src[k];
-            }
-        }
+        // W of (λ, q') for every j'.  FP64: when the first entry turns up.  Many units of the sparse channels have
+        // none, and with two blocks per SM nothing hides the copy (all modes of 3^3, FP64, ++: 409 -> 249 us, --:
+        // 328 -> 161; two q of 6^3, +-: 1.69 ms either way).
+        const C *src = wall + (size_t)unit * (NB * nk * 9);
+        if constexpr (!WARP)
+            for (int k = threadIdx.x; k < NB * nk * 9; k += kTileQ) sW[k] = src[k];
+        bool have_w = !WARP;
         float base32[NB];
 #pragma unroll
         for (int j = 0; j < NB; ++j) base32[j] = w0f + (float)s1 * t.om32[q1 * NB + j];
@@ -655,6 +651,14 @@ rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
             // The ablation instantiation (NOCOMP, fc4_set_ablation) has each thread evaluate the entries
             // its own window found, as an uncompacted GPU-only loop would.
             if constexpr (WARP) {
+              if (total && !have_w) {
+                for (int k = threadIdx.x; k < NB * nk * 9; k += kTileQ) {
+                    const int j = k / (nk * 9), rem = k - j * (nk * 9);
+                    sW[k] = paired_value(t.perm4, rem / 9, src + j * (nk * 9) + rem % 9, 9);
+                }
+                __syncthreads();
+                have_w = true;
+              }
               const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
               unsigned char *wItem = s_item + wid * 32 * NB;
               unsigned char *wProc = s_proc + wid * 32 * NB;
