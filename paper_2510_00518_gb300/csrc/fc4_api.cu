@@ -43,7 +43,7 @@ thread_local std::string g_init_error;
 
 void fc4::set_host_error(const char *msg) { g_init_error = msg; }
 
-constexpr int kKappaEager = 8, kKappaCaptured = 24;   // scratch slots of the κ kernel
+constexpr int kKappaSlots = 8;          // scratch slots of the κ kernel
 
 struct fc4_ctx {
     fc4::Tables t{};
@@ -87,15 +87,12 @@ struct fc4_ctx {
     long long *part_n = nullptr, *part_items = nullptr, *part_ent = nullptr;
     long long *part_ev = nullptr, *part_cev = nullptr;
     size_t part_cap = 0;
-    // scratch of the κ kernel, one slot a launch in flight (KappaSlot)
+    // scratch of the κ kernel, one slot a launch in flight (with_kappa_slot)
     double *kappa_part = nullptr;           // [slots][kappa_blocks][9]
     unsigned *kappa_counter = nullptr;      // [slots] blocks that are done (0 between launches)
     std::mutex kappa_mu;
-    cudaEvent_t kappa_ev[kKappaEager] = {};
+    cudaEvent_t kappa_ev[kKappaSlots] = {};
     unsigned kappa_next = 0;
-    int kappa_n_cap = 0;
-    unsigned long long kappa_cap_id[kKappaCaptured] = {};
-    cudaStream_t kappa_cap_s[kKappaCaptured] = {};
     unsigned long long *stats = nullptr;    // [25] kept, items, entries, evaluated, visited per channel
     long long cand[5] = {0, 0, 0, 0, 0};    // candidates per channel of the last call
     int *modes = nullptr;
@@ -863,9 +860,9 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     FC4_TRY(cudaMemset(c->err, 0, sizeof(int)));
     FC4_TRY(place(c, &c->dev_err, 1));
     FC4_TRY(cudaMemset(c->dev_err, 0, sizeof(int)));
-    FC4_TRY(place(c, &c->kappa_part, 9 * (size_t)fc4::kappa_blocks(t) * (kKappaEager + kKappaCaptured)));
-    FC4_TRY(place(c, &c->kappa_counter, kKappaEager + kKappaCaptured));
-    FC4_TRY(cudaMemset(c->kappa_counter, 0, sizeof(unsigned) * (kKappaEager + kKappaCaptured)));
+    FC4_TRY(place(c, &c->kappa_part, 9 * (size_t)fc4::kappa_blocks(t) * kKappaSlots));
+    FC4_TRY(place(c, &c->kappa_counter, kKappaSlots));
+    FC4_TRY(cudaMemset(c->kappa_counter, 0, sizeof(unsigned) * kKappaSlots));
     t.om = c->om;
     t.om32 = c->om32;
     t.om32lo = c->om32lo;
@@ -948,30 +945,24 @@ namespace {
 // κ's prefactor 1/(N V_cell) with v in Å/ps (x 100 m/s) and 1/Γ in ps (x 1e-12 s): W/(m K)
 double kappa_scale(const fc4_ctx *c) { return 1e4 * 1e-12 / ((double)c->t.N * c->volume * 1e-30); }
 
-// A launch of the κ kernel with a scratch slot of its own: launches of a context may overlap on several
-// streams.  Eager launches take kKappaEager slots in turn, each after the slot's last launch; a captured one
-// takes a slot that its stream keeps for that capture (its launches are in order there) and that is never
-// given to another; when those are used up it runs without scratch, on one block.
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();                     // the legacy stream while another one captures
+    return true;
+}
+
+// A launch of the κ kernel: launches of a context may overlap on several streams.  Eager ones take kKappaSlots
+// scratch slots in turn, each after the slot's last launch.  Captured ones, and those of few modes, run as one
+// cluster without scratch: executable graphs of one capture may overlap, and a context may be captured any number
+// of times.
 template <typename F>
 cudaError_t with_kappa_slot(fc4_ctx *c, cudaStream_t s, F &&launch) {
+    if (!fc4::kappa_needs_scratch(c->t) || capturing(s)) return launch(nullptr, nullptr);
     std::lock_guard<std::mutex> lock(c->kappa_mu);
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    unsigned long long id = 0;
-    cudaError_t e = cudaStreamGetCaptureInfo(s, &st, &id);
-    if (e != cudaSuccess) return e;
     const size_t size = 9 * (size_t)fc4::kappa_blocks(c->t);
-    if (st != cudaStreamCaptureStatusNone) {
-        int k = 0;
-        while (k < c->kappa_n_cap && (c->kappa_cap_id[k] != id || c->kappa_cap_s[k] != s)) ++k;
-        if (k == kKappaCaptured) return launch(nullptr, nullptr);
-        if (k == c->kappa_n_cap) {
-            c->kappa_cap_id[k] = id;
-            c->kappa_cap_s[k] = s;
-            ++c->kappa_n_cap;
-        }
-        return launch(c->kappa_part + size * (kKappaEager + k), c->kappa_counter + kKappaEager + k);
-    }
-    const unsigned k = c->kappa_next++ % kKappaEager;
+    const unsigned k = c->kappa_next++ % kKappaSlots;
+    cudaError_t e;
     if (c->kappa_ev[k]) e = cudaStreamWaitEvent(s, c->kappa_ev[k], 0);
     else e = cudaEventCreateWithFlags(&c->kappa_ev[k], cudaEventDisableTiming);
     if (e != cudaSuccess) return e;
@@ -984,13 +975,6 @@ size_t w_cap(const fc4_ctx *c) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) total_b = 0;
     return c->w_limit ? c->w_limit : std::max<size_t>(4ull << 30, total_b / 4);
-}
-
-bool capturing(cudaStream_t s) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
-    cudaGetLastError();                     // the legacy stream while another one captures
-    return true;
 }
 
 // A call on s is about to use the W scratch.  Replays of a captured call rewrite it without the host knowing, and

@@ -160,9 +160,11 @@ cudaError_t launch_bte_update(const Tables &t, const double *gamma, int mask, co
                               float *F32, cudaStream_t s);
 cudaError_t launch_to_f32(const double *in, float *out, size_t n, cudaStream_t s);
 // κ from Γ (RTA) or from the field F: part holds 9 doubles for each of kappa_blocks(t) blocks, counter is 0
-// between launches; both belong to one launch at a time (nullptr: one block, no scratch)
+// between launches; both belong to one launch at a time (nullptr, or without kappa_needs_scratch: one cluster,
+// same bits)
 constexpr int kKappaBlocks = 608;      // 4 small blocks on each of 152 SMs
 int kappa_blocks(const Tables &t);
+bool kappa_needs_scratch(const Tables &t);
 cudaError_t launch_kappa_F(const Tables &t, double hbar_over_kT, double kB, const double *F, double scale,
                            double *part, unsigned *counter, double *kappa, cudaStream_t s);
 cudaError_t launch_reduce(const Tables &t, const RateArgs &a, int channel_mask, double c3,

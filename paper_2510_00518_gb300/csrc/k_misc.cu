@@ -1,9 +1,15 @@
 // k_misc.cu - the harmonic prelude (batched FP64 Jacobi eigensolver of D(q), Hellmann-Feynman
 // group velocities), per-mode tables, occupations, key phase tables, the deterministic reduction
 // of per-(λ, q') partials into Γ / WP / counts, the RTA conductivity, and process lists.
+#include <algorithm>
+#include <cooperative_groups.h>
+#include <utility>
+
 #include "fc4_window.cuh"
 
 namespace fc4 {
+
+namespace cg = cooperative_groups;
 
 // ------------------------------------------------------------------------------ harmonic
 
@@ -399,27 +405,21 @@ __device__ __forceinline__ double gamma_total(const double *gamma, int nm, int m
 }
 
 // κ_ab = scale Σ_λ C_λ v_a f_b, C = k_B x² n (n + 1), over modes with ω > 0: f = v / Γ over modes with
-// Γ > 0 (RTA), or with FIELD the deviation vector F of the iterative BTE.  Every block writes its nine
-// sums to a slot of part, and the block that finishes last adds the slots in block order, so the
-// result does not depend on the order the blocks run in; the counter wraps to 0 by itself.  part and
-// counter belong to the launch until it ends; a launch of one block takes none.
+// Γ > 0 (RTA), or with FIELD the deviation vector F of the iterative BTE.  The modes are dealt out to
+// kappa_blocks groups of 64 threads; a group adds its nine sums, and the groups' sums are added in group
+// order, so the result does not depend on the order the groups run in.
 // Bound: FP64 latency and issue (expm1 and the divides are ~100 FP64 operations a mode, one warp
 // operation per ~19 clocks and SM).  κ and its gradient for the 24576 modes of a 16^3 mesh took 406 us
-// with one block of 256 threads, and take 34 us with blocks of 64 on every SM.
+// with one block of 256 threads, and take 34 us with groups of 64 on every SM.
 constexpr int kKappaThreads = 64;
 
+// The sums of one thread of a group, of n_groups.
 template <bool FIELD>
-__global__ void __launch_bounds__(kKappaThreads)
-kappa_kernel(int nm, const double *om, const double *vel, double x_per_w, double kB, const double *src,
-             int mask, double scale, double *part, unsigned *counter, double *kappa) {
-    __shared__ double s_red[9 * 32];
-    __shared__ long long s_none[32];
-    __shared__ bool s_last;
-    double acc[9];
-    long long none[1] = {0};
+__device__ __forceinline__ void kappa_sums(int nm, const double *om, const double *vel, double x_per_w, double kB,
+                                           const double *src, int mask, int group, int thread, int n_groups, double (&acc)[9]) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] = 0.0;
-    for (int i = blockIdx.x * kKappaThreads + threadIdx.x; i < nm; i += gridDim.x * kKappaThreads) {
+    for (int i = group * kKappaThreads + thread; i < nm; i += n_groups * kKappaThreads) {
         const double w = om[i];
         const double g = FIELD ? 1.0 : gamma_total(src, nm, mask, i);
         if (!(w > 0.0) || !(g > 0.0)) continue;
@@ -433,13 +433,21 @@ kappa_kernel(int nm, const double *om, const double *vel, double x_per_w, double
 #pragma unroll
             for (int b = 0; b < 3; ++b) acc[3 * a + b] += c * v[a] * f[b];
     }
+}
+
+// A block per group.  Every block writes its sums to a slot of part, and the block that finishes last adds the
+// slots; the counter wraps to 0 by itself.  part and counter belong to the launch until it ends.
+template <bool FIELD>
+__global__ void __launch_bounds__(kKappaThreads)
+kappa_kernel(int nm, const double *om, const double *vel, double x_per_w, double kB, const double *src,
+             int mask, double scale, double *part, unsigned *counter, double *kappa) {
+    __shared__ double s_red[9 * 32];
+    __shared__ long long s_none[32];
+    __shared__ bool s_last;
+    double acc[9];
+    long long none[1] = {0};
+    kappa_sums<FIELD>(nm, om, vel, x_per_w, kB, src, mask, blockIdx.x, threadIdx.x, gridDim.x, acc);
     block_sum_multi<9, 1>(acc, none, s_red, s_none);
-    if (gridDim.x == 1) {
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int k = 0; k < 9; ++k) kappa[k] = acc[k] * scale;
-        return;
-    }
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) part[9 * (size_t)blockIdx.x + k] = acc[k];
@@ -460,23 +468,107 @@ kappa_kernel(int nm, const double *om, const double *vel, double x_per_w, double
         for (int k = 0; k < 9; ++k) kappa[k] = acc[k] * scale;
 }
 
+// The same sums to the bit by one cluster, without memory outside the launch: the groups are dealt out to the
+// cluster's blocks, at most kKappaBlockGroups at a time, and their sums meet in the first block's shared memory.  For
+// captured calls, whose graphs may be instantiated and replayed side by side at will, and for few groups, where it saves
+// the hand-over between blocks and the events that guard their scratch.
+constexpr int kKappaBlockGroups = 8, kKappaCluster = 16, kKappaFew = 48;
+
+template <bool FIELD>
+__global__ void __launch_bounds__(kKappaThreads * kKappaBlockGroups)
+kappa_cluster_kernel(int nm, int n_groups, const double *om, const double *vel, double x_per_w, double kB, const double *src,
+                     int mask, double scale, double *kappa) {
+    __shared__ double s_part[9 * kKappaBlocks];                 // the first block's is used
+    __shared__ double s_warp[kKappaBlockGroups][2][9];
+    const cg::cluster_group cluster = cg::this_cluster();
+    auto started = cluster.barrier_arrive();
+    const int group = threadIdx.x / kKappaThreads, thread = threadIdx.x % kKappaThreads;
+    const int per = blockDim.x / kKappaThreads, step = cluster.num_blocks() * per;
+    double acc[9];
+    // a group's sums in the order of a block of its own: butterfly, then its two warps
+    auto warp_sums = [&]() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) acc[k] += __shfl_xor_sync(kFull, acc[k], o);
+        if ((thread & 31) == 0)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) s_warp[group][thread >> 5][k] = acc[k];
+    };
+    auto group_sum = [&](int k) { return (0.0 + s_warp[group][0][k]) + s_warp[group][1][k]; };
+    for (int b0 = 0; b0 < n_groups; b0 += step) {
+        const int b = b0 + cluster.block_rank() * per + group;
+        if (b < n_groups) {
+            kappa_sums<FIELD>(nm, om, vel, x_per_w, kB, src, mask, b, thread, n_groups, acc);
+            warp_sums();
+        }
+        if (b0 == 0) cluster.barrier_wait(std::move(started));   // the first block is there
+        __syncthreads();
+        if (b < n_groups && thread < 9) {
+            if (n_groups == 1) kappa[thread] = group_sum(thread) * scale;
+            else cluster.map_shared_rank(s_part, 0)[9 * b + thread] = group_sum(thread);
+        }
+        __syncthreads();
+    }
+    if (n_groups == 1) return;
+    cluster.sync();                                              // every group's sums are there
+    if (cluster.block_rank() != 0 || group != 0) return;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) acc[k] = 0.0;
+    for (int b = thread; b < n_groups; b += kKappaThreads)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[k] += s_part[9 * b + k];
+    warp_sums();
+    asm volatile("bar.sync 1, 64;" ::: "memory");                // the 64 threads of the group
+    if (thread < 9) kappa[thread] = group_sum(thread) * scale;
+}
+
 int kappa_blocks(const Tables &t) {
     const long long b = ((long long)t.N * t.nb + kKappaThreads - 1) / kKappaThreads;
     return (int)(b < kKappaBlocks ? b : kKappaBlocks);
 }
 
+// One cluster up to 48 groups: alone, 162 modes 25 us against 29 with a block per group and 28 with one block of 256
+// threads, 3072 modes (48 groups) 20 against 23 (replays of a graph); 6000 modes (94) 25 against 23.  Captured calls
+// beyond that pay for 16 SMs: 24576 modes 62 against 27 us, one block 407.
+bool kappa_needs_scratch(const Tables &t) { return kappa_blocks(t) > kKappaFew; }
+
+template <bool FIELD>
+static cudaError_t launch_kappa_any(const Tables &t, double hbar_over_kT, double kB, const double *src, int mask,
+                                    double scale, double *part, unsigned *counter, double *kappa, cudaStream_t s) {
+    const int nm = t.N * t.nb, groups = kappa_blocks(t);
+    if (part && kappa_needs_scratch(t)) {
+        kappa_kernel<FIELD><<<groups, kKappaThreads, 0, s>>>(nm, t.om, t.vel, hbar_over_kT, kB, src, mask, scale, part,
+                                                             counter, kappa);
+        return cudaGetLastError();
+    }
+    int blocks = 1;
+    while (blocks < kKappaCluster && blocks < groups) blocks *= 2;
+    const int per = std::min((groups + blocks - 1) / blocks, kKappaBlockGroups);
+    cudaError_t e = cudaFuncSetAttribute(kappa_cluster_kernel<FIELD>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kKappaThreads * per);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kappa_cluster_kernel<FIELD>, nm, groups, t.om, t.vel, hbar_over_kT, kB, src, mask, scale,
+                              kappa);
+}
+
 cudaError_t launch_kappa(const Tables &t, double hbar_over_kT, double kB, const double *gamma, int mask,
                          double scale, double *part, unsigned *counter, double *kappa, cudaStream_t s) {
-    kappa_kernel<false><<<part ? kappa_blocks(t) : 1, kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, gamma,
-                                                                  mask, scale, part, counter, kappa);
-    return cudaGetLastError();
+    return launch_kappa_any<false>(t, hbar_over_kT, kB, gamma, mask, scale, part, counter, kappa, s);
 }
 
 cudaError_t launch_kappa_F(const Tables &t, double hbar_over_kT, double kB, const double *F, double scale,
                            double *part, unsigned *counter, double *kappa, cudaStream_t s) {
-    kappa_kernel<true><<<part ? kappa_blocks(t) : 1, kKappaThreads, 0, s>>>(t.N * t.nb, t.om, t.vel, hbar_over_kT, kB, F, 0,
-                                                                 scale, part, counter, kappa);
-    return cudaGetLastError();
+    return launch_kappa_any<true>(t, hbar_over_kT, kB, F, 0, scale, part, counter, kappa, s);
 }
 
 // dL/dΓ_ch(λ) = Σ_ab dL/dκ_ab dκ_ab/dΓ_tot(λ) = -scale C_λ (v . G v) / Γ_tot² for every channel in
