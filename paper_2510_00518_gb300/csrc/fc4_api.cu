@@ -138,7 +138,10 @@ fc4_status fail(fc4_ctx *ctx, fc4_status s, const std::string &msg) {
     return s;
 }
 
+// The error is reported here: cudaGetLastError takes it away, so that the launch check of the next call does not
+// find it again.
 fc4_status cuda_fail(fc4_ctx *ctx, cudaError_t e, const char *where) {
+    cudaGetLastError();
     return fail(ctx, e == cudaErrorMemoryAllocation ? FC4_ERR_OOM : FC4_ERR_CUDA,
                 std::string(where) + ": " + cudaGetErrorString(e));
 }
@@ -1340,8 +1343,7 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
             // 4ph--: 15 ms in one chunk, 21 in chunks of 64 modes, 89 of 8, 173 of 4, 647 mode by mode).
             constexpr size_t kAdjUnits = 16384;
             modes = std::max<size_t>(1, std::min({(size_t)nm, w_cap(c) / per_mode, (kAdjUnits + units - 1) / units}));
-            // without the memory: the general adjoint
-            if (!capturing(s) && ensure_wbuf(c, modes * per_mode) != FC4_OK) cudaGetLastError();
+            if (!capturing(s)) (void)ensure_wbuf(c, modes * per_mode);      // without the memory: the general adjoint
             modes = std::min((size_t)nm, c->wbuf_bytes / per_mode);
         }
         // Where the cap leaves many small chunks, the general adjoint, which takes all modes in one launch, is the
@@ -1703,9 +1705,11 @@ fc4_status bfail(fc4_batch *b, fc4_status s, const std::string &msg) {
 #define FC4_BCUDA(b, call)                                                                  \
     do {                                                                                    \
         cudaError_t e_ = (call);                                                            \
-        if (e_ != cudaSuccess)                                                              \
+        if (e_ != cudaSuccess) {                                                            \
+            cudaGetLastError();                                                             \
             return bfail((b), e_ == cudaErrorMemoryAllocation ? FC4_ERR_OOM : FC4_ERR_CUDA, \
                          std::string(#call) + ": " + cudaGetErrorString(e_));               \
+        }                                                                                   \
     } while (0)
 
 }  // namespace
