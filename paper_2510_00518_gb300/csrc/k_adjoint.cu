@@ -575,7 +575,7 @@ adj3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
     }
     for (int k = threadIdx.x; k < NB; k += kR3Threads) se0[k] = t.ev[(p.q0 * NB + k) * NB + p.j0];
     __syncthreads();
-    three_G(t, p, se0, sG);
+    three_G<false>(t, p, se0, sG);
     for (int k = threadIdx.x; k < nk * 9; k += kR3Threads) sH[k] = czero<C>();
     auto round = [&](int qlo, int first, int n) {
         if ((int)threadIdx.x < n) {
@@ -606,7 +606,7 @@ adj3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
         int queued = 0;
         for (int qb = qlo; qb < qhi; qb += kR3Threads)
             for (int jb = 0; jb < NB; jb += JB) {
-                queued = three_append<NB, ADA>(t, a, p, qlo, qb, qhi, jb, queued, sList, s_scan);
+                queued = three_append<NB, ADA, JB>(t, a, p, qlo, qb, qhi, jb, queued, sList, s_scan);
                 for (; queued >= kR3Threads; queued -= kR3Threads) round(qlo, queued - kR3Threads, kR3Threads);
             }
         if (queued) round(qlo, 0, queued);

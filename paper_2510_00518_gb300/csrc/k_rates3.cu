@@ -41,7 +41,6 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     const int N = t.N, nk = t.n_keys3;
     extern __shared__ __align__(16) unsigned char smem[];
     C *sG = reinterpret_cast<C *>(smem);                        // [nk][9], in the FP64 key order
-    C *sG0 = sG + nk * 9;                                       // [nk][9], by key
     __shared__ unsigned long long s_list[kSpan3Pair];           // points: q' - qlo, domain code, kept (j', j'')
     __shared__ unsigned short s_proc[kR3Threads * NB * NB];     // per warp: processes (lane, j', j'') of 32 points
     __shared__ C se0[NB];
@@ -61,10 +60,14 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     if (!(p.q0 == 0 && p.j0 < 3)) {
         for (int k = threadIdx.x; k < NB; k += kR3Threads) se0[k] = t.ev[(p.q0 * NB + k) * NB + p.j0];
         __syncthreads();
-        three_G(t, p, se0, sG0);
+        three_G<true>(t, p, se0, sG);
         __syncthreads();
-        for (int k = threadIdx.x; k < nk * 9; k += kR3Threads)     // ordered before its use by the scans' barriers
-            sG[k] = paired_value(t.perm3, k / 9, sG0 + k % 9, 9);
+        for (int k = threadIdx.x; k < nk * 9; k += kR3Threads)     // mirror pairs x, y -> x + y, i (x - y) in place;
+            if (t.perm3[k / 9] >> 28 == 1) {                       // ordered before its use by the scans' barriers
+                const C x = sG[k], y = sG[k + 9];
+                sG[k] = cmake(x.x + y.x, x.y + y.y);
+                sG[k + 9] = cmake(y.y - x.y, x.x - y.x);
+            }
         int total = 0;
         for (int qb = qlo; qb < qhi; qb += kR3Threads) {
             const int q1 = qb + threadIdx.x;
@@ -115,8 +118,9 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
             total += n;
         }
         __syncthreads();
-        // 32 points to a warp (the first warp differs from mode to mode, each has its own scheduler's FP64 pipe;
-        // not from block to block: the order of the sums must not depend on the chunk or the subset); a lane forms its point's T, and the processes of the 32 points go one to a lane
+        // 32 points to a warp: a lane forms its point's T, and the processes of the 32 points go one to a lane.
+        // The first warp differs from mode to mode (each has its own scheduler's FP64 pipe) but not from block to
+        // block: the order of the sums must not depend on the chunk or the subset.
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         unsigned short *wProc = s_proc + wid * 32 * NB * NB;
         for (int pb = ((wid + p.m0 + span) & 3) * 32; pb < total; pb += kR3Threads) {
@@ -204,10 +208,10 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     }
 }
 
-template <int NA, bool ADA>
+template <int NA, bool ADA, int JB>
 __global__ void __launch_bounds__(kR3Threads, 4)
 rates3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int mask, int n_span) {
-    constexpr int NB = 3 * NA, JB = jb3(NB), kSpan3 = span3(NB);
+    constexpr int NB = 3 * NA, kSpan3 = span3(NB);
     static_assert(kSpan3 <= kQueueSpan3, "a queued process holds q' - qlo in 16 bits");
     const int ch = channel3(mask);
     const int N = t.N;
@@ -228,7 +232,7 @@ rates3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs
     if (!(p.q0 == 0 && p.j0 < 3)) {
         for (int k = threadIdx.x; k < NB; k += kR3Threads) se0[k] = t.ev[(p.q0 * NB + k) * NB + p.j0];
         __syncthreads();
-        three_G(t, p, se0, sG);                // ordered before its use by the first append's barriers
+        three_G<false>(t, p, se0, sG);         // ordered before its use by the first append's barriers
         auto evaluate = [&](int it) {
             const ThreeProcess z = three_evaluate<NA, ADA>(t, a, p, qlo, sList[it], sG);
             const double gp = z.w * (z.V.x * z.V.x + z.V.y * z.V.y);
@@ -245,7 +249,7 @@ rates3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs
         int queued = 0;
         for (int qb = qlo; qb < qhi; qb += kR3Threads)
             for (int jb = 0; jb < NB; jb += JB) {
-                queued = three_append<NB, ADA>(t, a, p, qlo, qb, qhi, jb, queued, sList, s_scan);
+                queued = three_append<NB, ADA, JB>(t, a, p, qlo, qb, qhi, jb, queued, sList, s_scan);
                 if (queued >= kR3Threads) {            // full rounds from the tail; < 128 entries stay
                     for (; queued >= kR3Threads; queued -= kR3Threads)
                         evaluate(queued - kR3Threads + (int)threadIdx.x);
@@ -271,19 +275,30 @@ rates3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs
     }
 }
 
+// The pair kernel serves cells of up to two atoms whose G fits beside its lists (1500 keys); larger lists, and larger
+// cells, take rates3_kernel, with one partner branch a round (a shorter queue) where the G of the usual rounds would
+// not fit (1567 keys for two atoms, 1499 for eight).  Clusters with a key each, two atoms, one q of 5^3, σ 2 THz,
+// cluster by cluster and now: 900 clusters 62.9 and 1.4 ms, 1540 clusters 115.6 and 2.2 ms.
 template <int NA>
 static cudaError_t launch3(const Tables &t, RateArgs &a, int mask, cudaStream_t s) {
-    constexpr int NB = 3 * NA;
-    const int per = NA <= 2 ? kSpan3Pair : span3(NB), n_span = (t.N + per - 1) / per;
+    constexpr int NB = 3 * NA, JB = jb3(NB);
+    constexpr size_t kMost = 227 * 1024, kPairStatic = 16 * 1024, kStatic = 3 * 1024;   // with static shared memory
+    const size_t g = sizeof(double2) * 9 * (size_t)t.n_keys3;
+    auto queue = [](int jb) { return sizeof(unsigned) * (size_t)kR3Threads * (jb * NB + 1); };
+    const bool few = NA <= 2 && g + kPairStatic <= kMost;
+    const int jb = NA <= 2 || g + queue(JB) + kStatic > kMost ? 1 : JB;
+    const int per = few ? kSpan3Pair : span3(NB), n_span = (t.N + per - 1) / per;
     for (int ch = 0; ch < 2; ++ch)
         if ((mask >> ch) & 1) a.n_part[ch] = n_span;
     if (a.n_modes == 0 || !mask) return cudaSuccess;
-    const size_t smem = sizeof(double2) * (size_t)t.n_keys3 * 9 * (NA <= 2 ? 2 : 1) +
-                        (NA <= 2 ? 0 : sizeof(unsigned) * (size_t)kR3Threads * (jb3(NB) * NB + 1));
+    const size_t smem = few ? g : g + queue(jb);
     if ((long long)a.n_modes * n_span > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    void (*kern)(Tables, RateArgs, int, int);
-    if constexpr (NA <= 2) kern = a.adaptive ? rates3_pair_kernel<NA, true> : rates3_pair_kernel<NA, false>;
-    else kern = a.adaptive ? rates3_kernel<NA, true> : rates3_kernel<NA, false>;
+    void (*kern)(Tables, RateArgs, int, int) = a.adaptive ? rates3_kernel<NA, true, 1> : rates3_kernel<NA, false, 1>;
+    if constexpr (NA <= 2) {
+        if (few) kern = a.adaptive ? rates3_pair_kernel<NA, true> : rates3_pair_kernel<NA, false>;
+    } else if (jb != 1) {
+        kern = a.adaptive ? rates3_kernel<NA, true, JB> : rates3_kernel<NA, false, JB>;
+    }
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<dim3((unsigned)((long long)a.n_modes * n_span), mask == 3 ? 2 : 1), kR3Threads, smem, s>>>(t, a, mask, n_span);

@@ -7,7 +7,7 @@ namespace fc4 {
 
 constexpr int kR3Threads = 128;
 
-// partner branches j' tested per compaction (bounds the queue: kR3Threads * (jb3 * nb + 1) entries)
+// partner branches j' tested per compaction (JB; bounds the queue: kR3Threads * (JB * nb + 1) entries)
 constexpr int jb3(int nb) { return nb <= 6 ? nb : nb <= 12 ? 3 : 1; }
 
 // A queued process is one word: q' - qlo in its upper 16 bits, j' and j'' in 8 each.  A queue therefore holds
@@ -25,11 +25,12 @@ struct Three {
           w0(t.om[m]), w0f(t.om32[m]) {}
 };
 
-// G_r[βγ] = Σ_{clusters in r} exp(-i q.R2) / sqrt(m) Σ_α Φ[αβγ] e_λ(aα) into sG [n_keys3][9];
-// se0: e_λ in shared memory.
+// G_r[βγ] = Σ_{clusters in r} exp(-i q.R2) / sqrt(m) Σ_α Φ[αβγ] e_λ(aα) into sG [n_keys3][9], by key or (PERM) in the
+// FP64 key order; se0: e_λ in shared memory.
+template <bool PERM>
 __device__ __forceinline__ void three_G(const Tables &t, const Three &p, const double2 *se0, double2 *sG) {
     for (int k = threadIdx.x; k < t.n_keys3 * 9; k += kR3Threads) {
-        const int r = k / 9, bg = k - 9 * r;
+        const int bg = k % 9, r = PERM ? t.perm3[k / 9] & kKeyMask : k / 9;
         double2 g = czero<double2>();
         for (int i = t.k3_start[r]; i < t.k3_start[r + 1]; ++i) {
             const int c = t.k3_idx[i], a0 = t.c3_at[c].x;
@@ -47,10 +48,9 @@ __device__ __forceinline__ void three_G(const Tables &t, const Three &p, const d
 // Window of the partner points qb + thread (below qhi <= qlo + kQueueSpan3) and branches jb .. jb + JB - 1 against every
 // j'': the kept processes (q' - qlo, j', j'') are appended in order to sList at queued.  Returns the new
 // length.  Ends with a block barrier.
-template <int NB, bool ADA>
+template <int NB, bool ADA, int JB>
 __device__ __forceinline__ int three_append(const Tables &t, const RateArgs &a, const Three &p, int qlo, int qb,
                                             int qhi, int jb, int queued, unsigned *sList, int *s_scan) {
-    constexpr int JB = jb3(NB);
     const int q1 = qb + threadIdx.x;
     int q2 = 0;
     unsigned v1 = 0, v2 = 0;

@@ -27,3 +27,28 @@ def test_a_refused_call_leaves_no_error_behind():
         with pytest.raises(FC4Error):
             e.rates(300.0, 0.1, 3)
         make_engine(_system(20), (2, 2, 2), inject=False).close()
+
+
+@pytest.mark.parametrize("atoms,n3,mesh,sigma,adaptive", [
+    (2, 900, (3, 2, 3), 1.0, False), (2, 1500, (2, 3, 2), 2.0, False), (2, 1545, (2, 3, 2), 1.0, True),
+    (2, 1600, (2, 3, 2), 2.0, False), (1, 1530, (3, 3, 2), 3.0, False), (4, 1500, (2, 2, 1), 1.0, False)])
+def test_rates_with_many_keys(atoms, n3, mesh, sigma, adaptive):
+    """Against the oracle at the bars of the other three-phonon tests: one copy of G in the pair kernel (to 1500
+    keys), then the kernel of the larger cells, with a short queue at its own limit."""
+    from synth import diamond_crystal, morse_ifcs, supercell_crystal
+    from tests.test_gpu_rates3 import _check
+    if atoms == 2:
+        sysm = _system(n3)
+    elif atoms == 4:
+        c = supercell_crystal(diamond_crystal(), 2, np.linspace(12.0, 90.0, 4))
+        p2, p3, p4 = morse_ifcs(c, seed=1)
+        sysm = c, p2, random_cluster_ifcs(c, 3, n3, seed=5, max_cell=6), p4
+    else:
+        c = supercell_crystal(diamond_crystal(), 1)
+        c.positions, c.masses = c.positions[:1], c.masses[:1]
+        p2 = random_cluster_ifcs(c, 2, 6, seed=1, scale=0.5)
+        p2.atoms = np.concatenate([p2.atoms, [[0, 0]]]).astype(np.int32)
+        p2.cells = np.concatenate([p2.cells, np.zeros((1, 1, 3))]).astype(np.int32)
+        p2.phi = np.concatenate([p2.phi, [np.diag([10.0, 40.0, 160.0]).reshape(-1)]])
+        sysm = c, p2, random_cluster_ifcs(c, 3, n3, seed=5, max_cell=9), random_cluster_ifcs(c, 4, 5, seed=6)
+    _check(sysm, mesh, [1, int(np.prod(mesh)) - 1], sigma, adaptive)
