@@ -674,8 +674,13 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
         int *d_perm, *d_pairs;
         FC4_TRY(upload(c, &d_perm, perm));
         FC4_TRY(upload(c, &d_pairs, pairs));
+        std::vector<int> pos(perm.size());
+        for (size_t k = 0; k < perm.size(); ++k) pos[perm[k] & ((1 << 28) - 1)] = (int)k;
+        int *d_pos;
+        FC4_TRY(upload(c, &d_pos, pos));
         t.perm3 = d_perm;
         t.pairs3 = d_pairs;
+        t.pos3 = d_pos;
         t.k3_start = d_ks;
         t.k3_idx = d_ki;
         t.grp3_start = d_gs;

@@ -56,6 +56,7 @@ struct Tables {
     const int *k3_idx;           // [nc3] clusters grouped by key, ascending within a key
     const int *grp3_start;       // [n_atoms * n_atoms + 1] key range of group b * n_atoms + c
     const int *perm3, *pairs3;   // FP64 order of the keys (see perm4), [n_keys3] and [n_atoms * n_atoms]
+    const int *pos3;             // [n_keys3] place of a key in that order
     const double2 *P3;           // [N][n_keys3] exp(i q.(R1 - R2)) of each key
     // fourth order: clusters sorted by key; keys sorted by (leg-2 atom, leg-3 atom) group
     int nc4, n_keys;

@@ -30,7 +30,7 @@ struct Three {
 template <bool PERM>
 __device__ __forceinline__ void three_G(const Tables &t, const Three &p, const double2 *se0, double2 *sG) {
     for (int k = threadIdx.x; k < t.n_keys3 * 9; k += kR3Threads) {
-        const int bg = k % 9, r = PERM ? t.perm3[k / 9] & kKeyMask : k / 9;
+        const int r = k / 9, bg = k - 9 * r;
         double2 g = czero<double2>();
         for (int i = t.k3_start[r]; i < t.k3_start[r + 1]; ++i) {
             const int c = t.k3_idx[i], a0 = t.c3_at[c].x;
@@ -41,7 +41,7 @@ __device__ __forceinline__ void three_G(const Tables &t, const Three &p, const d
             const double2 ph = cconj(t.rt[phase_index(p.c0, t.c3_r2[c], t.L)]);
             g = cfma(cmake(ph.x * t.c3_ism[c], ph.y * t.c3_ism[c]), v, g);
         }
-        sG[k] = g;
+        sG[PERM ? 9 * t.pos3[r] + bg : k] = g;
     }
 }
 
