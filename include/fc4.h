@@ -249,7 +249,8 @@ fc4_status fc4_kappa_backward(fc4_ctx *ctx, double T_K, const double *gamma, int
  * Deterministic (fixed summation order).  dL_dgamma: device [5][n_q*nb]; dphi3: device
  * [nc3][27]; dphi4: device [nc4][81], in the cluster order given to fc4_init (overwritten;
  * either may be NULL to skip that order).  Cells of at most 4 atoms.  Returns FC4_ERR_STATE
- * before any fc4_rates call.  Scratch: n_q*nb*max(27 nc3, 81 nc4) doubles (grown on demand); in an
+ * before any fc4_rates call.  Scratch: n_q*nb*max(27 nc3, 81 nc4) doubles (grown on demand), and
+ * n_q*nb*36 doubles a Φ3 key (atoms of legs 1 and 2, R1 - R2) where there are more than ~560 keys; in an
  * FC4_FP64 context with a cell of at most 2 atoms also the W scratch of the rates (so the next
  * fc4_rates forms its W anew) and, where twice W of all modes fits its bound, as much again. */
 fc4_status fc4_rates_backward(fc4_ctx *ctx, const double *dL_dgamma, double *dphi3,

@@ -1316,7 +1316,10 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
     if (nm == 0) return FC4_OK;
     if (!dL_dgamma) return fail(c, FC4_ERR_INVALID, "dL_dgamma is NULL");
     const size_t width = std::max<size_t>(27 * (size_t)c->nc3, 81 * (size_t)c->nc4);
-    const size_t need = (size_t)nm * std::max<size_t>(width, 1);
+    const size_t slices = (size_t)nm * std::max<size_t>(width, 1);      // doubles; G and H of the 3ph keys follow
+    const bool three = dphi3 && c->nc3 && (c->last_mask & 3);
+    const size_t gh3 = three ? fc4::adj3_scratch_per_mode(c->t) : 0, gh3_at = (slices + 1) & ~(size_t)1;
+    const size_t need = gh3 ? gh3_at + (size_t)nm * (gh3 / sizeof(double)) : slices;
     if (need > c->adj_cap) {
         if (c->adj_part) {
             cudaFree(c->adj_part);
@@ -1337,6 +1340,7 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
     fc4::RateArgs a{};
     a.n_modes = nm;
     a.modes = c->modes;
+    if (gh3) a.gh3 = reinterpret_cast<double2 *>(c->adj_part + gh3_at);
     set_window(c, a, c->last_adaptive, c->last_sigma);
     // FP64 cells of up to two atoms: the tiled adjoint, in chunks of modes whose W fits in the W scratch
     if (c->precision == FC4_FP64 && dphi4 && c->nc4 && (c->last_mask & 0b11100) && fc4::adj4_tiled(c->t)) {

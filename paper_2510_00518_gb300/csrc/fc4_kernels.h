@@ -100,6 +100,7 @@ struct RateArgs {
     void *wbuf;                  // optional scratch for the tiled 4ph path (W per (λ, q')); may be NULL
     size_t wbuf_bytes;
     void *hbuf;                  // FP64 adjoint: place for H of every mode (else H replaces W)
+    double2 *gh3;                // 3ph adjoint: G and H of every mode, adj3_scratch_per_mode(t) bytes each
     int w_reuse;                 // 1: wbuf already holds W of every mode for this channel's sign s1
     // adaptive broadening: σ of a process from the velocities of the two legs its free partner
     // sum moves together (3ph: λ', λ''; 4ph: λ'', λ'''), σ = s |ΔP| / sqrt(6)
@@ -195,6 +196,8 @@ cudaError_t launch_unpermute(int nc, int width, const int *perm, const double *i
 // the tiled 4ph adjoint (FP64, up to two atoms) runs when a.wbuf is set (W of >= 1 mode); it takes the
 // triangular domain of a.tri, for which the slices are summed with the swapped clusters
 bool adj4_tiled(const Tables &t);
+// device memory of the 3ph adjoint per mode (0: its tables fit in shared memory)
+size_t adj3_scratch_per_mode(const Tables &t);
 // fp64 = 0: the 4ph adjoint in FP32 (slices of FP32 Kahan pairs; sum them with kahan32 = 1)
 cudaError_t launch_adjoint(const Tables &t, const RateArgs &a, int ch, const double *dLdG, double cst,
                            double *part, int fp64, cudaStream_t s);

@@ -551,7 +551,8 @@ adj4_fold_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
 // and the mode's gradient slice is 2 Re(exp(-i q.R2) e_λ(aα) H_r(c)[βγ]) / sqrt(m).
 // Bound: FP64 (966 complex multiply-adds a process for the diamond cell); adding to all 27 nc3 entries
 // process by process took 12.8 ms for the 384 modes of a 4^3 mesh.
-template <int NA, bool ADA>
+// GLOBAL: G and H of more keys than shared memory holds (adj3_scratch_per_mode) lie in a.gh3, a part for each mode.
+template <int NA, bool ADA, bool GLOBAL>
 __global__ void __launch_bounds__(kR3Threads)
 adj3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int ch,
             const double *__restrict__ dLdG, double cst, double *dphi_part) {
@@ -559,9 +560,9 @@ adj3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
     using C = double2;
     const int N = t.N, nc3 = t.nc3, nk = t.n_keys3;
     extern __shared__ __align__(16) unsigned char smem[];
-    C *sG = reinterpret_cast<C *>(smem);                        // [nk][9]
+    C *sG = GLOBAL ? a.gh3 + (size_t)blockIdx.x * (nk * 18) : reinterpret_cast<C *>(smem);   // [nk][9]
     C *sH = sG + nk * 9;                                        // [nk][9]
-    C *sE = sH + nk * 9;                                        // [2 NB][LD] G conj(V) e^s_λ' and e*_λ''
+    C *sE = GLOBAL ? reinterpret_cast<C *>(smem) : sH + nk * 9; // [2 NB][LD] G conj(V) e^s_λ' and e*_λ''
     unsigned *sList = reinterpret_cast<unsigned *>(sE + 2 * NB * LD);
     __shared__ C se0[NB];
     __shared__ int s_scan[32], s_q1[kR3Threads];
@@ -620,6 +621,20 @@ adj3_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a
             dphi[(size_t)c * 27 + abg] = 2.0 * t.c3_ism[c] * z.x;
         }
     }
+}
+
+// Shared memory of the 3ph adjoint beside G and H: the processes of a round and their queue.
+static size_t adj3_lists_smem(int na) {
+    const int nb = 3 * na;
+    return sizeof(double2) * (size_t)2 * nb * (kR3Threads + 1) + sizeof(unsigned) * (size_t)kR3Threads * (jb3(nb) * nb + 1);
+}
+
+// 288 bytes of G and H a key: up to 650 keys (two atoms; four: 565) in shared memory, beyond that in device memory
+// (a block's G and H stay in L2).  Clusters with a key each, one q, cluster by cluster and now: two atoms, 5^3, 500
+// clusters 44 and 4.1 ms, 700 (in device memory) 62 and 6.0 ms; four atoms, 3^3, 1500 clusters 566 and 74 ms.
+size_t adj3_scratch_per_mode(const Tables &t) {
+    const size_t gh = sizeof(double2) * (size_t)t.n_keys3 * 18;
+    return t.n_atoms <= 4 && gh + adj3_lists_smem(t.n_atoms) > 226 * 1024 ? gh : 0;
 }
 
 // ------------------------------------------------------------------------------ slices -> gradient
@@ -701,10 +716,11 @@ static cudaError_t launch_adj_na(const Tables &t, const RateArgs &a, int ch, con
                                  double *part, int fp64, cudaStream_t s) {
     if (a.n_modes == 0) return cudaSuccess;
     if (ch < 2) {
-        constexpr int NB = 3 * NA;
-        const size_t smem = sizeof(double2) * ((size_t)t.n_keys3 * 18 + 2 * NB * (kR3Threads + 1)) +
-                            sizeof(unsigned) * (size_t)kR3Threads * (jb3(NB) * NB + 1);
-        auto kern = a.adaptive ? adj3_kernel<NA, true> : adj3_kernel<NA, false>;
+        const bool global = adj3_scratch_per_mode(t) != 0;
+        if (global && !a.gh3) return cudaErrorInvalidValue;
+        const size_t gh = sizeof(double2) * (size_t)t.n_keys3 * 18, smem = adj3_lists_smem(NA) + (global ? 0 : gh);
+        auto kern = global ? (a.adaptive ? adj3_kernel<NA, true, true> : adj3_kernel<NA, false, true>)
+                           : (a.adaptive ? adj3_kernel<NA, true, false> : adj3_kernel<NA, false, false>);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         kern<<<a.n_modes, kR3Threads, smem, s>>>(t, a, ch, dLdG, cst, part);

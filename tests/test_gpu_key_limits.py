@@ -52,3 +52,43 @@ def test_rates_with_many_keys(atoms, n3, mesh, sigma, adaptive):
         p2.phi = np.concatenate([p2.phi, [np.diag([10.0, 40.0, 160.0]).reshape(-1)]])
         sysm = c, p2, random_cluster_ifcs(c, 3, n3, seed=5, max_cell=9), random_cluster_ifcs(c, 4, 5, seed=6)
     _check(sysm, mesh, [1, int(np.prod(mesh)) - 1], sigma, adaptive)
+
+
+@pytest.mark.parametrize("atoms,n3,mesh,sigma,adaptive", [
+    (2, 640, (3, 3, 2), 1.0, False), (2, 690, (3, 3, 2), 1.0, False), (2, 1530, (3, 2, 2), 2.0, False),
+    (2, 900, (4, 3, 2), 1.0, True), (4, 700, (2, 2, 1), 1.0, False), (4, 1400, (2, 2, 1), 1.0, False)])
+def test_gradient_with_many_keys(atoms, n3, mesh, sigma, adaptive):
+    """G and H in shared memory and, from 650 (two atoms) or 560 keys (four) on, in device memory.  L is quadratic
+    in Φ3: L(Φ + Φ') - L(Φ - Φ') = 2 <dL/dΦ, Φ'> to the rounding of the two L (1e-10 of each, dL/dΓ > 0; the terms
+    of an L are positive where 1 + n' + n'' weighs them, so 3ph- only)."""
+    from synth import diamond_crystal, morse_ifcs, supercell_crystal
+    if atoms == 2:
+        sysm = _system(n3)
+    else:
+        c = supercell_crystal(diamond_crystal(), 2, np.linspace(12.0, 90.0, 4))
+        p2, p3, p4 = morse_ifcs(c, seed=1)
+        sysm = c, p2, random_cluster_ifcs(c, 3, n3, seed=5, max_cell=6), p4
+    e = make_engine(sysm, mesh, precision=0, inject=False)
+    n, nb = int(np.prod(mesh)), 3 * atoms
+    sub = [1, n - 1]
+    dL = torch.tensor(np.random.default_rng(3).uniform(0.5, 1.5, (5, nb * len(sub))), device="cuda")
+
+    def loss():
+        return float((dL * e.rates(300.0, sigma, 2, q_subset=sub, adaptive=adaptive)[0]).sum())
+
+    assert loss() > 0.0
+    d3 = e.backward(dL)[0].clone()
+    assert torch.equal(d3, e.backward(dL)[0])
+    phi, rng = sysm[2].phi, np.random.default_rng(5)
+    for k in (0, n3 // 2, n3 - 1, None):
+        step = rng.normal(size=phi.shape)
+        if k is not None:
+            step[np.arange(n3) != k] = 0.0
+        L = []
+        for sgn in (1, -1):
+            e.update_anharmonic(phi3=phi + sgn * step)
+            L.append(loss())
+        e.update_anharmonic(phi3=phi)
+        got = float((d3.cpu().numpy() * step).sum())
+        assert abs((L[0] - L[1]) / 2 - got) <= 1e-10 * (abs(L[0]) + abs(L[1])), (k, L, got)
+    e.close()
