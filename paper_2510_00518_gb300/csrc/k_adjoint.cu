@@ -677,11 +677,15 @@ static size_t adj4_fold_smem(const Tables &t) {
     return sizeof(double2) * ((size_t)t.n_keys * NA * 27 + t.nc4 + 9 * NA * NA) + sizeof(int) * (size_t)t.nc4;
 }
 
-// The tiled path serves FP64 cells of up to two atoms whose tables fit in shared memory.
-bool adj4_tiled(const Tables &t) {
+// The tiled path serves FP64 cells of up to two atoms whose tables fit in shared memory, those of its W included.
+template <int NA>
+static bool adj4_fits(const Tables &t) {
     constexpr size_t most = 220 * 1024;
-    if (t.n_atoms == 1) return adj4_tile_smem<1>(t) <= most && adj4_fold_smem<1>(t) <= most;
-    return t.n_atoms == 2 && adj4_tile_smem<2>(t) <= most && adj4_fold_smem<2>(t) <= most;
+    return adj4_tile_smem<NA>(t) <= most && adj4_fold_smem<NA>(t) <= most && w4_smem_bytes<double, NA>(t) <= kW4MostSmem;
+}
+
+bool adj4_tiled(const Tables &t) {
+    return t.n_atoms == 1 ? adj4_fits<1>(t) : t.n_atoms == 2 && adj4_fits<2>(t);
 }
 
 template <int NA, bool ADA>

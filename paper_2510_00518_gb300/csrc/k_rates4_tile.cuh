@@ -941,20 +941,29 @@ size_t tile_w_bytes_per_mode(const Tables &t) {
     return sizeof(Cplx<R>) * (size_t)t.N * 3 * NA * t.n_keys * 9;
 }
 
-// W of the units of modes [m, m + nm) into a.wbuf.
+// Shared memory of w4_kernel.
+template <typename R, int NA>
+size_t w4_smem_bytes(const Tables &t) {
+    constexpr int NB = 3 * NA;
+    return sizeof(Cplx<R>) * ((size_t)t.nc4 * 28 + NB * NB + NB + (size_t)t.n_keys * NA * 27);
+}
+constexpr size_t kW4MostSmem = 227 * 1024;
+
+// W of the units of modes [m, m + nm) into a.wbuf.  FP32 by columns where its tables fit: 240 bytes a cluster and 4 a
+// (key, atom), against 224 and 216 for Ψ in shared memory, so lists of 969 to some 1030 clusters with few keys (36 and
+// fewer) take w4_kernel.
 template <typename R, int NA>
 cudaError_t launch_w4(const Tables &t, const RateArgs &a, int ch, int m, int nm, cudaStream_t s) {
     using C = Cplx<R>;
-    constexpr int NB = 3 * NA;
     C *w = reinterpret_cast<C *>(a.wbuf);
     cudaError_t e;
-    if constexpr (sizeof(R) == 8) {
-        const size_t smem = sizeof(C) * ((size_t)t.nc4 * 28 + NB * NB + NB + (size_t)t.n_keys * NA * 27);
+    if (sizeof(R) == 8 || W4Smem<NA>::bytes(t) > kW4MostSmem) {
+        const size_t smem = w4_smem_bytes<R, NA>(t);
         e = cudaFuncSetAttribute(w4_kernel<R, NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const long long ngrp = (t.N + kW4Group - 1) / kW4Group;
         w4_kernel<R, NA><<<(unsigned)(nm * ngrp), kW4Threads, smem, s>>>(t, a, ch, m, w);
-    } else {
+    } else if constexpr (sizeof(R) == 4) {
         const size_t smem = W4Smem<NA>::bytes(t);
         e = cudaFuncSetAttribute(w4_column_kernel<NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

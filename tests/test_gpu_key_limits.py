@@ -92,3 +92,42 @@ def test_gradient_with_many_keys(atoms, n3, mesh, sigma, adaptive):
         got = float((d3.cpu().numpy() * step).sum())
         assert abs((L[0] - L[1]) / 2 - got) <= 1e-10 * (abs(L[0]) + abs(L[1])), (k, L, got)
     e.close()
+
+
+def _few_keys(n4):
+    """n4 distinct Φ4 clusters, all with legs 2 and 3 in one cell: four keys."""
+    from synth.morse import IFC
+    c, p2, p3, _ = morse_system(seed=3)
+    rng = np.random.default_rng(8)
+    legs = {(*rng.integers(0, 2, 4), *rng.integers(-4, 5, 6)) for _ in range(n4 + 50)}
+    legs = np.array(sorted(tuple(int(x) for x in v) for v in legs)[:n4])
+    cells = np.stack([legs[:, 4:7], legs[:, 7:], legs[:, 7:]], 1)
+    return c, p2, p3, IFC(4, legs[:, :4].astype(np.int32), cells.astype(np.int32), rng.normal(size=(n4, 81)))
+
+
+@pytest.mark.parametrize("n4", [960, 1000, 1028])
+def test_mixed_rates_with_many_clusters_of_few_keys(n4):
+    """W by columns and, from 969 to 1028 clusters of four keys, with Ψ in shared memory, against the general kernel (counts
+    exact, the mixed bar of 1e-4)."""
+    e = make_engine(_few_keys(n4), (3, 3, 2), precision=1, inject=False)
+    assert e.info()["n_keys"] == 4
+    q = [4, 11]
+    g, wp, cnt = (x.cpu().numpy() for x in e.rates(300.0, 0.3, 28, q_subset=q))
+    G, WP, CNT = (x.cpu().numpy() for x in e.rates_static(300.0, 0.3, 28, q))
+    assert CNT.sum() and np.array_equal(cnt, CNT)
+    for x, y in ((g, G), (wp, WP)):
+        assert np.abs(x[2:] - y[2:]).max() <= 1e-4 * np.abs(y[2:]).max()
+    e.close()
+
+
+def test_gradient_where_the_w_of_the_tiled_path_does_not_fit():
+    """600 clusters: mixed rates, then the FP64 gradient of that call; its tiled form would need a W kernel that does
+    not fit, the general one takes it.  Against the mixed gradient (1e-4 of the largest entry)."""
+    e = make_engine(_few_keys(600), (3, 2, 2), precision=1, inject=False)
+    dL = torch.tensor(np.random.default_rng(1).uniform(0.5, 1.5, (5, 6)), device="cuda")
+    e.rates(300.0, 0.3, 28, q_subset=[5])
+    ref = e.backward(dL)[1].clone()
+    e.set_precision(0)
+    got = e.backward(dL)[1]
+    assert (got - ref).abs().max() <= 1e-4 * ref.abs().max()
+    e.close()
