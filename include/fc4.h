@@ -135,7 +135,8 @@ fc4_status fc4_get_modes(fc4_ctx *ctx, double *omega, double *vel, double *evec)
  * fixed (checked on the host to 1e-12 of max |Φ4| at fc4_init and fc4_update_anharmonic).  One
  * process of each swapped pair is evaluated with weight 2; counts and Γ are those of the
  * rectangular sum (Γ to rounding).  The same holds for 3ph- under (λ', λ'') when Φ3 is invariant under
- * exchanging legs 1 and 2 (cells of up to two atoms).
+ * exchanging legs 1 and 2 to rounding (1e-15 of max |Φ3|; cells of up to two atoms).  A list that holds a cluster
+ * twice is summed over the rectangle.
  *
  * T_K > 0.  sigma_adaptive = 0: fixed Gaussian width sigma_value in THz (σ = 2π sigma_value
  * rad/ps).  sigma_adaptive = 1: adaptive width per process from the group velocities of the two

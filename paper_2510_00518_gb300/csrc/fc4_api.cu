@@ -66,8 +66,8 @@ struct fc4_ctx {
     std::vector<int> perm4;                 // device cluster slot -> input cluster index
     std::vector<int> swap12, swap23;        // input cluster -> the cluster with legs 1,2 (2,3) swapped
     std::vector<int> swap12_3;              // third order: the cluster with legs 1, 2 swapped (-1: none)
-    bool sym12_3 = false;                   // Φ3 invariant under that swap (3ph- domain)
-    bool sym12 = false, sym23 = false;      // Φ4 invariant under those swaps (triangular domains)
+    // how far Φ3 and Φ4 are from invariance under those swaps (swap_asymmetry; the domains)
+    double asym12_3 = INFINITY, asym12 = INFINITY, asym23 = INFINITY;
     std::vector<double> om_host;            // current ω (for the prefilter bound)
     double vmax = 0.0;                      // max |v| over modes (adaptive prefilter bound)
     // writable views of the tables
@@ -346,49 +346,45 @@ fc4_status ensure_occupations(fc4_ctx *c, double T, cudaStream_t s) {
     return FC4_OK;
 }
 
-// Leg-swap invariance of Φ4 (input cluster order): every cluster has its partner with legs 1, 2
-// (resp. 2, 3) exchanged, with the correspondingly transposed tensor, to 1e-12 of max |Φ4|.  The
-// triangular domains of the 4ph sums are used only then (a single perturbed entry, as in a
-// finite-difference check of the gradient, falls back to the rectangular sum).
-void check_sym4(fc4_ctx *c, const double *phi) {
-    double mx = 0.0;
-    for (size_t k = 0; k < 81 * (size_t)c->nc4; ++k) mx = std::max(mx, std::fabs(phi[k]));
-    const double tol = 1e-12 * mx;
-    auto ok = [&](const std::vector<int> &sw, bool twelve) {
-        for (int i = 0; i < c->nc4; ++i) {
-            const int j = sw[i];
-            if (j < 0) return false;
-            const double *p = phi + 81 * (size_t)i, *q = phi + 81 * (size_t)j;
-            for (int al = 0; al < 3; ++al)
-                for (int x = 0; x < 3; ++x)
-                    for (int y = 0; y < 3; ++y)
-                        for (int z = 0; z < 3; ++z) {
-                            const double v = p[((al * 3 + x) * 3 + y) * 3 + z];
-                            const double w = twelve ? q[((al * 3 + y) * 3 + x) * 3 + z] : q[((al * 3 + x) * 3 + z) * 3 + y];
-                            if (std::fabs(v - w) > tol) return false;
-                        }
+// Leg-swap asymmetry of Φ of nc clusters (input order; tensors of 3^order entries, swap[i] the cluster with legs
+// l and l + 1 exchanged): the largest difference between an entry and its transposed one, relative to max |Φ|.
+// Infinite where a cluster has no partner of its own (none stored, or a repeated cluster) or an entry is NaN.
+double swap_asymmetry(const double *phi, int nc, int order, int l, const std::vector<int> &swap) {
+    int size = 1, in = 1;                   // entries of a cluster, entries per value of leg l + 1's index
+    for (int k = 0; k < order; ++k) size *= 3;
+    for (int k = l + 2; k < order; ++k) in *= 3;
+    double mx = 0.0, diff = 0.0;
+    for (size_t k = 0; k < (size_t)size * nc; ++k) mx = std::max(mx, std::fabs(phi[k]));
+    for (int i = 0; i < nc; ++i) {
+        const int j = swap[i];
+        if (j < 0 || swap[j] != i) return INFINITY;
+        const double *p = phi + (size_t)size * i, *q = phi + (size_t)size * j;
+        for (int e = 0; e < size; ++e) {
+            const int lo = e % in, y = (e / in) % 3, x = (e / (3 * in)) % 3, hi = e / (9 * in);
+            const double d = std::fabs(p[e] - q[((hi * 3 + y) * 3 + x) * in + lo]);
+            if (std::isnan(d)) return INFINITY;
+            diff = std::max(diff, d);
         }
-        return true;
-    };
-    c->sym12 = ok(c->swap12, true);
-    c->sym23 = ok(c->swap23, false);
+    }
+    return diff == 0.0 ? 0.0 : diff / mx;
 }
 
-// The same for Φ3 and legs 1, 2 (the domain of 3ph-).
-void check_sym3(fc4_ctx *c, const double *phi) {
-    double mx = 0.0;
-    for (size_t k = 0; k < 27 * (size_t)c->nc3; ++k) mx = std::max(mx, std::fabs(phi[k]));
-    c->sym12_3 = true;
-    for (int i = 0; i < c->nc3 && c->sym12_3; ++i) {
-        const int j = c->swap12_3[i];
-        if (j < 0 || c->swap12_3[j] != i) { c->sym12_3 = false; break; }       // (a repeated cluster: no pairing)
-        for (int al = 0; al < 3; ++al)
-            for (int x = 0; x < 3; ++x)
-                for (int y = 0; y < 3; ++y)
-                    if (!(std::fabs(phi[27 * (size_t)i + (al * 3 + x) * 3 + y] - phi[27 * (size_t)j + (al * 3 + y) * 3 + x]) <=
-                          1e-12 * mx))
-                        c->sym12_3 = false;
-    }
+// The domains that Φ4 allows.  The triangular domains of the 4ph rates are used up to an asymmetry of 1e-12 (a single
+// perturbed entry, as in a finite-difference check of the gradient, falls back to the rectangular sum); the gradient
+// and 3ph- were rectangular sums for longer, and use theirs only where the asymmetry is one of rounding: soft
+// modes amplify it (9e-13 of max |Φ3|: 3ph- off by 6e-11 at 8^3, 8e-10 on a 1x1x127 mesh).
+constexpr double kSymmetric4 = 1e-12, kSymmetricRounding = 1e-15;
+
+void check_sym4(fc4_ctx *c, const double *phi) {
+    c->asym12 = swap_asymmetry(phi, c->nc4, 4, 1, c->swap12);
+    c->asym23 = swap_asymmetry(phi, c->nc4, 4, 2, c->swap23);
+}
+
+void check_sym3(fc4_ctx *c, const double *phi) { c->asym12_3 = swap_asymmetry(phi, c->nc3, 3, 1, c->swap12_3); }
+
+// The bits of RateArgs::tri that Φ allows at up to tol of Φ4 (adaptive σ breaks the symmetry in legs 1 and 2).
+int domains(const fc4_ctx *c, bool adaptive, double tol) {
+    return (c->asym23 <= tol ? 1 : 0) | (c->asym12 <= tol && !adaptive ? 2 : 0) | (c->asym12_3 <= kSymmetricRounding ? 4 : 0);
 }
 
 // Prefilter thresholds: |Δ32 - Δ64| <= 13 u ω_max (u = 2^-24; three roundings of the inputs'
@@ -429,7 +425,7 @@ void set_window(const fc4_ctx *c, fc4::RateArgs &a, bool adaptive, double sigma_
     a.spin_limit = c->timeout_cycles;
     a.err = c->dev_err;
     a.n_kernels = const_cast<long long *>(&c->n_launches);
-    a.tri = (c->sym23 ? 1 : 0) | (c->sym12 && !adaptive ? 2 : 0) | (c->sym12_3 ? 4 : 0);
+    a.tri = domains(c, adaptive, kSymmetric4);
     a.no_compact = c->no_compact;
     a.sample_all = c->sample_all;
     a.sample_threshold = c->sample_threshold;
@@ -1378,6 +1374,7 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
             }
             a.wbuf = c->wbuf;
             a.wbuf_bytes = c->wbuf_bytes;
+            a.tri = domains(c, c->last_adaptive, kSymmetricRounding);
             note_w_use(c, s);
             c->w_s1 = 0;                    // the W of the last rates call is overwritten
         }
