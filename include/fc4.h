@@ -258,7 +258,9 @@ fc4_status fc4_rates_backward(fc4_ctx *ctx, const double *dL_dgamma, double *dph
                               double *dphi4, void *stream);
 
 /* fc4_update_anharmonic - replace the Φ3 and/or Φ4 values (host, same cluster lists and layout
- * as fc4_init; NULL keeps the current values).  Modes and phase tables are unchanged. */
+ * as fc4_init; NULL keeps the current values).  Modes and phase tables are unchanged.  Replays of calls
+ * captured before use the new values; four-phonon rates keep the partner domain of their capture (see
+ * fc4_rates), so capture them again after giving up a leg-exchange symmetry of Φ4. */
 fc4_status fc4_update_anharmonic(fc4_ctx *ctx, const double *phi3, const double *phi4);
 
 /* fc4_stats - work counters of the last fc4_rates call (synchronises the device), for channels

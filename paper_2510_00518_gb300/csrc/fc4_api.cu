@@ -68,6 +68,7 @@ struct fc4_ctx {
     std::vector<int> swap12_3;              // third order: the cluster with legs 1, 2 swapped (-1: none)
     // how far Φ3 and Φ4 are from invariance under those swaps (swap_asymmetry; the domains)
     double asym12_3 = INFINITY, asym12 = INFINITY, asym23 = INFINITY;
+    int *domains = nullptr, domains_stored = -1;        // device: Tables::domains
     std::vector<double> om_host;            // current ω (for the prefilter bound)
     double vmax = 0.0;                      // max |v| over modes (adaptive prefilter bound)
     // writable views of the tables
@@ -346,27 +347,37 @@ fc4_status ensure_occupations(fc4_ctx *c, double T, cudaStream_t s) {
     return FC4_OK;
 }
 
+double max_abs(const double *phi, size_t n) {
+    double mx = 0.0;
+    for (size_t k = 0; k < n; ++k) mx = std::max(mx, std::fabs(phi[k]));
+    return mx;
+}
+
 // Leg-swap asymmetry of Φ of nc clusters (input order; tensors of 3^order entries, swap[i] the cluster with legs
-// l and l + 1 exchanged): the largest difference between an entry and its transposed one, relative to max |Φ|.
+// l and l + 1 exchanged): the largest difference between an entry and its transposed one, relative to mx = max |Φ|.
 // Infinite where a cluster has no partner of its own (none stored, or a repeated cluster) or an entry is NaN.
-double swap_asymmetry(const double *phi, int nc, int order, int l, const std::vector<int> &swap) {
+double swap_asymmetry(const double *phi, double mx, int nc, int order, int l, const std::vector<int> &swap) {
     int size = 1, in = 1;                   // entries of a cluster, entries per value of leg l + 1's index
     for (int k = 0; k < order; ++k) size *= 3;
     for (int k = l + 2; k < order; ++k) in *= 3;
-    double mx = 0.0, diff = 0.0;
-    for (size_t k = 0; k < (size_t)size * nc; ++k) mx = std::max(mx, std::fabs(phi[k]));
+    double diff = 0.0;
+    bool nan = false;
     for (int i = 0; i < nc; ++i) {
         const int j = swap[i];
         if (j < 0 || swap[j] != i) return INFINITY;
-        const double *p = phi + (size_t)size * i, *q = phi + (size_t)size * j;
-        for (int e = 0; e < size; ++e) {
-            const int lo = e % in, y = (e / in) % 3, x = (e / (3 * in)) % 3, hi = e / (9 * in);
-            const double d = std::fabs(p[e] - q[((hi * 3 + y) * 3 + x) * in + lo]);
-            if (std::isnan(d)) return INFINITY;
-            diff = std::max(diff, d);
+        if (j < i) continue;                // compared from the other side
+        for (int at = 0; at < size; at += 9 * in) {
+            const double *p = phi + (size_t)size * i + at, *q = phi + (size_t)size * j + at;
+            for (int x = 0; x < 3; ++x)
+                for (int y = 0; y < 3; ++y)
+                    for (int z = 0; z < in; ++z) {
+                        const double d = std::fabs(p[(3 * x + y) * in + z] - q[(3 * y + x) * in + z]);
+                        nan |= d != d;
+                        diff = std::max(diff, d);
+                    }
         }
     }
-    return diff == 0.0 ? 0.0 : diff / mx;
+    return nan ? INFINITY : diff == 0.0 ? 0.0 : diff / mx;
 }
 
 // The domains that Φ4 allows.  The triangular domains of the 4ph rates are used up to an asymmetry of 1e-12 (a single
@@ -376,15 +387,25 @@ double swap_asymmetry(const double *phi, int nc, int order, int l, const std::ve
 constexpr double kSymmetric4 = 1e-12, kSymmetricRounding = 1e-15;
 
 void check_sym4(fc4_ctx *c, const double *phi) {
-    c->asym12 = swap_asymmetry(phi, c->nc4, 4, 1, c->swap12);
-    c->asym23 = swap_asymmetry(phi, c->nc4, 4, 2, c->swap23);
+    const double mx = max_abs(phi, 81 * (size_t)c->nc4);
+    c->asym12 = swap_asymmetry(phi, mx, c->nc4, 4, 1, c->swap12);
+    c->asym23 = swap_asymmetry(phi, mx, c->nc4, 4, 2, c->swap23);
 }
 
-void check_sym3(fc4_ctx *c, const double *phi) { c->asym12_3 = swap_asymmetry(phi, c->nc3, 3, 1, c->swap12_3); }
+void check_sym3(fc4_ctx *c, const double *phi) {
+    c->asym12_3 = swap_asymmetry(phi, max_abs(phi, 27 * (size_t)c->nc3), c->nc3, 3, 1, c->swap12_3);
+}
 
 // The bits of RateArgs::tri that Φ allows at up to tol of Φ4 (adaptive σ breaks the symmetry in legs 1 and 2).
 int domains(const fc4_ctx *c, bool adaptive, double tol) {
     return (c->asym23 <= tol ? 1 : 0) | (c->asym12 <= tol && !adaptive ? 2 : 0) | (c->asym12_3 <= kSymmetricRounding ? 4 : 0);
+}
+
+cudaError_t store_domains(fc4_ctx *c) {
+    const int d = domains(c, false, kSymmetricRounding);
+    if (d == c->domains_stored) return cudaSuccess;
+    c->domains_stored = d;
+    return cudaMemcpy(c->domains, &d, sizeof d, cudaMemcpyHostToDevice);
 }
 
 // Prefilter thresholds: |Δ32 - Δ64| <= 13 u ω_max (u = 2^-24; three roundings of the inputs'
@@ -862,6 +883,9 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     FC4_TRY(place(c, &c->mode4, nm));
     FC4_TRY(place(c, &c->err, 1));
     FC4_TRY(cudaMemset(c->err, 0, sizeof(int)));
+    c->domains_stored = domains(c, false, kSymmetricRounding);
+    FC4_TRY(upload(c, &c->domains, std::vector<int>{c->domains_stored}));
+    t.domains = c->domains;
     FC4_TRY(place(c, &c->dev_err, 1));
     FC4_TRY(cudaMemset(c->dev_err, 0, sizeof(int)));
     FC4_TRY(place(c, &c->kappa_part, 9 * (size_t)fc4::kappa_blocks(t) * kKappaSlots));
@@ -1392,12 +1416,14 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
         FC4_CUDA(c, fc4::launch_adjoint(c->t, a, ch, dL_dgamma, cst, c->adj_part, fp64, s));
         c->n_launches += 1;
         if (ch < 2) {
-            FC4_CUDA(c, fc4::launch_sum_slices(nm, 27 * c->nc3, c->adj_part, dphi3, first3 ? 0 : 1, 0, nullptr, 0, s));
+            FC4_CUDA(c, fc4::launch_sum_slices(nm, 27 * c->nc3, c->adj_part, dphi3, first3 ? 0 : 1, 0, nullptr, 0, nullptr,
+                                               s));
             first3 = false;
         } else {
             const bool swapped = a.wbuf && (a.tri & (ch == 3 ? 1 : 2));
             FC4_CUDA(c, fc4::launch_sum_slices(nm, 81 * c->nc4, c->adj_part, c->adj_tmp, first4 ? 0 : 1, !fp64,
-                                               !swapped ? nullptr : ch == 3 ? c->swap23_dev : c->swap12_dev, ch != 3, s));
+                                               !swapped ? nullptr : ch == 3 ? c->swap23_dev : c->swap12_dev, ch != 3,
+                                               c->t.domains, s));
             first4 = false;
         }
         c->n_launches += 1;
@@ -1428,6 +1454,7 @@ fc4_status fc4_update_anharmonic(fc4_ctx *c, const double *phi3, const double *p
         FC4_CUDA(c, cudaMemcpy(c->phi4, ph.data(), ph.size() * sizeof(double), cudaMemcpyHostToDevice));
         FC4_CUDA(c, cudaMemcpy(c->phi4_32, ph32.data(), ph32.size() * sizeof(float), cudaMemcpyHostToDevice));
     }
+    FC4_CUDA(c, store_domains(c));
     return FC4_OK;
 }
 

@@ -15,6 +15,8 @@ constexpr double kAdaptiveSigmaMin = 1e-9;           // rad/ps: adaptive widths 
 struct Tables {
     int n_atoms, nb, N, L;
     int mesh[3];
+    const int *domains;          // bits of RateArgs::tri that the present Φ allows 3ph- and the FP64 gradient: replays of a
+                                 // captured launch find them as they are then
     // mesh
     const int4 *qc;              // [N] integer coordinates (i1, i2, i3, 0)
     const double2 *rt;           // [L] exp(2πi k / L)
@@ -202,7 +204,7 @@ size_t adj3_scratch_per_mode(const Tables &t);
 cudaError_t launch_adjoint(const Tables &t, const RateArgs &a, int ch, const double *dLdG, double cst,
                            double *part, int fp64, cudaStream_t s);
 cudaError_t launch_sum_slices(int n_slices, int n, const double *part, double *out, int accumulate,
-                              int kahan32, const int *swap, int twelve, cudaStream_t s);
+                              int kahan32, const int *swap, int twelve, const int *domains, cudaStream_t s);
 cudaError_t launch_count_processes(const Tables &t, const RateArgs &a, int ch, int mode, int *counts,
                                    cudaStream_t s);
 cudaError_t launch_write_processes(const Tables &t, const RateArgs &a, int ch, int mode,

@@ -273,6 +273,7 @@ adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
     const int s1 = (ch == 4) ? -1 : 1;
     const int s2 = (ch == 2) ? 1 : -1;
     const int N = t.N, nk = t.n_keys;
+    const int domains = a.tri & *t.domains;
     extern __shared__ __align__(16) unsigned char smem[];
     C *sW = reinterpret_cast<C *>(smem);                        // [NB][nk][9]
     C *sZ = sW + NB * nk * 9;                                   // [NB * NB][kAdjLd]
@@ -311,14 +312,14 @@ adj4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
         if (q2 < N) {
             const int4 c2 = t.qc[q2];
             const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z, t.mesh[0], t.mesh[1], t.mesh[2]);
-            const int tri = tri_code(a, ch, q1, q2, q3);
+            const int tri = tri_code(domains, ch, q1, q2, q3);
             if (tri >= 0)
 #pragma unroll
                 for (int j1 = 0; j1 < NB; ++j1) {
                     if (!((vm1 >> j1) & 1u)) continue;
                     const int m1 = q1 * NB + j1;
                     unsigned mask[NB];
-                    if (window_masks<NB, ADA>(t, a, ch, s2, w0f + (float)s1 * t.om32[m1], m0, m1, w0, t.om[m1], q2, q3,
+                    if (window_masks<NB, ADA>(t, a, domains, ch, s2, w0f + (float)s1 * t.om32[m1], m0, m1, w0, t.om[m1], q2, q3,
                                               mask) == 0)
                         continue;
                     unsigned long long e = ((unsigned long long)threadIdx.x << 48) | ((unsigned long long)j1 << 40) |
@@ -639,10 +640,10 @@ size_t adj3_scratch_per_mode(const Tables &t) {
 
 // ------------------------------------------------------------------------------ slices -> gradient
 
-// out (+)= Σ_slices part in slice order; with swap set (Φ4 entries, 81 a cluster) each slice also adds the
-// entry of the cluster with two legs exchanged (twelve: legs 1 and 2, else 2 and 3).
+// out (+)= Σ_slices part in slice order; with swap set (Φ4 entries, 81 a cluster), and where Φ4 still has that
+// symmetry, each slice also adds the entry of the cluster with two legs exchanged (twelve: legs 1 and 2, else 2 and 3).
 __global__ void sum_slices_kernel(int n_slices, int n, const double *part, double *out, int accumulate,
-                                  int kahan32, const int *swap, int twelve) {
+                                  int kahan32, const int *swap, int twelve, const int *domains) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     double s = accumulate ? out[k] : 0.0;
@@ -654,7 +655,7 @@ __global__ void sum_slices_kernel(int n_slices, int n, const double *part, doubl
         }
     } else {
         for (int i = 0; i < n_slices; ++i) s += part[(size_t)i * n + k];
-        if (swap) {
+        if (swap && (*domains & (twelve ? 2 : 1))) {
             const int c = k / 81, e = k - 81 * c;
             const int al = e / 27, x = (e / 9) % 3, y = (e / 3) % 3, z = e % 3;
             const int o = 81 * swap[c] + (twelve ? ((al * 3 + y) * 3 + x) * 3 + z : ((al * 3 + x) * 3 + z) * 3 + y);
@@ -761,9 +762,9 @@ cudaError_t launch_adjoint(const Tables &t, const RateArgs &a, int ch, const dou
 }
 
 cudaError_t launch_sum_slices(int n_slices, int n, const double *part, double *out, int accumulate,
-                              int kahan32, const int *swap, int twelve, cudaStream_t s) {
+                              int kahan32, const int *swap, int twelve, const int *domains, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    sum_slices_kernel<<<(n + 63) / 64, 64, 0, s>>>(n_slices, n, part, out, accumulate, kahan32, swap, twelve);
+    sum_slices_kernel<<<(n + 63) / 64, 64, 0, s>>>(n_slices, n, part, out, accumulate, kahan32, swap, twelve, domains);
     return cudaGetLastError();
 }
 

@@ -53,7 +53,7 @@ rates3_pair_kernel(const __grid_constant__ Tables t, const __grid_constant__ Rat
     const int qlo = span * kSpan3Pair, qhi = min(N, qlo + kSpan3Pair);
     const Three p(t, ch, a.modes[ms], NB);
     // 3ph- is symmetric under (λ', λ'') (q' <-> q'' = q - q'): one process of each swapped pair, weight 2
-    const bool tri = ch == 1 && (a.tri & 4);
+    const bool tri = ch == 1 && (a.tri & *t.domains & 4);
     double acc_g = 0.0, acc_wp = 0.0;
     double acc_d[3] = {0.0, 0.0, 0.0};         // iterative BTE (a.part_d set): Σ γ Σ_k s_k ω_k F_k
     long long acc_n = 0, acc_ev = 0, acc_cev = 0;

@@ -90,13 +90,13 @@ __device__ __forceinline__ float delta_comp(float h0, float l0, float h1, float 
 
 // Triangular domain of a (q', q'') pair (partner-swap symmetry of the summand): -1 the pair is the
 // swap of one evaluated elsewhere; 0 no symmetry used (weight 1); 1 weight 2; 2 +- with q'' = q@3@
-// (keep j'' <= j@3@); 3 ++ / -- with q'' = q' (keep j'' >= j').
-__device__ __forceinline__ int tri_code(const RateArgs &a, int ch, int q1, int q2, int q3) {
+// (keep j'' <= j@3@); 3 ++ / -- with q'' = q' (keep j'' >= j').  domains: bits as RateArgs::tri.
+__device__ __forceinline__ int tri_code(int domains, int ch, int q1, int q2, int q3) {
     if (ch == 3) {
-        if (!(a.tri & 1)) return 0;
+        if (!(domains & 1)) return 0;
         return q2 > q3 ? -1 : (q2 < q3 ? 1 : 2);
     }
-    if (!(a.tri & 2)) return 0;
+    if (!(domains & 2)) return 0;
     return q2 < q1 ? -1 : (q2 > q1 ? 1 : 3);
 }
 
@@ -104,13 +104,18 @@ __device__ __forceinline__ int tri_code(const RateArgs &a, int ch, int q1, int q
 // its own pair and, off the diagonal (code 1), for its swapped pair ((λ, q', q@3@) for +-,
 // (λ, q'', q') for ++ and --); it keeps weight 2 when both are in the sample, becomes weight 1
 // (code 0) when one is, and is skipped (-1) when neither is.
-__device__ __forceinline__ int tri_code_sampled(const RateArgs &a, int ch, int m0, int q1, int q2, int q3, int N) {
-    const int tri = tri_code(a, ch, q1, q2, q3);
+__device__ __forceinline__ int tri_code_sampled(const RateArgs &a, int domains, int ch, int m0, int q1, int q2, int q3,
+                                                int N) {
+    const int tri = tri_code(domains, ch, q1, q2, q3);
     if (a.sample_all || tri < 0) return tri;
     const int sa = pair_sampled(a, m0, q1, q2, N) ? 1 : 0;
     if (tri != 1) return sa ? tri : -1;
     const int sb = (ch == 3 ? pair_sampled(a, m0, q1, q3, N) : pair_sampled(a, m0, q2, q1, N)) ? 1 : 0;
     return sa + sb == 2 ? 1 : sa + sb == 1 ? 0 : -1;
+}
+
+__device__ __forceinline__ int tri_code_sampled(const RateArgs &a, int ch, int m0, int q1, int q2, int q3, int N) {
+    return tri_code_sampled(a, a.tri, ch, m0, q1, q2, q3, N);
 }
 
 // weight of an evaluated process: 2 for a swapped pair, 1 on the diagonal or without symmetry
@@ -122,12 +127,12 @@ __device__ __forceinline__ int tri_weight(int tri, int j1, int j2, int j3) {
 // triangular domain).  FP32 prefilter with the proven bound; candidates inside the band are
 // decided by the exact FP64 Δ.
 template <int NB, bool ADA>
-__device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, int ch, int s2,
+__device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, int domains, int ch, int s2,
                                             float base32, int m0, int m1, double w0, double w1, int q2,
                                             int q3, unsigned (&mask)[NB]) {
     const unsigned v2 = t.vmask[q2], v3 = t.vmask[q3];
     const int q1 = m1 / NB, j1 = m1 - q1 * NB;
-    const int tri = tri_code_sampled(a, ch, m0, q1, q2, q3, t.N);
+    const int tri = tri_code_sampled(a, domains, ch, m0, q1, q2, q3, t.N);
     // no pair of the point can reach the window: FP32 sums are monotonic, and no width exceeds the one of
     // |P''| + |P'''|
     const float4 r2 = t.wrange[q2], r3 = t.wrange[q3];
@@ -407,7 +412,7 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                                                t.mesh[0], t.mesh[1], t.mesh[2]);
                         unsigned mask[NB];
                         if (tri_code_sampled(a, ch, m0, q1, q2, q3, N) >= 0) acc_cev += NB * NB;   // visited
-                        if (window_masks<NB, ADA>(t, a, ch, s2, base32, m0, m1, w0, w1, q2, q3, mask) > 0) {
+                        if (window_masks<NB, ADA>(t, a, a.tri, ch, s2, base32, m0, m1, w0, w1, q2, q3, mask) > 0) {
                             unsigned long long e = (unsigned long long)q2 << 40;
 #pragma unroll
                             for (int j3 = 0; j3 < NB; ++j3) e |= (unsigned long long)mask[j3] << (NB * j3);

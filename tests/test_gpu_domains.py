@@ -58,3 +58,31 @@ def test_repeated_cluster_takes_the_rectangle():
     d4 = e.backward(torch.tensor(dL, device="cuda"))[1].cpu().numpy()
     assert_close(d4.reshape(-1), prob.grad(modes_of(q, 6), dL)[1].reshape(-1), 1e-8, floor_frac=1e-9, what="dphi4")
     e.close()
+
+
+@pytest.mark.parametrize("call", ["rates", "static", "backward"])
+def test_replays_after_the_symmetry_is_gone(call):
+    """Captured with symmetric force constants, replayed with ones that are not (and back): as the eager call then,
+    to the bit."""
+    c, p2, p3, p4 = morse_system(seed=3)
+    rng = np.random.default_rng(4)
+    broken = [p.phi + 0.1 * np.abs(p.phi).max() * rng.normal(size=p.phi.shape) for p in (p3, p4)]
+    e = make_engine((c, p2, p3, p4), (3, 3, 3), inject=False)
+    sub = [3, 11, 20]
+    dL = torch.tensor(rng.uniform(0.5, 1.5, (5, 18)), device="cuda")
+    run = {"rates": lambda: e.rates(300.0, 0.3, 3, q_subset=sub),
+           "static": lambda: e.rates_static(300.0, 0.3, 3, sub),
+           "backward": lambda: e.backward(dL)}[call]
+    e.rates(300.0, 0.3, 31, q_subset=sub)
+    run()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="thread_local"):
+        out = run()
+    for phi3, phi4 in (broken, (p3.phi, p4.phi), broken):
+        e.update_anharmonic(phi3, phi4)
+        g.replay()
+        torch.cuda.synchronize()
+        got = [x.clone() for x in out]
+        assert all(torch.equal(x, y) for x, y in zip(got, run()))
+    e.close()
