@@ -99,7 +99,7 @@ struct fc4_ctx {
     int *modes = nullptr;
     size_t modes_cap = 0;
     unsigned char *hbuf = nullptr;         // H of the FP64 adjoint beside W
-    size_t hbuf_bytes = 0, hbuf_tried = 0;
+    size_t hbuf_bytes = 0;
     void *wbuf = nullptr;                  // W scratch of the tiled 4ph path
     size_t wbuf_bytes = 0;
     int w_s1 = 0;                          // sign s1 of the W held for w_modes (0: none)
@@ -1382,8 +1382,10 @@ fc4_status fc4_rates_backward(fc4_ctx *c, const double *dL_dgamma, double *dphi3
             // ++ and +- share W where W and H of all modes fit in the cap; without the memory H replaces W
             const size_t all = (size_t)nm * per_mode;
             if ((c->last_mask & 0b01100) == 0b01100 && c->wbuf_bytes >= all && 2 * all <= w_cap(c)) {
-                if (!capturing(s) && c->hbuf_tried < all) {        // once, and not while capturing
-                    c->hbuf_tried = all;
+                // not while capturing, and only where the memory is there (a smaller H is given back first)
+                size_t free_b = 0, total_b = 0;
+                if (c->hbuf_bytes < all && !capturing(s) && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+                    free_b + (c->w_captured ? 0 : c->hbuf_bytes) > all) {
                     if (c->hbuf && !c->w_captured) {
                         cudaFree(c->hbuf);
                         c->owned.erase(std::find(c->owned.begin(), c->owned.end(), (void *)c->hbuf));

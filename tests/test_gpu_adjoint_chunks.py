@@ -52,3 +52,30 @@ def test_gradient_within_a_capped_scratch(mesh, sub, w_modes):
     assert e.memory()["w_buffer"] <= w_modes * e.memory()["w_per_mode"]
     assert torch.equal(out[0], ref[0])
     assert (out[1] - ref[1]).abs().max() <= 1e-12 * ref[1].abs().max()
+
+
+def test_shared_w_after_memory_was_short():
+    """++ and +- share W where there is memory for H beside it.  A gradient without that memory does without, and the
+    next one with it takes it again; the same bits either way."""
+    e = _engine((8, 8, 8))
+    sub = [7, 100, 200, 300]
+    dL = torch.ones((5, 24), dtype=torch.float64, device="cuda")
+    e.rates(300.0, 0.1, 12, q_subset=sub)
+    e.backward(dL)
+    h = 24 * e.memory()["w_per_mode"]
+    assert e.memory()["w_buffer"] == h
+    ref = e.backward(dL)[1].clone()
+    full = e.memory()["total"]
+    e.close()
+    e = _engine((8, 8, 8))
+    e.rates(300.0, 0.1, 12, q_subset=sub)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - h // 2, dtype=torch.uint8, device="cuda")
+    assert torch.equal(e.backward(dL)[1], ref)
+    assert e.memory()["total"] == full - h
+    del rest
+    torch.cuda.empty_cache()
+    assert torch.equal(e.backward(dL)[1], ref)
+    assert e.memory()["total"] == full
+    e.close()
