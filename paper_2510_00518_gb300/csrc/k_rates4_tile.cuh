@@ -7,9 +7,10 @@
 // against every j' at once (branch-free FP32 prefilter, rare ambiguous candidates decided by the
 // exact FP64 Δ), compacts the (q'', j', masks) entries with a block scan, and evaluates them:
 //   X[c,d][γδ] = Σ_{r in (c,d)} P_r^s2 W_r[γδ] once per entry, Y = X e*''' per j''' (36 MACs).
-// FP64 holds X too (2 blocks of 255 registers per SM): its pipe issues a warp operation every ~19
-// clocks and SM, so what counts is the 198 + 36 items complex multiply-adds of an entry (306 + 36 items
-// without the pairing of mirror keys), against 408 an item key by key.
+// FP64 holds X too (2 blocks of 255 registers per SM; with one atom, whose X is a quarter, 3 blocks: all modes of
+// 3^3, ++, 149 -> 110 us): its pipe issues a warp operation every ~19 clocks and SM, so what counts is the
+// 198 + 36 items complex multiply-adds of an entry (306 + 36 items without the pairing of mirror keys), against
+// 408 an item key by key.
 // The same window decision, weights and accumulation as the general kernel (k_rates4.cuh).
 #pragma once
 #include "k_rates4.cuh"
@@ -250,7 +251,7 @@ w4_column_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateA
 //   Δ_λ = Σ_p γ_p Σ_k s_k (ω_k / ω_λ) F_k  (partner signs: ++ (-, -, +), +- (-, +, +), -- (+, +, +)),
 // into a.part_d; the partner combination is symmetric under the swap the triangular domain uses.
 template <typename R, int NA, bool ADA, int kQPT, bool BTE = false, bool NOCOMP = false>
-__global__ void __launch_bounds__(kTileQ, sizeof(R) == 8 ? 2 : ADA ? 3 : 4)
+__global__ void __launch_bounds__(kTileQ, sizeof(R) == 8 ? (NA == 1 ? 3 : 2) : ADA ? 3 : 4)
 rates4_tile_kernel(const __grid_constant__ Tables t, const __grid_constant__ RateArgs a, int ch,
                    int mode0, const Cplx<R> *__restrict__ wall) {
     using C = Cplx<R>;

@@ -40,3 +40,20 @@ def test_window_without_entries_costs_no_w():
         e.close()
     print("ms", t)
     assert t[0] <= 2.0 * t[1], t
+
+
+@pytest.mark.parametrize("mesh,sigma,adaptive", [((3, 3, 3), 0.1, False), ((5, 4, 3), 1.0, True)])
+def test_one_atom(mesh, sigma, adaptive):
+    """Cells of one atom (three blocks per SM) against the oracle."""
+    import oracle
+    from tests.helpers import modes_of
+    from tests.test_gpu_adaptive_list import _system
+    prob = oracle.Problem(*_system(1), mesh, sigma=sigma, sigma_adaptive=adaptive)
+    e = make_engine(_system(1), mesh, precision=0, prob=prob)
+    q = [1, int(np.prod(mesh)) - 1]
+    G, WP, CNT = prob.rates(modes_of(q, 3), channel_mask=28)
+    g, wp, cnt = (x.cpu().numpy() for x in e.rates(300.0, sigma, 28, q_subset=q, adaptive=adaptive))
+    assert CNT[2:].sum() > 0 and np.array_equal(cnt, CNT)
+    assert_close(g[2:], G[2:], 1e-10, what="gamma")
+    assert_close(wp[2:], WP[2:], 1e-10, what="wp")
+    e.close()
