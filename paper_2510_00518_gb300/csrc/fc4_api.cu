@@ -349,7 +349,8 @@ fc4_status ensure_occupations(fc4_ctx *c, double T, cudaStream_t s) {
 
 double max_abs(const double *phi, size_t n) {
     double mx = 0.0;
-    for (size_t k = 0; k < n; ++k) mx = std::max(mx, std::fabs(phi[k]));
+    for (size_t k = 0; k < n; ++k)          // a rarely taken branch: no chain of dependent maxima
+        if (std::fabs(phi[k]) > mx) mx = std::fabs(phi[k]);
     return mx;
 }
 
@@ -361,7 +362,6 @@ double swap_asymmetry(const double *phi, double mx, int nc, int order, int l, co
     for (int k = 0; k < order; ++k) size *= 3;
     for (int k = l + 2; k < order; ++k) in *= 3;
     double diff = 0.0;
-    bool nan = false;
     for (int i = 0; i < nc; ++i) {
         const int j = swap[i];
         if (j < 0 || swap[j] != i) return INFINITY;
@@ -372,12 +372,14 @@ double swap_asymmetry(const double *phi, double mx, int nc, int order, int l, co
                 for (int y = 0; y < 3; ++y)
                     for (int z = 0; z < in; ++z) {
                         const double d = std::fabs(p[(3 * x + y) * in + z] - q[(3 * y + x) * in + z]);
-                        nan |= d != d;
-                        diff = std::max(diff, d);
+                        if (!(d <= diff)) {
+                            if (std::isnan(d)) return INFINITY;
+                            diff = d;
+                        }
                     }
         }
     }
-    return nan ? INFINITY : diff == 0.0 ? 0.0 : diff / mx;
+    return diff == 0.0 ? 0.0 : diff / mx;
 }
 
 // The domains that Φ4 allows.  The triangular domains of the 4ph rates are used up to an asymmetry of 1e-12 (a single
@@ -393,6 +395,7 @@ void check_sym4(fc4_ctx *c, const double *phi) {
 }
 
 void check_sym3(fc4_ctx *c, const double *phi) {
+    if (c->t.n_atoms > 2) return;           // their 3ph kernel sums the rectangle
     c->asym12_3 = swap_asymmetry(phi, max_abs(phi, 27 * (size_t)c->nc3), c->nc3, 3, 1, c->swap12_3);
 }
 
