@@ -622,27 +622,23 @@ fc4_status fc4_init(const fc4_crystal *crystal, const fc4_ifc *phi2, const fc4_i
     c->nc3 = phi3 ? phi3->n_clusters : 0;
     t.nc3 = c->nc3;
     {
-        std::vector<int4> at(c->nc3), r2(c->nc3), r12(c->nc3);
+        std::vector<int4> at(c->nc3), r2(c->nc3);
         std::vector<double> im(c->nc3), ph(27 * (size_t)c->nc3);
         for (int i = 0; i < c->nc3; ++i) {
             const int *a = phi3->atoms + 3 * i, *R = phi3->cells + 6 * i;
             at[i] = make_int4(a[0], a[1], a[2], 0);
-            const int d12[3] = {R[0] - R[3], R[1] - R[4], R[2] - R[5]};
             r2[i] = phase_vec(R + 3, mesh, L);
-            r12[i] = phase_vec(d12, mesh, L);
             im[i] = ism({a[0], a[1], a[2]});
         }
         if (c->nc3) std::copy(phi3->phi, phi3->phi + 27 * (size_t)c->nc3, ph.begin());
-        int4 *d_at, *d_r2, *d_r12;
+        int4 *d_at, *d_r2;
         double *d_im;
         FC4_TRY(upload(c, &d_at, at));
         FC4_TRY(upload(c, &d_r2, r2));
-        FC4_TRY(upload(c, &d_r12, r12));
         FC4_TRY(upload(c, &d_im, im));
         FC4_TRY(upload(c, &c->phi3, ph));
         t.c3_at = d_at;
         t.c3_r2 = d_r2;
-        t.c3_r12 = d_r12;
         t.c3_ism = d_im;
         t.phi3 = c->phi3;
         {   // leg-swap partner of every cluster

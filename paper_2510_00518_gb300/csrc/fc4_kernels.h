@@ -49,7 +49,6 @@ struct Tables {
     int nc3;
     const int4 *c3_at;           // [nc3] (a, b, c, 0)
     const int4 *c3_r2;           // [nc3] R2 (L/n) mod L
-    const int4 *c3_r12;          // [nc3] (R1 - R2)(L/n) mod L
     const double *c3_ism;        // [nc3] 1/sqrt(m_a m_b m_c)
     const double *phi3;          // [nc3][27]
     // keys of the rate kernel: (leg-1 atom, leg-2 atom, R1 - R2), sorted by (leg-1, leg-2) group

@@ -4,15 +4,15 @@
 // The paper (Algorithms 3-4) enumerates the kept processes on the CPU, ships index lists to
 // the GPU and evaluates V per process.  Here the same work is fused and factored so that the
 // dense parts are shared.  One thread block owns a unit (λ = (q, j), q') and loops over the
-// partner branch j'.  With q@3@ = q + s1 q' + s2 q'', the phase of a cluster factorises as
-//   exp(i(s1 q'.R1 + s2 q''.R2 - q@3@.R3)) = exp(-i q.R3) exp(i s1 q'.(R1 - R3)) exp(i s2 q''.(R2 - R3)),
+// partner branch j'.  With q''' = q + s1 q' + s2 q'', the phase of a cluster factorises as
+//   exp(i(s1 q'.R1 + s2 q''.R2 - q'''.R3)) = exp(-i q.R3) exp(i s1 q'.(R1 - R3)) exp(i s2 q''.(R2 - R3)),
 // so with a "key" r = (leg-2 atom c, leg-3 atom d, R2 - R3) the element is
-//   V = Σ_r P_r(q'')^s2 Σ_γδ W_r[γδ] e^s2_λ''(cγ) e*_λ@3@(dδ),
+//   V = Σ_r P_r(q'')^s2 Σ_γδ W_r[γδ] e^s2_λ''(cγ) e*_λ'''(dδ),
 //   W_r[γδ] = Σ_{clusters in r} exp(-i q.R3 + i s1 q'.(R1 - R3)) / sqrt(m) Σ_αβ Φ[αβγδ] e_λ(aα) e^s1_λ'(bβ),
 // W built once per (λ, q', j') in shared memory.  Partners q'' are enumerated one per thread,
 // the window is tested with an FP32 prefilter of proven error bound (ambiguous cases are
-// decided by the exact FP64 Δ), kept (q'', j@3@, j''-mask) items are compacted in order by a
-// block scan, and each item computes Y[cγ] = Σ_r P_r Σ_δ W_r[γδ] e*_λ@3@(dδ) once for all its
+// decided by the exact FP64 Δ), kept (q'', j''', j''-mask) items are compacted in order by a
+// block scan, and each item computes Y[cγ] = Σ_r P_r Σ_δ W_r[γδ] e*_λ'''(dδ) once for all its
 // j'' (V = Σ_cγ e^s2_λ''(cγ) Y[cγ]).
 #pragma once
 #include <algorithm>
@@ -76,7 +76,7 @@ __device__ __forceinline__ float two_sum(float a, float b, float &e) {
     return s;
 }
 
-// Δ = ω + s1 ω' + s2 ω'' - ω@3@ from hi/lo FP32 splits of each ω (|error| ~ 2^-44 ω_max): the
+// Δ = ω + s1 ω' + s2 ω'' - ω''' from hi/lo FP32 splits of each ω (|error| ~ 2^-44 ω_max): the
 // Gaussian's argument in the mixed path without FP64 instructions.
 __device__ __forceinline__ float delta_comp(float h0, float l0, float h1, float l1, float h2, float l2,
                                             float h3, float l3, int s1, int s2) {
@@ -89,8 +89,8 @@ __device__ __forceinline__ float delta_comp(float h0, float l0, float h1, float 
 }
 
 // Triangular domain of a (q', q'') pair (partner-swap symmetry of the summand): -1 the pair is the
-// swap of one evaluated elsewhere; 0 no symmetry used (weight 1); 1 weight 2; 2 +- with q'' = q@3@
-// (keep j'' <= j@3@); 3 ++ / -- with q'' = q' (keep j'' >= j').  domains: bits as RateArgs::tri.
+// swap of one evaluated elsewhere; 0 no symmetry used (weight 1); 1 weight 2; 2 +- with q'' = q'''
+// (keep j'' <= j'''); 3 ++ / -- with q'' = q' (keep j'' >= j').  domains: bits as RateArgs::tri.
 __device__ __forceinline__ int tri_code(int domains, int ch, int q1, int q2, int q3) {
     if (ch == 3) {
         if (!(domains & 1)) return 0;
@@ -101,7 +101,7 @@ __device__ __forceinline__ int tri_code(int domains, int ch, int q1, int q2, int
 }
 
 // tri_code of a (q', q'') pair of mode m0 under the sampling estimate: a representative stands for
-// its own pair and, off the diagonal (code 1), for its swapped pair ((λ, q', q@3@) for +-,
+// its own pair and, off the diagonal (code 1), for its swapped pair ((λ, q', q''') for +-,
 // (λ, q'', q') for ++ and --); it keeps weight 2 when both are in the sample, becomes weight 1
 // (code 0) when one is, and is skipped (-1) when neither is.
 __device__ __forceinline__ int tri_code_sampled(const RateArgs &a, int domains, int ch, int m0, int q1, int q2, int q3,
@@ -123,7 +123,7 @@ __device__ __forceinline__ int tri_weight(int tri, int j1, int j2, int j3) {
     return tri == 0 ? 1 : tri == 1 ? 2 : tri == 2 ? (j2 < j3 ? 2 : 1) : (j2 > j1 ? 2 : 1);
 }
 
-// Window masks of one q'': bit j'' of mask[j@3@] is set iff the process is kept (restricted to the
+// Window masks of one q'': bit j'' of mask[j'''] is set iff the process is kept (restricted to the
 // triangular domain).  FP32 prefilter with the proven bound; candidates inside the band are
 // decided by the exact FP64 Δ.
 template <int NB, bool ADA>
@@ -143,7 +143,7 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
         for (int j3 = 0; j3 < NB; ++j3) mask[j3] = 0u;
         return 0;
     }
-    // branch pairs of the domain: j'' <= j@3@ (tri 2) or j'' >= j' (tri 3)
+    // branch pairs of the domain: j'' <= j''' (tri 2) or j'' >= j' (tri 3)
     auto dom = [&](int j3) -> unsigned {
         return tri == 2 ? (2u << j3) - 1u : tri == 3 ? ~((1u << j1) - 1u) : ~0u;
     };
@@ -184,7 +184,7 @@ __device__ __forceinline__ int window_masks(const Tables &t, const RateArgs &a, 
     return n;
 }
 
-// One row of the window of (λ, λ'; q''): bit j'' set iff the process with λ@3@ = (q3, j3) is kept,
+// One row of the window of (λ, λ'; q''): bit j'' set iff the process with λ''' = (q3, j3) is kept,
 // restricted to the triangular domain.  A row none of whose |Δ32| can reach the window (FP32 sums are
 // monotonic in ω''; lo2, hi2: range of s2 ω'' over the participating branches; thr bounds the window of
 // every pair) is decided without looking at its pairs.
@@ -244,7 +244,7 @@ struct GeneralSmem {
     unsigned long long *Q;         // X route: entries (q'', masks) [kQChunk]
     unsigned short *ent;           // else: entries (q'') [kQChunk]
     unsigned *found;               // bit per q'' of the chunk
-    unsigned *mask;                // [NB][kSubBatch] kept j'' per (j@3@, entry of the sub-batch)
+    unsigned *mask;                // [NB][kSubBatch] kept j'' per (j''', entry of the sub-batch)
     unsigned long long *item;      // [kSubBatch * NB]
     R *proc;                       // [128 * NB][2] weight and |V|^2 of a pass' processes
     int n_con;                     // clusters per piece
@@ -281,7 +281,7 @@ struct GeneralSmem {
 // the batched persistent kernel, which takes its units from a work list over many contexts).
 //
 // Up to two atoms, X[c,d][γδ] = Σ_r P_r W_r[γδ] is formed once per entry (q'') by the entry's thread, then
-// 36 complex multiply-adds per (q'', j@3@) item.  Larger cells list their entries, expand them into
+// 36 complex multiply-adds per (q'', j''') item.  Larger cells list their entries, expand them into
 // items a sub-batch at a time and take one item per thread: an item's Y (12 n_keys complex multiply-
 // adds) is the bulk of the work, and entries carry 1 to nb of them.  The weights of a pass go
 // through shared memory to the entry's owner thread, which adds them in order, so Γ's bits are those
@@ -461,7 +461,7 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                             for (int c = 0; c < NA; ++c)
 #pragma unroll
                                 for (int g = 0; g < 3; ++g) Y[c][g] = czero<C>();
-                            // Y[cγ] = Σ_dδ X[c,d][γδ] e*_λ@3@(dδ)
+                            // Y[cγ] = Σ_dδ X[c,d][γδ] e*_λ'''(dδ)
 #pragma unroll
                             for (int d = 0; d < NA; ++d) {
                                 C e3[3];
@@ -586,7 +586,7 @@ __device__ __forceinline__ void rates4_unit(const Tables &t, const RateArgs &a, 
                                 const int q3 = q_index(b0 + s2 * c2.x, b1 + s2 * c2.y, b2 + s2 * c2.z,
                                                        t.mesh[0], t.mesh[1], t.mesh[2]);
                                 const C *P = P4 + (size_t)iq2 * t.n_keys;
-                                // Y[cγ] = Σ_d Σ_{r in (c,d)} P_r^s2 Σ_δ W_r[γδ] e*_λ@3@(dδ)
+                                // Y[cγ] = Σ_d Σ_{r in (c,d)} P_r^s2 Σ_δ W_r[γδ] e*_λ'''(dδ)
                                 C Y[NA][3];
 #pragma unroll
                                 for (int c = 0; c < NA; ++c) {
