@@ -15,8 +15,6 @@ constexpr double kAdaptiveSigmaMin = 1e-9;           // rad/ps: adaptive widths 
 struct Tables {
     int n_atoms, nb, N, L;
     int mesh[3];
-    const int *domains;          // bits of RateArgs::tri that the present Φ allows 3ph- and the FP64 gradient: replays of a
-                                 // captured launch find them as they are then
     // mesh
     const int4 *qc;              // [N] integer coordinates (i1, i2, i3, 0)
     const double2 *rt;           // [L] exp(2πi k / L)
@@ -79,6 +77,8 @@ struct Tables {
     const double2 *P4;           // [N][n_keys] exp(i q.(R2 - R3)) of each key
     const float2 *P4_32;
     int grp_start[kGroups];      // key range of group g = c * n_atoms + d
+    const int *domains;          // bits of RateArgs::tri that the present Φ allows 3ph- and the FP64 gradient: replays of a
+                                 // captured launch find them as they are then
 };
 
 // Per-call parameters of the rate kernels.
