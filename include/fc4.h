@@ -252,8 +252,9 @@ fc4_status fc4_kappa_backward(fc4_ctx *ctx, double T_K, const double *gamma, int
  * either may be NULL to skip that order).  Cells of at most 4 atoms.  Returns FC4_ERR_STATE
  * before any fc4_rates call.  Scratch: n_q*nb*max(27 nc3, 81 nc4) doubles (grown on demand), and
  * n_q*nb*36 doubles a Φ3 key (atoms of legs 1 and 2, R1 - R2) where there are more than ~560 keys; in an
- * FC4_FP64 context with a cell of at most 2 atoms also the W scratch of the rates (so the next
- * fc4_rates forms its W anew) and, where twice W of all modes fits its bound, as much again. */
+ * FC4_FP64 context with a cell of at most 2 atoms also the W scratch of the rates, for up to 16384 (λ, q')
+ * within its bound whatever the chunks of the rates were (so the next fc4_rates forms its W anew), and,
+ * where twice W of all modes fits the bound, as much again. */
 fc4_status fc4_rates_backward(fc4_ctx *ctx, const double *dL_dgamma, double *dphi3,
                               double *dphi4, void *stream);
 
@@ -319,9 +320,9 @@ fc4_status fc4_set_sampling(fc4_ctx *ctx, double fraction, unsigned long long se
 /* fc4_set_ablation - measurement switches of the tiled 4ph kernels (results do not change):
  * bit 0: no compaction - each thread evaluates the (q'', j') entries its own window test found, as
  * an uncompacted GPU-only loop does (the paper's Algorithm 2 and its warp divergence, Results),
- * instead of the block's entries being dealt out to all threads in order.  0 (the default)
- * restores compaction.  Mixed-precision tiled kernels only (others ignore it).  Other bits return
- * FC4_ERR_INVALID. */
+ * instead of the block's entries being dealt out to all threads in order; ++ and -- then also do
+ * without their list of candidate pairs and sweep the whole window.  0 (the default) restores both.
+ * Mixed-precision tiled kernels only (others ignore it).  Other bits return FC4_ERR_INVALID. */
 fc4_status fc4_set_ablation(fc4_ctx *ctx, int flags);
 
 /* fc4_set_precision - change the arithmetic of later fc4_rates calls (any fc4_precision; the
